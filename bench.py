@@ -47,8 +47,11 @@ NEWTON_TILE = (128, 8, 256, 3, 8, 1, 1, 0, 63, 1, 0)
 
 
 def fp32_ops_per_interaction(tile) -> int:
-    """FP32 pipe operations per interaction of a pair-kernel tile: 13 with the
-    special-function unit's rsqrt used as is, 16 with one Newton step."""
+    """FP32 pipe operations per interaction of a pair-kernel tile on equal
+    masses: 13 with the special-function unit's rsqrt used as is, 16 with one
+    Newton step, 8 for a mutual shape (each unordered pair once, 16)."""
+    if tile[8] & 64:
+        return 8
     return 16 if tile[9] else 13
 
 
@@ -736,12 +739,12 @@ def run_ours(args):
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     sm_max_mhz = (peaks or {}).get("sm_max_mhz") or clocks.get("sm_max_mhz") or 2070.0
     pair_ms_total, pair_launches = plain_k["pair"]
-    pair_ms = pair_ms_total / max(pair_launches, 1)
+    pair_ms = pair_ms_total / args.steps  # a call may run its pair kernel in several panels
     achieved = interactions / (pair_ms * 1e-3) / 1e9                     # G-int/s
     plain_tile = tuple(tiles[nb.NB_PLAIN].as_tuple())
     ops = fp32_ops_per_interaction(plain_tile)
     peak = alu_peak(sm_count, sm_max_mhz, ops)
-    comp_pair_ms = comp_k["pair"][0] / max(comp_k["pair"][1], 1)
+    comp_pair_ms = comp_k["pair"][0] / args.steps
 
     if rank != 0:
         if world > 1:
@@ -773,7 +776,7 @@ def run_ours(args):
                         "tile": list(tiles.get(nb.NB_COMPENSATED, tiles[nb.NB_PLAIN]).as_tuple()),
                         "gpu_launches": sum(v[1] for v in comp_k.values()),
                         "pair_ms": comp_pair_ms},
-        "kernels_ms_per_step": {k: v[0] / max(v[1], 1) for k, v in plain_k.items()},
+        "kernels_ms_per_step": {k: v[0] / args.steps for k, v in plain_k.items()},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G-int/s",
                      "frac": achieved / peak,
                      "traffic": (PROFILED_DRAM_BYTES * n / PROFILED_N

@@ -95,7 +95,8 @@ typedef struct nb_ctx nb_ctx;
  * registers (0), and `packed` a bit mask of the interaction's operation
  * groups that run as packed FP32x2 instructions (1 difference, 2 distance,
  * 4 Newton step, 8 potential term, 16 force weight, 32 force accumulation;
- * the others run as scalar FP32; every mask gives bit-identical results),
+ * the others run as scalar FP32; every mask gives bit-identical results; 64
+ * marks a mutual shape, see below),
  * and `refine` the Newton-Raphson steps applied to the special-function
  * unit's reciprocal square root (0 or 1). With refine = 0 a pair costs 13
  * FP32 operations instead of 16 (mask bit 4 then has no effect). On sm_103a
@@ -128,7 +129,15 @@ typedef struct nb_ctx nb_ctx;
  * the next kernel on the stream may be scheduled while the previous one runs,
  * and each waits for its predecessor's results before reading. Callers that
  * pass packed FP64 state (the leap-frog) use the non-fused shape of the same
- * size class instead. */
+ * size class instead.
+ * `packed` & 64 marks a mutual shape (the built-in choice from n = 24576): each
+ * unordered pair is evaluated once and added to both particles, in 8 to 9.5 FP32
+ * operations per ordered pair (8 when all masses are equal; which form a call
+ * takes is decided on the device). Its i-blocks hold `threads` * `ipt`
+ * particles, its running sums are always compensated (NB_PLAIN and
+ * NB_COMPENSATED run the same kernel), and its scratch grows with n^2, n^2 / 128
+ * bytes up to 1 GiB; where that cannot be allocated the built-in choice for that n
+ * and above is a direct shape instead. */
 typedef struct nb_tile {
     int threads;
     int ipt;

@@ -25,7 +25,7 @@ enum KernelClass { K_PACK = 0, K_PAIR = 1, K_REDUCE = 2, K_LEAPFROG = 3, K_BATCH
                    K_COUNT = 8 };
 
 struct PendingTiming {
-    int kernel;
+    int kernel, launches;
     cudaEvent_t start, stop;
 };
 
@@ -92,8 +92,8 @@ cudaEvent_t take_event(nb_ctx *ctx) {
 
 }  // namespace
 
-nbx::TimedLaunch::TimedLaunch(nb_ctx *ctx, int kernel, cudaStream_t st)
-    : ctx_(ctx), kernel_(kernel), st_(st) {
+nbx::TimedLaunch::TimedLaunch(nb_ctx *ctx, int kernel, cudaStream_t st, int launches)
+    : ctx_(ctx), kernel_(kernel), launches_(launches), st_(st) {
     if (!ctx_->timing) return;
     start_ = take_event(ctx_);
     stop_ = take_event(ctx_);
@@ -103,7 +103,7 @@ nbx::TimedLaunch::TimedLaunch(nb_ctx *ctx, int kernel, cudaStream_t st)
 nbx::TimedLaunch::~TimedLaunch() {
     if (!ctx_->timing || !start_ || !stop_) return;
     cudaEventRecord(stop_, st_);
-    ctx_->pending.push_back({kernel_, start_, stop_});
+    ctx_->pending.push_back({kernel_, launches_, start_, stop_});
 }
 
 namespace nbx {
@@ -239,6 +239,9 @@ ClusterLoad cluster_load(nb_ctx *ctx, const PairVariant &v, int64_t n) {
 // of 5 where one CTA per SM allows only 2 (29.8 against 32.2 us per call);
 // at N = 1024 clusters of 8 CTAs fit only at two per SM (5.7 against 7.5 us).
 int default_index(nb_ctx *ctx, int64_t n, bool comp) {
+    // The mutual shapes, unless their scratch has failed to allocate.
+    const int mutual = pair_mutual_index(comp, n);
+    if (mutual >= 0 && n <= ctx->ext.mutual_max_n) return mutual;
     const int k = pair_default_index(comp, n);
     const PairVariant &v = *pair_variant(comp, k);
     if (v.tile.fused != 3) return k;
@@ -271,12 +274,29 @@ const PairVariant &choose_variant(nb_ctx *ctx, int64_t n, bool comp) {
     return *pair_variant(comp, default_index(ctx, n, comp));
 }
 
+// Whether the shape for n was forced or tuned rather than built in.
+bool shape_is_chosen(nb_ctx *ctx, int64_t n, bool comp) {
+    const int m = comp ? 1 : 0;
+    return ctx->has_override[m] || ctx->tuned[m].count(size_class(n)) > 0;
+}
+
 // Enqueue pack -> pair -> combine for one system of n particles already
 // packed or to be packed from FP32 x, m. `jp` may be supplied by the caller
 // (already packed); else x, m are packed into the context's buffer.
 nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *prepacked,
                     int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st) {
     const PairVariant *vp = &choose_variant(ctx, n, comp);
+    // The mutual kernels pack for themselves. The built-in choice falls back to
+    // a direct shape when their scratch cannot be allocated.
+    if (vp->mutual >= 0) {
+        if (!prepacked) {
+            const MutualShape &s = mutual_shape(vp->mutual, p != nullptr, false);
+            const nb_status rs = mutual_reserve(ctx, s, n);
+            if (rs == NB_OK) return run_mutual(ctx, s, x, m, n, eps, a, p, st);
+            if (rs != NB_ERR_OOM || shape_is_chosen(ctx, n, comp)) return rs;
+        }
+        vp = pair_variant(comp, pair_default_unfused_index(comp, n));
+    }
     // Packed input (FP64 state packed by the caller), or no potential wanted
     // (p NULL): a shape that reads packed particles.
     if ((prepacked || !p) && vp->tile.fused) vp = pair_variant(comp, pair_default_unfused_index(comp, n));
@@ -555,6 +575,14 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode) {
         const PairVariant *cands[2] = {pair_variant(comp, k), no_pot_twin(*pair_variant(comp, k))};
         for (const PairVariant *vp : cands) {
             if (!vp) continue;
+            if (vp->mutual >= 0) {
+                // Without this scratch the built-in choice is a direct shape.
+                for (bool pot : {true, false}) {
+                    const nb_status rs = mutual_reserve(ctx, mutual_shape(vp->mutual, pot, false), n);
+                    if (rs != NB_OK && rs != NB_ERR_OOM) return rs;
+                }
+                continue;
+            }
             const PairPlan plan = make_plan(*vp, n, resident_ctas(ctx, *vp));
             jp = std::max(jp, (size_t)plan.npad * sizeof(JPart));
             part = std::max(part, plan.partial_bytes);
@@ -739,6 +767,11 @@ nb_status nb_autotune(nb_ctx *ctx, int64_t n, nb_mode mode, void *stream, nb_til
         ctx->has_override[mi] = true;
         ctx->override_idx[mi] = k;
         st = run_force(ctx, x, m, nullptr, n, 1.0f / 64.f, a, p, comp, s);  // warm-up
+        if (st == NB_ERR_OOM && pair_variant(comp, k)->mutual >= 0) {  // no room for this shape
+            st = NB_OK;
+            order.pop_back();
+            continue;
+        }
         for (int rep = 0; st == NB_OK && rep < 2; ++rep) {
             float ms = 0.f;
             st = time_one(k, &ms);
@@ -793,7 +826,7 @@ nb_status nb_timing_read(nb_ctx *ctx, int kernel, double *total_ms, int64_t *lau
         float ms = 0.f;
         cudaEventElapsedTime(&ms, pt.start, pt.stop);
         ctx->total_ms[pt.kernel] += ms;
-        ctx->launches[pt.kernel] += 1;
+        ctx->launches[pt.kernel] += pt.launches;
         ctx->spare_events.push_back(pt.start);
         ctx->spare_events.push_back(pt.stop);
     }

@@ -29,6 +29,12 @@ enum ExtSlot : int {
     SLOT_ADJOINT,       // leap-frog adjoint: replayed state, position history, VJP operands
     SLOT_BATCH_FRAME,   // per-cluster HL frames (centre, grid) of the batched leap-frog
     SLOT_BATCH_PLANNED, // the offsets and eps the current batched plan was made for
+    SLOT_MUTUAL_CP,     // mutual kernels: packed particles
+    SLOT_MUTUAL_PI,     //   segment sums of the i-side
+    SLOT_MUTUAL_PJ,     //   j-side sums of a panel of rows
+    SLOT_MUTUAL_ROWS,   //   first and last CTA of each row
+    SLOT_MUTUAL_STATE,  //   sums carried from panel to panel
+    SLOT_MUTUAL_NOTES,  //   the form of the weights, and what the pack found
     SLOT_COUNT
 };
 
@@ -39,14 +45,17 @@ struct ExtState {
     int vjp_idx = -1;  // VJP shape forced by nb_set_vjp_tile (-1: built-in)
     // (n_clusters, n_total) of the batched plan in the scratch (-1: none).
     int64_t plan_clusters = -1, plan_total = -1;
+    // Largest n whose mutual scratch is known not to have failed to allocate:
+    // above it the built-in choice is a direct shape.
+    int64_t mutual_max_n = INT64_MAX;
 };
 void ext_release(ExtState &s);
 
-// Brackets one kernel launch with CUDA events on its stream when the
-// context's timing is on (nb_timing_enable).
+// Brackets one kernel launch (or `launches` of them) with CUDA events on its
+// stream when the context's timing is on (nb_timing_enable).
 class TimedLaunch {
   public:
-    TimedLaunch(nb_ctx *ctx, int kernel, cudaStream_t st);
+    TimedLaunch(nb_ctx *ctx, int kernel, cudaStream_t st, int launches = 1);
     ~TimedLaunch();
     TimedLaunch(const TimedLaunch &) = delete;
     TimedLaunch &operator=(const TimedLaunch &) = delete;
@@ -54,6 +63,7 @@ class TimedLaunch {
   private:
     nb_ctx *ctx_;
     int kernel_;
+    int launches_;
     cudaStream_t st_;
     cudaEvent_t start_ = nullptr, stop_ = nullptr;
 };
@@ -88,6 +98,19 @@ nb_status reserve_hl(nb_ctx *ctx, int64_t n);
 // pack (unless prepacked) -> pair -> combine, enqueued on st.
 nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const nbk::JPart *prepacked,
                     int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st);
+
+// Mutual kernels (nb_mutual.cu). mutual_reserve allocates what n needs; the
+// records are then packed by run_mutual from x, m, or, with x NULL, by a kernel
+// of the caller's (mutual_pack_blocks blocks of kMutualPackThreads) into
+// mutual_records, with mutual_note on mutual_notes. a or p may be NULL.
+constexpr int kMutualPackThreads = 128;
+inline int64_t mutual_pack_blocks(int64_t npad) { return (npad + kMutualPackThreads - 1) / kMutualPackThreads; }
+int64_t mutual_npad(const nbk::MutualShape &s, int64_t n);
+nb_status mutual_reserve(nb_ctx *ctx, const nbk::MutualShape &s, int64_t n);
+float4 *mutual_records(nb_ctx *ctx);
+int *mutual_notes(nb_ctx *ctx);
+nb_status run_mutual(nb_ctx *ctx, const nbk::MutualShape &s, const float *x, const float *m, int64_t n, float eps,
+                     float *a, float *p, cudaStream_t st);
 
 struct DeviceGuard {
     int prev = -1;

@@ -112,6 +112,50 @@ struct ReduceArgs {
     int *err;              // device error word (debug build)
 };
 
+// Arguments of the mutual pair kernel (nb_mutual.cu): rows r0 .. r1 - 1 of the
+// triangle of (i-block, j-tile) units.
+struct MutualArgs {
+    const float4 *cp;      // [npad] packed particles (HL: two records each)
+    float4 *pi;            // [grid + rows][2][ib] segment sums and carries
+    float4 *pj;            // j-side sums, one per (row, particle of a later block)
+    int *row_first;        // [nib] first and last CTA with a segment of the row
+    int *row_last;
+    int *notes;            // what the pack found (MutualNote)
+    int *weights;          // the form of the weights (out), for the combine
+    int *err;              // device error word
+    int64_t njt, nib;      // j-tiles and i-blocks covering n
+    int64_t r0, r1;
+    int64_t cost;          // of the rows' tiles
+    int grid;              // CTAs launched
+    int wide_eps;          // eps is outside the fast range
+    float eps, eps2;
+    int64_t fault_unit;    // test hook: unit whose copy is never issued (-1: none)
+    uint64_t wait_ns;
+    int64_t npad, pi_len, pj_len;  // extents (bounds checks of the debug build)
+};
+
+// Arguments of its combine.
+struct MutualOut {
+    float *a, *p;          // [n][3], [n]; either may be nullptr
+    float4 *state;         // [n][2] sum and carry between panels
+    int64_t n;
+    int ib, jt, hl;
+    int last;              // this panel is the last
+};
+
+// A compiled mutual shape.
+struct MutualShape {
+    int threads, ib, jt;
+    bool hl, pot;
+    const void *kernel[3];  // by the form of the weights
+    size_t smem;
+    cudaError_t (*launch)(MutualArgs, const int (&grid)[3], size_t smem, cudaStream_t);
+};
+constexpr int kMutualSizes = 2;  // j-tile sizes compiled
+const MutualShape &mutual_shape(int size, bool pot, bool hl);
+// Bound on the j-side sums held at once (a panel of one row may exceed it).
+constexpr size_t kMutualPartialBytes = size_t(1) << 30;
+
 inline bool same_tile(const nb_tile &a, const nb_tile &b) {
     return a.threads == b.threads && a.ipt == b.ipt && a.jtile == b.jtile && a.stages == b.stages &&
            a.unroll == b.unroll && a.minblocks == b.minblocks && a.release == b.release &&
@@ -138,6 +182,7 @@ struct PairVariant {
     size_t smem;               // dynamic shared memory bytes
     cudaError_t (*launch)(const PairArgs &, int grid, size_t smem, cudaStream_t);
     cudaError_t (*launch_fused)(const FusedArgs &, int grid, size_t smem, cudaStream_t);
+    int mutual = -1;           // index of the mutual shape (nb_mutual.cu), -1: direct kernels
 };
 
 // Registry of compiled variants (nb_pair.cu).
@@ -155,6 +200,8 @@ int pair_default_index(bool comp, int64_t n);
 // The built-in shape for n among those that read packed particles (not
 // fused), for callers that pack themselves (leap-frog from FP64 state).
 int pair_default_unfused_index(bool comp, int64_t n);
+// The built-in mutual shape for n, or -1 (see nb_mutual.cu).
+int pair_mutual_index(bool comp, int64_t n);
 // Whether the tuner times the fused (single-launch, small-n) shapes at n.
 bool fused_candidate(int64_t n);
 

@@ -1131,6 +1131,11 @@ static_assert(kClusterOneSmSmem >= kFusedJmax * sizeof(JPart) + 2 * kClusterSlot
      (const void *)fused_sk_kernel<T / 32, I, J, U, M, (N != 0), C>, kFusedJmax * sizeof(JPart), \
      nullptr, launch_fused_sk<T / 32, I, J, U, M, (N != 0), C>}
 
+// A mutual shape (nb_mutual.cu), K its index there: bit 64 of the mask, with
+// the groups that run packed.
+#define NB_MUTUAL_ENTRY(J, K, C)                                                                \
+    {{128, 8, J, 3, 4, 3, 0, 1, 64 + 2 + 16, 0, 0}, C, nullptr, 0, nullptr, nullptr, K}
+
 // Plain shapes. The first group evaluates the reciprocal square root without
 // the Newton step (refine 0, 13 FP32 ops per pair); the second keeps the
 // step (16 ops) for comparison and for callers that ask for it. Measured on
@@ -1179,6 +1184,8 @@ static const PairVariant kPlain[] = {
     NB_FUSED_CL(256, 2, 32, 4, 1, 0, false),
     NB_FUSED_CL(256, 4, 32, 4, 2, 0, false),
     NB_FUSED_CL(256, 2, 32, 4, 2, 0, false),
+    NB_MUTUAL_ENTRY(32, 0, false),
+    NB_MUTUAL_ENTRY(128, 1, false),
 };
 static const PairVariant kComp[] = {
     NB_VARIANT(128, 6, 256, 3, 8, 1, 0, 1, 63, 0, true),
@@ -1211,6 +1218,8 @@ static const PairVariant kComp[] = {
     NB_FUSED_CL(256, 2, 32, 4, 1, 0, true),
     NB_FUSED_CL(256, 4, 32, 4, 2, 0, true),
     NB_FUSED_CL(256, 2, 32, 4, 2, 0, true),
+    NB_MUTUAL_ENTRY(32, 0, true),
+    NB_MUTUAL_ENTRY(128, 1, true),
 };
 // HL variants (compensated, positions from FP64 state as HL records), with
 // and without the potential, for large and for small n.
@@ -1238,6 +1247,7 @@ static_assert(kDefaultRefine == 0, "the no-potential and HL shapes have no Newto
 #undef NB_FUSED
 #undef NB_FUSED_SK
 #undef NB_FUSED_CL
+#undef NB_MUTUAL_ENTRY
 
 static int pair_variant_index(bool comp, const nb_tile &t);
 
@@ -1321,6 +1331,13 @@ int pair_default_unfused_index(bool comp, int64_t n) {
 constexpr int64_t kClusterMaxN = (int64_t)76 * 128;
 constexpr int64_t kClusterWideMinN = (int64_t)3 << 10;
 constexpr int64_t kFusedMaxN = (int64_t)3 << 13;
+// Mutual shapes from kMutualMinN, where the stream-K form ends (N = 24576, equal
+// / unequal masses: 209 / 234 us against 280; N = 65536: 1301 / 1454 against 1717),
+// with 32-particle j-tiles, which split the work more evenly, below
+// kMutualLargeN and 128-particle tiles, with fewer barriers, from there (N =
+// 32768: 351 / 390 us against 360 / 408; N = 49152: 762 / 840 against 745 / 836).
+constexpr int64_t kMutualMinN = kFusedMaxN;
+constexpr int64_t kMutualLargeN = (int64_t)5 << 13;
 
 bool fused_candidate(int64_t n) { return n < (int64_t)1 << 16; }
 
@@ -1340,6 +1357,15 @@ int pair_default_index(bool comp, int64_t n) {
     const int cls = n < kClusterWideMinN ? 0 : n <= kClusterMaxN ? 1 : 2;
     const int k = idx[cls][comp ? 1 : 0];
     return k >= 0 ? k : pair_default_unfused_index(comp, n);
+}
+
+// The built-in mutual shape for n (nb_mutual.cu), or -1 below kMutualMinN.
+int pair_mutual_index(bool comp, int64_t n) {
+    if (n < kMutualMinN) return -1;
+    const int size = n < kMutualLargeN ? 0 : 1;
+    for (int k = 0; k < pair_variant_count(comp); ++k)
+        if (pair_variant(comp, k)->mutual == size) return k;
+    return -1;
 }
 
 PairPlan make_plan(const PairVariant &v, int64_t n, int resident_ctas) {
