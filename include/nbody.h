@@ -128,12 +128,14 @@ typedef struct nb_ctx nb_ctx;
  * single-launch shapes are launched with programmatic stream serialization:
  * the next kernel on the stream may be scheduled while the previous one runs,
  * and each waits for its predecessor's results before reading. Callers that
- * pass packed FP64 state (the leap-frog) use the non-fused shape of the same
- * size class instead.
- * `packed` & 64 marks a mutual shape (the built-in choice from n = 24576): each
- * unordered pair is evaluated once and added to both particles, in 8 to 9.5 FP32
- * operations per ordered pair (8 when all masses are equal; which form a call
- * takes is decided on the device). Its i-blocks hold `threads` * `ipt`
+ * pass FP64 state (the leap-frog) leave a single-launch shape for their
+ * built-in choice.
+ * `packed` & 64 marks a mutual shape (the built-in choice from n = 13312, and at
+ * every n for the calls on FP64 positions): each unordered pair is evaluated once
+ * and added to both particles, in 8 to 9.5 FP32 operations per ordered pair (8
+ * when all masses are equal; which form a call takes is decided on the device).
+ * It packs, sums and combines in launches of its own; `fused` = 2 then marks the
+ * shape that runs every form in one kernel instead of one each. Its i-blocks hold `threads` * `ipt`
  * particles, its running sums are always compensated (NB_PLAIN and
  * NB_COMPENSATED run the same kernel), and its scratch grows with n^2, n^2 / 128
  * bytes up to 1 GiB; where that cannot be allocated the built-in choice for that n

@@ -280,6 +280,15 @@ bool shape_is_chosen(nb_ctx *ctx, int64_t n, bool comp) {
     return ctx->has_override[m] || ctx->tuned[m].count(size_class(n)) > 0;
 }
 
+int mutual_from_fp64(nb_ctx *ctx, int64_t n, bool comp) {
+    if (!comp && shape_is_chosen(ctx, n, comp)) {
+        const PairVariant &v = choose_variant(ctx, n, comp);
+        // (a single-launch shape leaves it to the built-in choice)
+        if (!v.tile.fused || v.mutual >= 0) return v.mutual;
+    }
+    return n <= ctx->ext.mutual_max_n ? mutual_size_from_fp64(n) : -1;
+}
+
 // Enqueue pack -> pair -> combine for one system of n particles already
 // packed or to be packed from FP32 x, m. `jp` may be supplied by the caller
 // (already packed); else x, m are packed into the context's buffer.

@@ -12,12 +12,14 @@
 // running them apart), fused with the drift and the FP32 packing of the new
 // positions. Steps after the first are replayed from a CUDA graph.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 
 #include "nb_device.cuh"
 #include "nb_ext.h"
 #include "nb_internal.h"
+#include "nb_mutual.cuh"
 
 namespace nbk {
 
@@ -67,6 +69,97 @@ __global__ void kick_drift_pack_kernel(double *__restrict__ x, double *__restric
         xn[c] = xc;
     }
     pack_one(jp, i, xn[0], xn[1], xn[2], m[i]);
+}
+
+// The same for the mutual kernels' records (nb_mutual.cuh): one thread per
+// padded particle, in blocks of nbx::kMutualPackThreads. KICK: the kicks and the
+// drift first (kick_back as above), else the positions as they are.
+template <bool KICK>
+__global__ void mutual_pack_f64_kernel(double *__restrict__ x, double *__restrict__ v,
+                                       const float *__restrict__ a, const float *__restrict__ m, int64_t n,
+                                       int64_t npad, double dt, int kick_back, float eps, MPart *__restrict__ cp,
+                                       int *__restrict__ notes) {
+    pdl_wait_then_release();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    MPart r = mutual_padding();
+    if (i < n) {
+        const double h = 0.5 * dt;
+        float q[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double xc = x[3 * i + c];
+            if (KICK) {
+                const double g = -(double)a[3 * i + c];
+                double vc = v[3 * i + c];
+                if (kick_back) vc = vc + h * g;  // Eq. (3) of the previous step
+                vc = vc + h * g;                 // Eq. (1)
+                xc = xc + dt * vc;               // Eq. (2)
+                v[3 * i + c] = vc;
+                x[3 * i + c] = xc;
+            }
+            q[c] = (float)xc;
+        }
+        r = make_float4(-q[0], -q[1], -q[2], -0.5f * m[i]);
+    }
+    mutual_note(i < n, r, -0.5f * m[0], eps, notes);
+    if (i < npad) cp[i] = r;
+}
+
+// Order-preserving map of an FP64 value's bits to a signed 64-bit integer (its
+// own inverse): bounding boxes are reduced with integer min and max, which run
+// at the integer pipe's rate rather than the FP64 pipe's.
+__device__ __forceinline__ long long box_key(long long bits) {
+    return bits >= 0 ? bits : bits ^ 0x7fffffffffffffffll;
+}
+
+constexpr int kBoxBlocks = 512;  // most partial boxes
+
+// Compensated mode on the mutual kernels: kicks and drift (if kick; kick_back as
+// above), and one partial bounding box of the moved positions per block (lo x,
+// y, z, hi x, y, z as keys).
+__global__ void __launch_bounds__(256) kick_drift_box_kernel(double *__restrict__ x, double *__restrict__ v,
+                                                             const float *__restrict__ a, int64_t n, double dt,
+                                                             int kick, int kick_back,
+                                                             long long *__restrict__ box) {
+    __shared__ long long s[8][6];
+    pdl_wait_then_release();
+    const double h = 0.5 * dt;
+    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+    for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double xc = x[3 * i + c];
+            if (kick) {
+                const double g = -(double)a[3 * i + c];
+                double vc = v[3 * i + c];
+                if (kick_back) vc = vc + h * g;  // Eq. (3) of the previous step
+                vc = vc + h * g;                 // Eq. (1)
+                xc = xc + dt * vc;               // Eq. (2)
+                v[3 * i + c] = vc;
+                x[3 * i + c] = xc;
+            }
+            const long long k = box_key(__double_as_longlong(xc));
+            lo[c] = min(lo[c], k);
+            hi[c] = max(hi[c], k);
+        }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        for (int d = 16; d > 0; d >>= 1) {
+            lo[c] = min(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], d));
+            hi[c] = max(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], d));
+        }
+        if (lane == 0) {
+            s[warp][c] = lo[c];
+            s[warp][3 + c] = hi[c];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        long long k = s[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) k = threadIdx.x < 3 ? min(k, s[w][threadIdx.x]) : max(k, s[w][threadIdx.x]);
+        box[6 * blockIdx.x + threadIdx.x] = k;
+    }
 }
 
 // Kicks and drift without packing (the compensated path packs HL records
@@ -212,6 +305,69 @@ __global__ void __launch_bounds__(kBoxThreads) hl_frame_kernel(const double *__r
 
 // Particle i as HL records relative to the frame: h = y rounded to the grid
 // (exact in FP32: |y| <= 2^E), l = fl32(y - h); rows n..npad-1 are inert.
+__device__ __forceinline__ void hl_split(const double *__restrict__ x, int64_t i,
+                                         const double *__restrict__ frame, float (&h)[3], float (&l)[3]) {
+    const double g = frame[3], ginv = 1.0 / g;  // a power of two: exact
+    for (int c = 0; c < 3; ++c) {
+        const double y = x[3 * i + c] - frame[c];
+        const double yh = rint(y * ginv) * g;
+        h[c] = (float)yh;
+        l[c] = (float)(y - yh);
+    }
+}
+
+// The same as records of the mutual kernels. Every block joins the partial boxes
+// of kick_drift_box_kernel and forms the frame for itself.
+__global__ void __launch_bounds__(nbx::kMutualPackThreads)
+    mutual_hl_pack_kernel(const double *__restrict__ x, const float *__restrict__ m, int64_t n, int64_t npad,
+                          const long long *__restrict__ box, int nbox, float eps, MPart *__restrict__ cp,
+                          int *__restrict__ notes) {
+    constexpr int W = nbx::kMutualPackThreads / 32;
+    __shared__ long long s[W][6];
+    __shared__ double frame[4];
+    pdl_wait_then_release();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        long long k = c < 3 ? LLONG_MAX : LLONG_MIN;
+        for (int q = threadIdx.x; q < nbox; q += nbx::kMutualPackThreads)
+            k = c < 3 ? min(k, __ldcg(box + 6 * q + c)) : max(k, __ldcg(box + 6 * q + c));
+        for (int d = 16; d > 0; d >>= 1) {
+            const long long o = __shfl_xor_sync(0xffffffffu, k, d);
+            k = c < 3 ? min(k, o) : max(k, o);
+        }
+        if (lane == 0) s[warp][c] = k;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double ext = 0.0;
+        for (int c = 0; c < 3; ++c) {
+            long long l = s[0][c], h = s[0][3 + c];
+            for (int w = 1; w < W; ++w) {
+                l = min(l, s[w][c]);
+                h = max(h, s[w][3 + c]);
+            }
+            const double dl = __longlong_as_double(box_key(l)), dh = __longlong_as_double(box_key(h));
+            frame[c] = 0.5 * (dl + dh);
+            ext = fmax(ext, 0.5 * (dh - dl));
+        }
+        frame[3] = ldexp(1.0, hl_grid_exponent(ext) - 23);
+    }
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)nbx::kMutualPackThreads + threadIdx.x;
+    MPart hi = mutual_padding(), lo = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < n) {
+        float h[3], l[3];
+        hl_split(x, i, frame, h, l);
+        hi = make_float4(-h[0], -h[1], -h[2], -0.5f * m[i]);
+        lo = make_float4(-l[0], -l[1], -l[2], 0.f);
+    }
+    mutual_note(i < n, hi, -0.5f * m[0], eps, notes);
+    if (i >= npad) return;
+    cp[kHLRecords * i] = hi;
+    cp[kHLRecords * i + 1] = lo;
+}
+
 __global__ void hl_pack_kernel(const double *__restrict__ x, const float *__restrict__ m, int64_t n,
                                int64_t npad, const double *__restrict__ frame,
                                JPart *__restrict__ jp) {
@@ -219,13 +375,7 @@ __global__ void hl_pack_kernel(const double *__restrict__ x, const float *__rest
     if (i >= npad) return;
     float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f}, hm = 0.f;
     if (i < n) {
-        const double g = frame[3], ginv = 1.0 / g;  // a power of two: exact
-        for (int c = 0; c < 3; ++c) {
-            const double y = x[3 * i + c] - frame[c];
-            const double yh = rint(y * ginv) * g;
-            h[c] = (float)yh;
-            l[c] = (float)(y - yh);
-        }
+        hl_split(x, i, frame, h, l);
         hm = -0.5f * m[i];
     }
     float4 *dst = reinterpret_cast<float4 *>(jp + kHLRecords * i);
@@ -304,6 +454,26 @@ nb_status ensure_slot(nb_ctx *ctx, int k, size_t bytes) {
 
 unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
+// How one call evaluates forces from FP64 positions: by a mutual shape, or by
+// the direct kernels (`mutual` NULL). Decided once per call.
+struct Evaluator {
+    const MutualShape *mutual = nullptr;
+    bool comp = false;
+};
+
+// The mutual shape for n, with its scratch, if the built-in choice or the shape
+// forced or tuned for a plain call is one and the scratch can be had.
+nb_status choose_evaluator(nb_ctx *ctx, int64_t n, bool comp, bool pot, Evaluator *ev) {
+    ev->comp = comp;
+    ev->mutual = nullptr;
+    const int size = mutual_from_fp64(ctx, n, comp);
+    if (size < 0) return NB_OK;
+    const MutualShape &s = mutual_shape(size, pot, comp);
+    const nb_status st = mutual_reserve(ctx, s, n);
+    if (st == NB_OK) ev->mutual = &s;
+    return st == NB_ERR_OOM ? NB_OK : st;
+}
+
 // Reserve everything one force evaluation from packed FP64 positions needs
 // (HL records, two JParts per particle, in compensated mode).
 nb_status reserve_force(nb_ctx *ctx, int64_t n, bool comp) {
@@ -326,9 +496,27 @@ nb_status reserve_hl_state(nb_ctx *ctx, int64_t n) {
     return reserve_hl(ctx, n);
 }
 
+// The same through the mutual kernels, after kicks and drift (if kick).
+nb_status step_hl_mutual(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
+                         int64_t n, float eps, double dt, int kick, int kick_back, cudaStream_t st) {
+    long long *box = static_cast<long long *>(slot(ctx, S_BOX));
+    const int nbox = (int)std::min<int64_t>(kBoxBlocks, (n + 255) / 256);
+    cudaError_t e = launch_with_pdl(kick_drift_box_kernel, dim3((unsigned)nbox), dim3(256), 0, st, x, v,
+                                    (const float *)a, n, dt, kick, kick_back, box);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+    const int64_t npad = mutual_npad(*ev.mutual, n);
+    e = launch_with_pdl(mutual_hl_pack_kernel, dim3((unsigned)mutual_pack_blocks(npad)), dim3(kMutualPackThreads), 0,
+                        st, (const double *)x, m, n, npad, (const long long *)box, nbox, eps, mutual_records(ctx),
+                        mutual_notes(ctx));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "HL pack launch");
+    return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
+}
+
 // Eq. (gravity) from FP64 positions through HL records (p may be NULL).
-nb_status force_hl(nb_ctx *ctx, const double *x, const float *m, int64_t n, float eps, float *a,
-                   float *p, cudaStream_t st) {
+nb_status force_hl(nb_ctx *ctx, const Evaluator &ev, const double *x, const float *m, int64_t n, float eps,
+                   float *a, float *p, cudaStream_t st) {
+    if (ev.mutual)  // (the positions are only read)
+        return step_hl_mutual(ctx, ev, const_cast<double *>(x), nullptr, m, a, p, n, eps, 0.0, 0, 0, st);
     JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
     double *part = static_cast<double *>(slot(ctx, S_BOX));
     double *frame = part + 6 * box_blocks(n);
@@ -341,15 +529,41 @@ nb_status force_hl(nb_ctx *ctx, const double *x, const float *m, int64_t n, floa
     return run_force_hl(ctx, jp, n, eps, a, p, st);
 }
 
-// Enqueue the steps 1 .. nsteps-1 body: fused kicks+drift+pack, force.
-nb_status steady_step(nb_ctx *ctx, double *x, double *v, const float *m, float *a, float *p,
-                      int64_t n, float eps, double dt, bool comp, cudaStream_t st) {
+// Plain mode: Eq. (gravity) at the FP64 positions as they are.
+nb_status force_plain(nb_ctx *ctx, const Evaluator &ev, double *x, const float *m, int64_t n, float eps, float *a,
+                      float *p, cudaStream_t st) {
     JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
-    kick_drift_pack_kernel<<<blocks_for(padded(n), 256), 256, 0, st>>>(x, v, a, m, n, padded(n), dt,
-                                                                        1, jp);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
-    return run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, comp, st);
+    cudaError_t e;
+    if (ev.mutual) {
+        const int64_t npad = mutual_npad(*ev.mutual, n);
+        e = launch_with_pdl(mutual_pack_f64_kernel<false>, dim3((unsigned)mutual_pack_blocks(npad)),
+                            dim3(kMutualPackThreads), 0, st, x, (double *)nullptr, (const float *)nullptr, m, n, npad,
+                            0.0, 0, eps, mutual_records(ctx), mutual_notes(ctx));
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
+        return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
+    }
+    pack_f64_kernel<<<blocks_for(padded(n), 256), 256, 0, st>>>(x, m, n, padded(n), jp);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
+    return run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, st);
+}
+
+// Plain mode, one step but its last kick: fused kicks, drift and packing, then
+// the force.
+nb_status step_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
+                     int64_t n, float eps, double dt, int kick_back, cudaStream_t st) {
+    JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
+    cudaError_t e;
+    if (ev.mutual) {
+        const int64_t npad = mutual_npad(*ev.mutual, n);
+        e = launch_with_pdl(mutual_pack_f64_kernel<true>, dim3((unsigned)mutual_pack_blocks(npad)),
+                            dim3(kMutualPackThreads), 0, st, x, v, (const float *)a, m, n, npad, dt, kick_back, eps,
+                            mutual_records(ctx), mutual_notes(ctx));
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+        return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
+    }
+    kick_drift_pack_kernel<<<blocks_for(padded(n), 256), 256, 0, st>>>(x, v, a, m, n, padded(n), dt, kick_back, jp);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+    return run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, st);
 }
 
 // With x_hist set, copy the positions after step t (t = 0 for the entry
@@ -364,21 +578,22 @@ nb_status record(nb_ctx *ctx, double *x_hist, int t, const double *x, int64_t n,
 // The compensated leap-frog: every force evaluation packs the FP64 positions
 // as HL records (force_hl). Steps after the first are replayed from a graph,
 // unless the positions of every step are recorded (x_hist).
-nb_status leapfrog_hl(nb_ctx *ctx, double *x, double *v, const float *m, float *a, float *p,
+nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
                       int64_t n, float eps, double dt, int nsteps, int a_valid, cudaStream_t s,
                       double *x_hist) {
     nb_status st = reserve_hl_state(ctx, n);
     if (st != NB_OK) return st;
     cudaError_t e;
-    if (!a_valid && (st = force_hl(ctx, x, m, n, eps, a, p, s)) != NB_OK) return st;
+    if (!a_valid && (st = force_hl(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
     if ((st = record(ctx, x_hist, 0, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
     const unsigned nb3 = blocks_for(3 * n, 256);
     auto step = [&](int kick_back) -> nb_status {
+        if (ev.mutual) return step_hl_mutual(ctx, ev, x, v, m, a, p, n, eps, dt, 1, kick_back, s);
         kick_drift_kernel<<<nb3, 256, 0, s>>>(x, v, a, n, dt, kick_back);
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return cuda_fail(ctx, le, "leap-frog update launch");
-        return force_hl(ctx, x, m, n, eps, a, p, s);
+        return force_hl(ctx, ev, x, m, n, eps, a, p, s);
     };
     if ((st = step(0)) != NB_OK || (st = record(ctx, x_hist, 1, x, n, s)) != NB_OK) return st;
     const int rest = nsteps - 1;
@@ -415,25 +630,17 @@ nb_status leapfrog_hl(nb_ctx *ctx, double *x, double *v, const float *m, float *
 // The plain leap-frog (scratch reserved by the caller): fused kicks, drift
 // and FP32 packing, then the pair kernel. Steps after the first are replayed
 // from a graph unless the positions of every step are recorded (x_hist).
-nb_status leapfrog_plain(nb_ctx *ctx, double *x, double *v, const float *m, float *a, float *p,
+nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
                          int64_t n, float eps, double dt, int nsteps, int a_valid, cudaStream_t s,
                          double *x_hist) {
-    JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
     cudaError_t e;
     nb_status st;
-    if (!a_valid) {
-        pack_f64_kernel<<<blocks_for(padded(n), 256), 256, 0, s>>>(x, m, n, padded(n), jp);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
-        if ((st = run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, s)) != NB_OK) return st;
-    }
+    if (!a_valid && (st = force_plain(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
     if ((st = record(ctx, x_hist, 0, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
 
     // Step 0: front kick + drift + pack, force.
-    kick_drift_pack_kernel<<<blocks_for(padded(n), 256), 256, 0, s>>>(x, v, a, m, n, padded(n), dt, 0,
-                                                                      jp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
-    if ((st = run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, s)) != NB_OK) return st;
+    if ((st = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 0, s)) != NB_OK) return st;
     if ((st = record(ctx, x_hist, 1, x, n, s)) != NB_OK) return st;
 
     // Steps 1 .. nsteps-1: the same kernels with the same arguments each
@@ -446,7 +653,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, double *x, double *v, const float *m, floa
         e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture begin");
         const bool timing = ctx_set_timing(ctx, false);  // no event nodes in the graph
-        nb_status cst = steady_step(ctx, x, v, m, a, p, n, eps, dt, false, s);
+        nb_status cst = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 1, s);
         ctx_set_timing(ctx, timing);
         e = cudaStreamEndCapture(s, &graph);
         if (cst != NB_OK) {
@@ -462,7 +669,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, double *x, double *v, const float *m, floa
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     } else {
         for (int k = 0; k < rest; ++k)
-            if ((st = steady_step(ctx, x, v, m, a, p, n, eps, dt, false, s)) != NB_OK ||
+            if ((st = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 1, s)) != NB_OK ||
                 (st = record(ctx, x_hist, k + 2, x, n, s)) != NB_OK)
                 return st;
     }
@@ -498,9 +705,11 @@ nb_status nb_leapfrog_step(nb_ctx *ctx, double *x, double *v, const float *m, fl
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // Scratch first (allocation never happens inside the captured graph).
     if ((st = reserve_leapfrog(ctx, n, mode)) != NB_OK) return st;
+    Evaluator ev;
+    if ((st = choose_evaluator(ctx, n, mode == NB_COMPENSATED, p != nullptr, &ev)) != NB_OK) return st;
     if (mode == NB_COMPENSATED)
-        return leapfrog_hl(ctx, x, v, m, a, p, n, eps, dt, nsteps, a_valid, s, nullptr);
-    return leapfrog_plain(ctx, x, v, m, a, p, n, eps, dt, nsteps, a_valid, s, nullptr);
+        return leapfrog_hl(ctx, ev, x, v, m, a, p, n, eps, dt, nsteps, a_valid, s, nullptr);
+    return leapfrog_plain(ctx, ev, x, v, m, a, p, n, eps, dt, nsteps, a_valid, s, nullptr);
 }
 
 nb_status nb_leapfrog_adjoint(nb_ctx *ctx, const double *x, const double *v, const float *a,
@@ -527,6 +736,8 @@ nb_status nb_leapfrog_adjoint(nb_ctx *ctx, const double *x, const double *v, con
     const size_t total = 2 * b_xv + b_hist + 4 * b_v3 + b_s;
     if ((st = ensure_slot(ctx, S_ADJ, total)) != NB_OK) return st;
     if ((st = reserve_leapfrog(ctx, n, mode)) != NB_OK) return st;
+    Evaluator ev;
+    if ((st = choose_evaluator(ctx, n, mode == NB_COMPENSATED, false, &ev)) != NB_OK) return st;
     unsigned char *base = static_cast<unsigned char *>(slot(ctx, S_ADJ));
     double *xw = reinterpret_cast<double *>(base);
     double *vw = reinterpret_cast<double *>(base + b_xv);
@@ -544,8 +755,8 @@ nb_status nb_leapfrog_adjoint(nb_ctx *ctx, const double *x, const double *v, con
     if (e == cudaSuccess && a) e = cudaMemcpyAsync(aw, a, n3 * sizeof(float), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint replay copies");
     st = mode == NB_COMPENSATED
-             ? leapfrog_hl(ctx, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist)
-             : leapfrog_plain(ctx, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist);
+             ? leapfrog_hl(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist)
+             : leapfrog_plain(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist);
     if (st != NB_OK) return st;
 
     // Reverse sweep, last step first: one VJP of Eq. (gravity) per step.
@@ -589,18 +800,16 @@ nb_status nb_energy(nb_ctx *ctx, const double *x, const double *v, const float *
     const int nblk = (int)std::min<int64_t>(1024, (n + kEnergyThreads - 1) / kEnergyThreads);
     if ((st = ensure_slot(ctx, S_EBLK, (size_t)nblk * sizeof(double2))) != NB_OK) return st;
     if ((st = ensure_slot(ctx, S_EOUT, sizeof(double2))) != NB_OK) return st;
-    JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
+    Evaluator ev;
+    if ((st = choose_evaluator(ctx, n, comp, true, &ev)) != NB_OK) return st;
     float *abuf = static_cast<float *>(slot(ctx, S_A));
     float *pbuf = static_cast<float *>(slot(ctx, S_P));
     cudaError_t e;
     if (comp) {
         if ((st = reserve_hl_state(ctx, n)) != NB_OK) return st;
-        if ((st = force_hl(ctx, x, m, n, eps, abuf, pbuf, s)) != NB_OK) return st;
-    } else {
-        pack_f64_kernel<<<blocks_for(padded(n), 256), 256, 0, s>>>(x, m, n, padded(n), jp);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
-        if ((st = run_force(ctx, nullptr, nullptr, jp, n, eps, abuf, pbuf, comp, s)) != NB_OK) return st;
+        if ((st = force_hl(ctx, ev, x, m, n, eps, abuf, pbuf, s)) != NB_OK) return st;
+    } else if ((st = force_plain(ctx, ev, const_cast<double *>(x), m, n, eps, abuf, pbuf, s)) != NB_OK) {
+        return st;  // (the positions are only read)
     }
     double2 *blk = static_cast<double2 *>(slot(ctx, S_EBLK));
     double2 *out = static_cast<double2 *>(slot(ctx, S_EOUT));

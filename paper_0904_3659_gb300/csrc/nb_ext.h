@@ -105,6 +105,9 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const nbk::JPar
 // mutual_records, with mutual_note on mutual_notes. a or p may be NULL.
 constexpr int kMutualPackThreads = 128;
 inline int64_t mutual_pack_blocks(int64_t npad) { return (npad + kMutualPackThreads - 1) / kMutualPackThreads; }
+// The index of the mutual shape that a call on n FP64 positions takes, or -1:
+// the built-in one, or for a plain call the one forced or tuned.
+int mutual_from_fp64(nb_ctx *ctx, int64_t n, bool comp);
 int64_t mutual_npad(const nbk::MutualShape &s, int64_t n);
 nb_status mutual_reserve(nb_ctx *ctx, const nbk::MutualShape &s, int64_t n);
 float4 *mutual_records(nb_ctx *ctx);

@@ -151,7 +151,9 @@ struct MutualShape {
     size_t smem;
     cudaError_t (*launch)(MutualArgs, const int (&grid)[3], size_t smem, cudaStream_t);
 };
-constexpr int kMutualSizes = 2;  // j-tile sizes compiled
+// Compiled sizes: 32-particle j-tiles with one kernel for all forms of the
+// weights, the same with a kernel for each, 128-particle tiles with the latter.
+enum MutualSize : int { kMutualSmall = 0, kMutualMid = 1, kMutualLarge = 2, kMutualSizes = 3 };
 const MutualShape &mutual_shape(int size, bool pot, bool hl);
 // Bound on the j-side sums held at once (a panel of one row may exceed it).
 constexpr size_t kMutualPartialBytes = size_t(1) << 30;
@@ -202,6 +204,8 @@ int pair_default_index(bool comp, int64_t n);
 int pair_default_unfused_index(bool comp, int64_t n);
 // The built-in mutual shape for n, or -1 (see nb_mutual.cu).
 int pair_mutual_index(bool comp, int64_t n);
+// The mutual shape for n FP64 positions (leap-frog, energy), or -1.
+int mutual_size_from_fp64(int64_t n);
 // Whether the tuner times the fused (single-launch, small-n) shapes at n.
 bool fused_candidate(int64_t n);
 

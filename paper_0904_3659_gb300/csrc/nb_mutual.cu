@@ -104,15 +104,43 @@ __device__ __forceinline__ bool met(int o, int w, bool odd) {
     return (o >= G && o < 2 * G) || (o >= 2 * G && o < 3 * G && (w == 0 || w == 3) != odd);
 }
 
+// The group functions for the kernel's form of the weights.
+template <int P, int UNR, bool POT, bool HL, int W>
+__device__ __forceinline__ void run_group(int weights, const MPart *G, int lane, const MutualI<P, HL> &I,
+                                          float2 (&acc)[P][4], float (&ja)[4], float2 eps2) {
+    if constexpr (W != kAny)
+        mutual_group<P, UNR, POT, HL, W>(G, lane, I, acc, ja, eps2);
+    else if (weights == kEqual)
+        mutual_group<P, UNR, POT, HL, kEqual>(G, lane, I, acc, ja, eps2);
+    else if (weights == kProduct)
+        mutual_group<P, UNR, POT, HL, kProduct>(G, lane, I, acc, ja, eps2);
+    else
+        mutual_group<P, 1, POT, HL, kWide>(G, lane, I, acc, ja, eps2);
+}
+
+template <int P, bool POT, bool HL, int W>
+__device__ __forceinline__ void run_self(int weights, const MPart *G, int lane, int self, const MutualI<P, HL> &I,
+                                         float2 (&acc)[P][4], float2 eps2) {
+    if constexpr (W != kAny)
+        self_group<P, POT, HL, W>(G, lane, self, I, acc, eps2);
+    else if (weights == kEqual)
+        self_group<P, POT, HL, kEqual>(G, lane, self, I, acc, eps2);
+    else if (weights == kProduct)
+        self_group<P, POT, HL, kProduct>(G, lane, self, I, acc, eps2);
+    else
+        self_group<P, POT, HL, kWide>(G, lane, self, I, acc, eps2);
+}
+
 // ---------------------------------------------------------------------------
 // WARPS x 32 threads, P packed i-pairs per thread, JT-particle j-tiles in
 // STAGES buffers, UNR the unroll of the j loop (16 no longer fits the instruction
 // cache: 25% slower), MINB the CTAs per SM that the registers are held to, POT
 // with the potential, HL on two-word positions.
-// W: the form of the weights. The three forms are three kernels; all are
-// launched and those not meant return at once (the choice is the pack's, on the
-// device): with the loops in one kernel each of them ran 5-8% slower, the
-// registers being allocated for the worst.
+// W: the form of the weights. From n = 24576 the three forms are three kernels;
+// all are launched and those not meant return at once (the choice is the pack's,
+// on the device): with the loops in one kernel (kAny) each of them runs 5-8%
+// slower, the registers being allocated for the worst. Below, the two launches
+// saved are worth more.
 template <int WARPS, int P, int JT, int STAGES, int UNR, int MINB, bool POT, bool HL, int W>
 __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualArgs A) {
     constexpr int THREADS = WARPS * 32;
@@ -139,9 +167,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_wait_then_release();  // the packed particles are ready
-    if (W != mutual_weights(__ldcg(A.notes) | (A.wide_eps ? kNoteWide : 0))) return;
+    const int weights = mutual_weights(__ldcg(A.notes) | (A.wide_eps ? kNoteWide : 0));
+    if (W != kAny && W != weights) return;
     const int64_t c = blockIdx.x;
-    if (c == 0 && tid == 0) *A.weights = W;  // for the combine
+    if (c == 0 && tid == 0) *A.weights = weights;  // for the combine
     const Triangle T{A.njt, A.nib, TPB};
     int64_t b, t, eb, et;
     T.locate(c * A.cost / A.grid, A.r0, A.r1, &b, &t);
@@ -259,7 +288,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
                 I.y[q] = make_float2(-u.y, -w.y);
                 I.z[q] = make_float2(-u.z, -w.z);
                 I.hm[q] = make_float2(u.w, w.w);
-                if (W == kProduct)
+                if (W == kProduct || (W == kAny && weights == kProduct))
                     I.hm[q] = make_float2(mutual_scale(u.w, A.cp[0].w, A.eps), mutual_scale(w.w, A.cp[0].w, A.eps));
                 if constexpr (HL) {
                     const float4 ul = A.cp[i0 * RS + 1], wl = A.cp[i1 * RS + 1];
@@ -291,9 +320,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
             float ja[4] = {0.f, 0.f, 0.f, 0.f};
             const int o = (int)own + g;  // the group, counted from the warp's first
             if (t >= (b + 1) * TPB || met<WARPS, 2 * P>(o, warp, b & 1))
-                mutual_group<P, UNR, POT, HL, W>(G, lane, I, acc, ja, eps2);
+                run_group<P, UNR, POT, HL, W>(weights, G, lane, I, acc, ja, eps2);
             else if (o >= 0 && o < 2 * P)
-                self_group<P, POT, HL, W>(G, lane, o, I, acc, eps2);
+                run_self<P, POT, HL, W>(weights, G, lane, o, I, acc, eps2);
             dst[32 * g] = make_float4(ja[0], ja[1], ja[2], ja[3]);
         }
         if (++held == FOLD) fold();
@@ -332,70 +361,92 @@ __device__ __forceinline__ void comp_add(float (&S)[4], float (&E)[4], const flo
     }
 }
 
-constexpr int kMutualCombineThreads = 64;
+// 32 particles per block, one per lane, and their entries (pj of the rows, then
+// the segments of their own row in CTA order) in equal contiguous shares for the
+// warps, whose sums are then added in warp order: a particle of the first row has
+// up to a hundred segments at small n, and reading them one after the other took
+// 17 us at N = 3001.
+constexpr int kCombineWarps = 8;
 
-// One thread per particle; a block lies inside one i-block. Up to K loads in
-// flight (L2 and HBM latency bound the sum of a particle's n / IB entries).
-__global__ void __launch_bounds__(kMutualCombineThreads) mutual_combine_kernel(const MutualArgs A,
-                                                                               const MutualOut O) {
+__global__ void __launch_bounds__(32 * kCombineWarps) mutual_combine_kernel(const MutualArgs A, const MutualOut O) {
+    __shared__ float part[kCombineWarps][8][32];
     pdl_wait_then_release();
     if (O.last && blockIdx.x == 0 && threadIdx.x == 0) *A.notes = 0;  // for the next call's pack
-    constexpr int K = 8;
-    const int64_t i = blockIdx.x * (int64_t)kMutualCombineThreads + threadIdx.x;
-    if (i >= O.n) return;
+    constexpr int K = 8;  // loads in flight
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + lane;  // below the padded count
     const int ib = O.ib;
-    const int64_t b = i / ib, w = i - b * ib;
-    const Triangle T{A.njt, A.nib, ib / O.jt};
+    const int64_t b = blockIdx.x * (int64_t)32 / ib, w = i - b * ib;
     float S[4] = {0.f, 0.f, 0.f, 0.f}, E[4] = {0.f, 0.f, 0.f, 0.f};
+    // j-side sums (of the opposite sign) of rows r0 .. below r1, up to its own.
+    const int64_t rend = b + 1 < A.r1 ? b + 1 : A.r1;
+    const int rows = rend > A.r0 ? (int)(rend - A.r0) : 0;
+    int c0 = 0, segs = 0;
+    if (b >= A.r0 && b < A.r1) {  // (clamped: after a timeout the two words may be stale)
+        c0 = max(A.row_first[b], 0);
+        segs = max(min(A.row_last[b], A.grid - 1) - c0 + 1, 0);
+    }
+    const int e0 = (int)((int64_t)(rows + segs) * warp / kCombineWarps);
+    const int e1 = (int)((int64_t)(rows + segs) * (warp + 1) / kCombineWarps);
+    // Row r's entry of i is (lin(r) - lin(r0)) JT + i - r ib; the next row's is
+    // (njt - r tpb) JT - ib further.
+    const Triangle T{A.njt, A.nib, ib / O.jt};
+    int64_t at = (T.lin(A.r0 + e0) - T.lin(A.r0)) * O.jt + i - (A.r0 + e0) * ib;
+    int64_t step = (A.njt - (A.r0 + e0) * T.tpb) * O.jt - ib;
+    for (int e = e0; e < e1 && e < rows; e += K) {
+        float4 v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e + k < e1 && e + k < rows && NB_IN(A.err, 44, at >= 0 && at < A.pj_len)) v[k] = __ldcg(A.pj + at);
+            at += step;
+            step -= ib;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float h[4] = {-v[k].x, -v[k].y, -v[k].z, v[k].w};
+            comp_add(S, E, h);  // (past the end: zeros)
+        }
+    }
+    // Segments: sum - carry.
+    for (int e = max(e0, rows); e < e1; e += K / 2) {
+        float4 hi[K / 2], lo[K / 2];
+#pragma unroll
+        for (int k = 0; k < K / 2; ++k) {
+            const int64_t o = (c0 + e + k - rows + b - A.r0) * 2 * (int64_t)ib + w;
+            hi[k] = lo[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e + k >= e1 || !NB_IN(A.err, 45, o >= 0 && o + ib < A.pi_len)) continue;
+            hi[k] = __ldcg(A.pi + o);
+            lo[k] = __ldcg(A.pi + o + ib);
+        }
+#pragma unroll
+        for (int k = 0; k < K / 2; ++k) {
+            const float h[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
+            const float l[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w};
+            comp_add(S, E, h);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) E[r] = __fsub_rn(E[r], l[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        part[warp][r][lane] = S[r];
+        part[warp][4 + r][lane] = E[r];
+    }
+    __syncthreads();
+    if (warp > 0 || i >= O.n) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) S[r] = E[r] = 0.f;
     if (A.r0 > 0) {
         const float4 s = O.state[2 * i], e = O.state[2 * i + 1];
         S[0] = s.x, S[1] = s.y, S[2] = s.z, S[3] = s.w;
         E[0] = e.x, E[1] = e.y, E[2] = e.z, E[3] = e.w;
     }
-    // j-side sums (of the opposite sign) of rows r0 .. below r1, up to its own.
-    const int64_t rend = b + 1 < A.r1 ? b + 1 : A.r1;
-    int64_t at = i - A.r0 * ib;  // of row r: (lin(r) - lin(r0)) JT + i - r ib
-    int64_t len = (A.njt - A.r0 * T.tpb) * O.jt;
-    for (int64_t r = A.r0; r < rend; r += K) {
-        float4 v[K];
+    for (int q = 0; q < kCombineWarps; ++q) {
+        const float h[4] = {part[q][0][lane], part[q][1][lane], part[q][2][lane], part[q][3][lane]};
+        comp_add(S, E, h);
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r + k < rend && NB_IN(A.err, 44, at >= 0 && at < A.pj_len)) v[k] = __ldcg(A.pj + at);
-            at += len - ib;
-            len -= ib;
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if (r + k >= rend) break;
-            const float h[4] = {-v[k].x, -v[k].y, -v[k].z, v[k].w};
-            comp_add(S, E, h);
-        }
-    }
-    // The segments of its own row, in CTA order: sum - carry, of -a/2 and -p/2.
-    if (b >= A.r0 && b < A.r1) {
-        // (Clamped: after a timeout the two words may be stale.)
-        const int c0 = max(A.row_first[b], 0), c1 = min(A.row_last[b], A.grid - 1);
-        for (int cc = c0; cc <= c1; cc += K / 2) {
-            float4 hi[K / 2], lo[K / 2];
-#pragma unroll
-            for (int k = 0; k < K / 2; ++k) {
-                const int64_t o = (cc + k + b - A.r0) * 2 * (int64_t)ib + w;
-                hi[k] = lo[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (cc + k > c1 || !NB_IN(A.err, 45, o >= 0 && o + ib < A.pi_len)) continue;
-                hi[k] = __ldcg(A.pi + o);
-                lo[k] = __ldcg(A.pi + o + ib);
-            }
-#pragma unroll
-            for (int k = 0; k < K / 2; ++k) {
-                if (cc + k > c1) break;
-                const float h[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
-                const float l[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w};
-                comp_add(S, E, h);
-#pragma unroll
-                for (int r = 0; r < 4; ++r) E[r] = __fsub_rn(E[r], l[r]);
-            }
-        }
+        for (int r = 0; r < 4; ++r) E[r] = __fadd_rn(E[r], part[q][4 + r][lane]);
     }
     if (!O.last) {
         O.state[2 * i] = make_float4(S[0], S[1], S[2], S[3]);
@@ -449,6 +500,20 @@ static cudaError_t launch_mutual(MutualArgs a, const int (&grid)[3], size_t smem
     return e;
 }
 
+template <int W, int P, int J, int S, int M, bool POT, bool HL>
+static cudaError_t launch_mutual_any(MutualArgs a, const int (&grid)[3], size_t smem, cudaStream_t st) {
+    a.grid = grid[0];
+    return launch_with_pdl(mutual_kernel<W, P, J, S, 4, M, POT, HL, kAny>, dim3((unsigned)a.grid), dim3(W * 32), smem,
+                           st, a);
+}
+
+// The three forms in one kernel.
+#define NB_MUTUAL_ANY(W, P, J, S, M, POT, HL)                                               \
+    {W * 32, 64 * P * W, J, HL, POT,                                                        \
+     {(const void *)mutual_kernel<W, P, J, S, 4, M, POT, HL, kAny>,                         \
+      (const void *)mutual_kernel<W, P, J, S, 4, M, POT, HL, kAny>,                         \
+      (const void *)mutual_kernel<W, P, J, S, 4, M, POT, HL, kAny>},                        \
+     mutual_smem<W, P, J, S, HL>(), launch_mutual_any<W, P, J, S, M, POT, HL>}
 #define NB_MUTUAL(W, P, J, S, M, POT, HL)                                               \
     {W * 32, 64 * P * W, J, HL, POT,                                                        \
      {(const void *)mutual_kernel<W, P, J, S, 8, M, POT, HL, kEqual>,                       \
@@ -456,14 +521,17 @@ static cudaError_t launch_mutual(MutualArgs a, const int (&grid)[3], size_t smem
       (const void *)mutual_kernel<W, P, J, S, 2, M, POT, HL, kWide>},                       \
      mutual_smem<W, P, J, S, HL>(), launch_mutual<W, P, J, S, M, POT, HL>}
 
-// [j-tile size][potential or not][HL]
+// [kMutualSmall, Mid, Large][potential or not][HL]
 static const MutualShape kMutualShapes[kMutualSizes][2][2] = {
+    {{NB_MUTUAL_ANY(4, 4, 32, 3, 3, true, false), NB_MUTUAL_ANY(4, 3, 32, 3, 3, true, true)},
+     {NB_MUTUAL_ANY(4, 4, 32, 3, 3, false, false), NB_MUTUAL_ANY(4, 3, 32, 3, 3, false, true)}},
     {{NB_MUTUAL(4, 4, 32, 3, 3, true, false), NB_MUTUAL(4, 3, 32, 3, 3, true, true)},
      {NB_MUTUAL(4, 4, 32, 3, 3, false, false), NB_MUTUAL(4, 3, 32, 3, 3, false, true)}},
     {{NB_MUTUAL(4, 4, 128, 3, 3, true, false), NB_MUTUAL(4, 3, 128, 3, 3, true, true)},
      {NB_MUTUAL(4, 4, 128, 3, 3, false, false), NB_MUTUAL(4, 3, 128, 3, 3, false, true)}},
 };
 #undef NB_MUTUAL
+#undef NB_MUTUAL_ANY
 
 const MutualShape &mutual_shape(int size, bool pot, bool hl) {
     return kMutualShapes[size][pot ? 0 : 1][hl ? 1 : 0];
@@ -598,7 +666,7 @@ nb_status run_mutual(nb_ctx *ctx, const MutualShape &s, const float *x, const fl
             grid[w] = (int)std::max<int64_t>(1, std::min<int64_t>(shape_resident(ctx, s, w), A.cost / kCostMutual));
         A.grid = most_resident(ctx, s);  // bounds the combine's reads
         {
-            TimedLaunch t(ctx, 1, st, 3);
+            TimedLaunch t(ctx, 1, st, s.kernel[0] == s.kernel[1] ? 1 : 3);
             e = s.launch(A, grid, s.smem, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "mutual pair kernel launch");
@@ -608,8 +676,7 @@ nb_status run_mutual(nb_ctx *ctx, const MutualShape &s, const float *x, const fl
         {
             TimedLaunch t(ctx, 2, st);
             e = launch_with_pdl(mutual_combine_kernel,
-                                dim3((unsigned)((n + kMutualCombineThreads - 1) / kMutualCombineThreads)),
-                                dim3(kMutualCombineThreads), 0, st, A, O);
+                                dim3((unsigned)((n + 31) / 32)), dim3(32 * kCombineWarps), 0, st, A, O);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "combine kernel launch");
         r0 = r1;

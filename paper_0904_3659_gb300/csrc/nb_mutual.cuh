@@ -51,7 +51,8 @@ using MPart = float4;
 // One weight for both sides also means fewer registers read. Measured at N =
 // 131072, G-interactions/s: kEqual 3450, kProduct 3090, and 2830-2980 for the
 // form w_i = (-m_j/2) y^3, w_j = (-m_i/2) y^3, also 18 operations.
-enum MutualWeights : int { kEqual = 0, kProduct = 1, kWide = 2 };
+// (kAny, of a kernel: it runs whichever the call needs.)
+enum MutualWeights : int { kEqual = 0, kProduct = 1, kWide = 2, kAny = 3 };
 constexpr float kMutualRange = 1099511627776.f;  // 2^40
 
 // What a pack block reports about its particles (bits).

@@ -1133,8 +1133,8 @@ static_assert(kClusterOneSmSmem >= kFusedJmax * sizeof(JPart) + 2 * kClusterSlot
 
 // A mutual shape (nb_mutual.cu), K its index there: bit 64 of the mask, with
 // the groups that run packed.
-#define NB_MUTUAL_ENTRY(J, K, C)                                                                \
-    {{128, 8, J, 3, 4, 3, 0, 1, 64 + 2 + 16, 0, 0}, C, nullptr, 0, nullptr, nullptr, K}
+#define NB_MUTUAL_ENTRY(J, F, K, C)                                                             \
+    {{128, 8, J, 3, 4, 3, 0, 1, 64 + 2 + 16, 0, F}, C, nullptr, 0, nullptr, nullptr, K}
 
 // Plain shapes. The first group evaluates the reciprocal square root without
 // the Newton step (refine 0, 13 FP32 ops per pair); the second keeps the
@@ -1184,8 +1184,9 @@ static const PairVariant kPlain[] = {
     NB_FUSED_CL(256, 2, 32, 4, 1, 0, false),
     NB_FUSED_CL(256, 4, 32, 4, 2, 0, false),
     NB_FUSED_CL(256, 2, 32, 4, 2, 0, false),
-    NB_MUTUAL_ENTRY(32, 0, false),
-    NB_MUTUAL_ENTRY(128, 1, false),
+    NB_MUTUAL_ENTRY(32, 2, kMutualSmall, false),
+    NB_MUTUAL_ENTRY(32, 0, kMutualMid, false),
+    NB_MUTUAL_ENTRY(128, 0, kMutualLarge, false),
 };
 static const PairVariant kComp[] = {
     NB_VARIANT(128, 6, 256, 3, 8, 1, 0, 1, 63, 0, true),
@@ -1218,8 +1219,9 @@ static const PairVariant kComp[] = {
     NB_FUSED_CL(256, 2, 32, 4, 1, 0, true),
     NB_FUSED_CL(256, 4, 32, 4, 2, 0, true),
     NB_FUSED_CL(256, 2, 32, 4, 2, 0, true),
-    NB_MUTUAL_ENTRY(32, 0, true),
-    NB_MUTUAL_ENTRY(128, 1, true),
+    NB_MUTUAL_ENTRY(32, 2, kMutualSmall, true),
+    NB_MUTUAL_ENTRY(32, 0, kMutualMid, true),
+    NB_MUTUAL_ENTRY(128, 0, kMutualLarge, true),
 };
 // HL variants (compensated, positions from FP64 state as HL records), with
 // and without the potential, for large and for small n.
@@ -1331,12 +1333,17 @@ int pair_default_unfused_index(bool comp, int64_t n) {
 constexpr int64_t kClusterMaxN = (int64_t)76 * 128;
 constexpr int64_t kClusterWideMinN = (int64_t)3 << 10;
 constexpr int64_t kFusedMaxN = (int64_t)3 << 13;
-// Mutual shapes from kMutualMinN, where the stream-K form ends (N = 24576, equal
-// / unequal masses: 209 / 234 us against 280; N = 65536: 1301 / 1454 against 1717),
-// with 32-particle j-tiles, which split the work more evenly, below
-// kMutualLargeN and 128-particle tiles, with fewer barriers, from there (N =
-// 32768: 351 / 390 us against 360 / 408; N = 49152: 762 / 840 against 745 / 836).
-constexpr int64_t kMutualMinN = kFusedMaxN;
+// Mutual shapes from kMutualMinN (equal / unequal masses, plain: N = 10007
+// 48.8 / 55.6 us against 53 for the stream-K form, N = 12288 66.7 / 75.8 against
+// 73.8, N = 16384 101 / 115 against 125, N = 65536 1298 / 1454 against 1717 for the
+// packed shapes): one kernel for all forms of the weights below kMutualMidN, one
+// for each from there (N = 20000: 144 / 164 us against 146 / 162; N = 262144
+// 20.0 / 22.9 ms for the latter); 32-particle j-tiles, which split the work more
+// evenly, below kMutualLargeN, 128-particle tiles, with fewer barriers, from
+// there (N = 32768: 351 / 390 us against 360 / 408; N = 49152: 762 / 840 against
+// 745 / 836).
+constexpr int64_t kMutualMinN = (int64_t)13 << 10;
+constexpr int64_t kMutualMidN = kFusedMaxN;
 constexpr int64_t kMutualLargeN = (int64_t)5 << 13;
 
 bool fused_candidate(int64_t n) { return n < (int64_t)1 << 16; }
@@ -1362,10 +1369,18 @@ int pair_default_index(bool comp, int64_t n) {
 // The built-in mutual shape for n (nb_mutual.cu), or -1 below kMutualMinN.
 int pair_mutual_index(bool comp, int64_t n) {
     if (n < kMutualMinN) return -1;
-    const int size = n < kMutualLargeN ? 0 : 1;
+    const int size = n < kMutualMidN ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
     for (int k = 0; k < pair_variant_count(comp); ++k)
         if (pair_variant(comp, k)->mutual == size) return k;
     return -1;
+}
+
+// From FP64 positions the mutual shapes are the fastest at every size (leap-frog
+// without the potential, equal masses, us per step against the direct kernels:
+// n = 256 16.8 / 22.3, 4096 26 / 31.5, 20011 141 / 191; compensated: 24 / 43.5,
+// 34 / 56, 190 / 290).
+int mutual_size_from_fp64(int64_t n) {
+    return n < kMutualMidN ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
 }
 
 PairPlan make_plan(const PairVariant &v, int64_t n, int resident_ctas) {
