@@ -313,15 +313,18 @@ nb_status nb_energy(nb_ctx *ctx, const double *x, const double *v, const float *
  * on a and gp [n] on p, the gradient of L = sum_i ga_i . a_i + gp_i p_i with
  * respect to the positions, gx [n][3], and masses, gm [n]. All FP32 device
  * arrays; gp may be NULL (no upstream gradient on p: a kernel without its
- * terms runs, 26 instead of 28 FP32 operations per pair). Computed as one
- * gather pass over all pairs (no atomics), so the result is reproducible.
- * Asynchronous.
+ * terms runs). Each unordered pair is evaluated once and added to both
+ * particles, 19 FP32 operations per ordered pair (17 without gp), in a fixed
+ * order without atomics, so the result is reproducible. Scratch grows with n^2
+ * (n^2 / 32 bytes, up to 1 GiB; where that cannot be allocated, a gather over all
+ * ordered pairs runs instead). Asynchronous.
  */
 nb_status nb_force_vjp(nb_ctx *ctx, const float *x, const float *m, int64_t n, float eps,
                        const float *ga, const float *gp, float *gx, float *gm, void *stream);
 
 /* Shape of nb_force_vjp's pair kernel (nb_tile fields threads, ipt, jtile,
- * stages, unroll, minblocks, release, sums_in_smem; the others as listed):
+ * stages, unroll, minblocks, release, sums_in_smem, and packed & 64 for a mutual
+ * shape; the others as listed):
  * force one of the compiled shapes listed by nb_list_vjp_tiles (NULL
  * restores the built-in choice, by size and by whether gp is NULL), read the
  * shape nb_force_vjp uses at size n for a call with gp non-NULL, list the

@@ -47,7 +47,7 @@ struct ExtState {
     int64_t plan_clusters = -1, plan_total = -1;
     // Largest n whose mutual scratch is known not to have failed to allocate:
     // above it the built-in choice is a direct shape.
-    int64_t mutual_max_n = INT64_MAX;
+    int64_t mutual_max_n = INT64_MAX, vjp_mutual_max_n = INT64_MAX;
 };
 void ext_release(ExtState &s);
 
@@ -114,6 +114,12 @@ float4 *mutual_records(nb_ctx *ctx);
 int *mutual_notes(nb_ctx *ctx);
 nb_status run_mutual(nb_ctx *ctx, const nbk::MutualShape &s, const float *x, const float *m, int64_t n, float eps,
                      float *a, float *p, cudaStream_t st);
+
+// nb_force_vjp on the mutual kernels (nb_vjp_mutual.cu); gp may be NULL.
+// NB_ERR_OOM when the scratch cannot be allocated (nothing is enqueued then).
+
+nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, int64_t n, float eps, const float *ga,
+                         const float *gp, float *gx, float *gm, cudaStream_t st);
 
 struct DeviceGuard {
     int prev = -1;

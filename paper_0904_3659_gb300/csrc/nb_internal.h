@@ -125,7 +125,7 @@ struct MutualArgs {
     int *err;              // device error word
     int64_t njt, nib;      // j-tiles and i-blocks covering n
     int64_t r0, r1;
-    int64_t cost;          // of the rows' tiles
+    int64_t tiles;         // of the rows
     int grid;              // CTAs launched
     int wide_eps;          // eps is outside the fast range
     float eps, eps2;
@@ -154,6 +154,7 @@ struct MutualShape {
 // Compiled sizes: 32-particle j-tiles with one kernel for all forms of the
 // weights, the same with a kernel for each, 128-particle tiles with the latter.
 enum MutualSize : int { kMutualSmall = 0, kMutualMid = 1, kMutualLarge = 2, kMutualSizes = 3 };
+constexpr int kVjpMutualSizes = 2;  // of the VJP's mutual shapes: 32- and 128-particle j-tiles
 const MutualShape &mutual_shape(int size, bool pot, bool hl);
 // Bound on the j-side sums held at once (a panel of one row may exceed it).
 constexpr size_t kMutualPartialBytes = size_t(1) << 30;

@@ -6,8 +6,8 @@
 // the triangle is i-block b against the tiles of its own block and of every
 // later block. In a tile of its own block a warp meets the groups of the warps
 // after it, and its own particles one-sided; the warps before have met theirs.
-// Tiles are listed row by row, weighted by their cost (kCostDiag :
-// kCostMutual), and the resident CTAs take equal contiguous cost ranges.
+// The resident CTAs take equal contiguous ranges of the tiles listed row by row
+// (nb_triangle.cuh).
 //
 // Sums. A thread keeps its i-particles' sums for a whole row segment, with
 // Kahan compensation across groups of tiles; a segment's sums go to the slot
@@ -27,14 +27,10 @@
 #include "nb_ext.h"
 #include "nb_internal.h"
 #include "nb_mutual.cuh"
+#include "nb_triangle.cuh"
 
 namespace nbk {
 using namespace nbdev;
-
-// A tile of the own block has half the work of another, but its slowest warp has
-// as much, and the CTA meets at a barrier after every tile (N = 24576, equal
-// masses: 212 us with equal costs, 255 with 5 : 8, 220 with 12 : 8).
-constexpr int kCostDiag = 8, kCostMutual = 8;
 
 // ---------------------------------------------------------------------------
 // Pack.
@@ -50,60 +46,6 @@ __global__ void mutual_pack_f32_kernel(const float *__restrict__ x, const float 
 }
 
 // ---------------------------------------------------------------------------
-// The triangle's listing. Linear index of row b's first tile (its own block's
-// first), counted from row 0, and the cost of the tiles before it. Closed forms,
-// with `tpb` tiles per block and `njt` in all; every row but the last has tpb
-// tiles of its own block.
-struct Triangle {
-    int64_t njt, nib;
-    int tpb;
-    __host__ __device__ int64_t lin(int64_t b) const { return b * njt - tpb * (b * (b - 1) / 2); }
-    __host__ __device__ int64_t cost(int64_t b) const {
-        if (b < nib)
-            return b * kCostDiag * tpb + kCostMutual * (b * njt - tpb * (b * (b + 1) / 2));
-        return cost(nib - 1) + kCostDiag * (njt - (nib - 1) * tpb);
-    }
-    __host__ __device__ int64_t diag_tiles(int64_t b) const {
-        return b < nib - 1 ? tpb : njt - b * tpb;
-    }
-    // The first tile of rows [r0, r1) whose cost, counted from row r0, is not
-    // below c: (row, tile); (r1, -) if there is none.
-    __device__ void locate(int64_t c, int64_t r0, int64_t r1, int64_t *b, int64_t *t) const {
-        c += cost(r0);
-        int64_t lo = r0, hi = r1;  // largest row with cost(row) <= c, or r1
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) / 2;
-            if (cost(mid) <= c) lo = mid;
-            else hi = mid - 1;
-        }
-        if (lo >= r1) {
-            *b = r1;
-            *t = r1 * tpb;
-            return;
-        }
-        const int64_t o = c - cost(lo), nd = diag_tiles(lo);
-        int64_t k = (o + kCostDiag - 1) / kCostDiag;
-        if (k > nd) k = nd + (o - nd * kCostDiag + kCostMutual - 1) / kCostMutual;
-        if (lo * tpb + k >= njt) {
-            ++lo;
-            k = 0;
-        }
-        *b = lo;
-        *t = lo * tpb + k;
-    }
-};
-
-// Whether, inside an i-block, warp `w` of WARPS (each with G groups) meets the
-// group `o`, counted from its own first group, for both sides: those of the
-// next warp, and two of the warps those of the warp after that (the other two
-// in odd rows), so that every pair of warps meets once.
-template <int WARPS, int G>
-__device__ __forceinline__ bool met(int o, int w, bool odd) {
-    static_assert(WARPS == 4, "written for four warps");
-    if (o < 0) o += WARPS * G;
-    return (o >= G && o < 2 * G) || (o >= 2 * G && o < 3 * G && (w == 0 || w == 3) != odd);
-}
-
 // The group functions for the kernel's form of the weights.
 template <int P, int UNR, bool POT, bool HL, int W>
 __device__ __forceinline__ void run_group(int weights, const MPart *G, int lane, const MutualI<P, HL> &I,
@@ -172,11 +114,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
     const int64_t c = blockIdx.x;
     if (c == 0 && tid == 0) *A.weights = weights;  // for the combine
     const Triangle T{A.njt, A.nib, TPB};
-    int64_t b, t, eb, et;
-    T.locate(c * A.cost / A.grid, A.r0, A.r1, &b, &t);
-    T.locate((c + 1) * A.cost / A.grid, A.r0, A.r1, &eb, &et);
-    const int64_t first = T.lin(b) + t - b * TPB;
-    const int count = (int)(T.lin(eb) + et - eb * TPB - first);
+    const int64_t u0 = c * A.tiles / A.grid, first = T.lin(A.r0) + u0;
+    const int count = (int)((c + 1) * A.tiles / A.grid - u0);
+    int64_t b, t;
+    T.locate(u0, A.r0, A.r1, &b, &t);
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -350,17 +291,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
 
 // ---------------------------------------------------------------------------
 // Combine.
-__device__ __forceinline__ void comp_add(float (&S)[4], float (&E)[4], const float (&h)[4]) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const float v = __fadd_rn(S[r], h[r]);  // TwoSum
-        const float bp = __fsub_rn(v, S[r]);
-        const float e = __fadd_rn(__fsub_rn(S[r], __fsub_rn(v, bp)), __fsub_rn(h[r], bp));
-        S[r] = v;
-        E[r] = __fadd_rn(E[r], e);
-    }
-}
-
 // 32 particles per block, one per lane, and their entries (pj of the rows, then
 // the segments of their own row in CTA order) in equal contiguous shares for the
 // warps, whose sums are then added in warp order: a particle of the first row has
@@ -564,18 +494,8 @@ Triangle triangle(const MutualShape &s, int64_t n) {
     return Triangle{(n + s.jt - 1) / s.jt, blocks_of(s, n), s.ib / s.jt};
 }
 
-// The last row + 1 of the panel that starts at row r0: as many rows as keep
-// pj within the bound, at least one.
-int64_t panel_end(const Triangle &T, const MutualShape &s, int64_t r0) {
-    const int64_t most = (int64_t)(kMutualPartialBytes / sizeof(float4)) / s.jt;  // tiles
-    int64_t lo = r0 + 1, hi = T.nib;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) / 2;
-        if (T.lin(mid) - T.lin(r0) <= most) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
+// Tiles whose j-side sums fit the bound on pj.
+int64_t panel_tiles(const MutualShape &s) { return (int64_t)(kMutualPartialBytes / sizeof(float4)) / s.jt; }
 
 }  // namespace
 
@@ -587,8 +507,8 @@ nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n) {
     int64_t pj = 1, rows = 1;
     bool panels = false;
     for (int64_t r0 = 0; r0 < T.nib;) {
-        const int64_t r1 = panel_end(T, s, r0);
-        pj = std::max(pj, (T.lin(r1) - T.lin(r0)) * s.jt);
+        const int64_t r1 = T.panel_end(r0, panel_tiles(s));
+        pj = std::max(pj, T.tiles(r0, r1) * s.jt);
         rows = std::max(rows, r1 - r0);
         panels = panels || r1 < T.nib;
         r0 = r1;
@@ -657,13 +577,13 @@ nb_status run_mutual(nb_ctx *ctx, const MutualShape &s, const float *x, const fl
     O.jt = s.jt;
     O.hl = s.hl;
     for (int64_t r0 = 0; r0 < T.nib;) {
-        const int64_t r1 = panel_end(T, s, r0);
+        const int64_t r1 = T.panel_end(r0, panel_tiles(s));
         A.r0 = r0;
         A.r1 = r1;
-        A.cost = T.cost(r1) - T.cost(r0);
+        A.tiles = T.tiles(r0, r1);
         int grid[3];
         for (int w = 0; w < 3; ++w)
-            grid[w] = (int)std::max<int64_t>(1, std::min<int64_t>(shape_resident(ctx, s, w), A.cost / kCostMutual));
+            grid[w] = triangle_grid(A.tiles, shape_resident(ctx, s, w));
         A.grid = most_resident(ctx, s);  // bounds the combine's reads
         {
             TimedLaunch t(ctx, 1, st, s.kernel[0] == s.kernel[1] ? 1 : 3);

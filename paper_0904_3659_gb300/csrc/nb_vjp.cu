@@ -458,6 +458,7 @@ struct VjpVariant {
     const void *kernel[2];  // [0]: no upstream gradient on p; [1]: with it
     size_t smem;
     void (*launch[2])(const VjpArgs &, int grid, size_t smem, cudaStream_t);
+    int mutual = -1;        // index of the mutual shape (nb_vjp_mutual.cu)
 };
 
 template <int T, int I, int J, int S, int U, int A, bool G, int M, int R>
@@ -477,6 +478,8 @@ constexpr size_t vjp_smem() {
       (const void *)vjp_kernel<T, I, J, S, U, A, true, M, R>},                              \
      vjp_smem<T, I, J, S, A>(),                                                             \
      {launch_vjp<T, I, J, S, U, A, false, M, R>, launch_vjp<T, I, J, S, U, A, true, M, R>}}
+// A mutual shape: bit 64 of the mask, with the groups that run packed.
+#define NB_VJP_MUTUAL(J, K) {{128, 4, J, 3, 4, 3, 0, 1, 64 + 2 + 16, kDefaultRefine, 0}, {}, 0, {}, K}
 #define NB_VJP_M(T, I, J, S, U, A, M) NB_VJP_MR(T, I, J, S, U, A, M, 0)
 #define NB_VJP(T, I, J, S, U, A) NB_VJP_M(T, I, J, S, U, A, 1)
 // One packed pair per thread at up to 128 registers: two 256-thread CTAs (or
@@ -491,12 +494,21 @@ const VjpVariant kVjp[] = {
     NB_VJP_MR(128, 4, 64, 4, 4, 0, 1, 1), NB_VJP_MR(128, 4, 64, 4, 4, 0, 3, 1),
     NB_VJP_MR(128, 4, 128, 3, 4, 0, 3, 1), NB_VJP_MR(128, 4, 128, 4, 4, 0, 1, 1),
     NB_VJP(512, 2, 64, 4, 2, 0), NB_VJP(512, 2, 128, 3, 4, 0),
+    NB_VJP_MUTUAL(32, 0), NB_VJP_MUTUAL(128, 1),
 };
 #undef NB_VJP
 #undef NB_VJP_M
+#undef NB_VJP_MUTUAL
 #undef NB_VJP_MR
 constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
-// Built-in shapes (GB300 sweep, G-pairs/s). With an upstream gradient on p:
+// Built-in: the mutual shapes at every size (us with / without gp, against the
+// direct shapes below: N = 1000 15 / 13.5 against 19.5 / 18.4, N = 4096 29.5 / 27
+// against 33 / 35, N = 16384 225 / 201 against 268 / 245, N = 65536 3305 / 2980
+// against 4090 / 3655), with 32-particle j-tiles below kVjpMutualLargeN (N = 8192
+// 71 / 62 against 72 / 65) and 128-particle tiles from there (N = 12000 133 / 119
+// against 138 / 120). The direct shapes remain for n whose mutual scratch cannot
+// be allocated.
+// Direct shapes (GB300 sweep, G-pairs/s). With an upstream gradient on p:
 // two packed pairs per thread in 128-thread CTAs with the barrier-free stage
 // release; below 2^15, 128-particle j-tiles at three CTAs per SM (at most 168
 // registers; N = 16384: 1010-1016, against 989-999 for 64-particle tiles at
@@ -510,11 +522,15 @@ constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
 // shared memory at four CTAs per SM (963-978 at 16384), an unroll of 8 (982),
 // and u^2 from the special-function unit's reciprocal instead of u * u (one
 // FP32 operation fewer, 1-3% slower).
+constexpr int kVjpMutualSmall = 21, kVjpMutualLarge = 22;
+constexpr int64_t kVjpMutualLargeN = 10240;
 constexpr int kVjpSmall = 17, kVjpLarge = 18, kVjpNoGpSmall = 19, kVjpNoGpLarge = 2;
 
 const VjpVariant &vjp_variant(nb_ctx *ctx, int64_t n, bool with_gp) {
     const int k = ctx_ext(ctx).vjp_idx;
     if (k >= 0 && k < kVjpCount) return kVjp[k];
+    if (n <= ctx_ext(ctx).vjp_mutual_max_n)
+        return kVjp[n < kVjpMutualLargeN ? kVjpMutualSmall : kVjpMutualLarge];
     const bool small = n < ((int64_t)1 << 15);
     if (!with_gp) return kVjp[small ? kVjpNoGpSmall : kVjpNoGpLarge];
     return kVjp[small ? kVjpSmall : kVjpLarge];
@@ -533,7 +549,13 @@ extern "C" nb_status nb_force_vjp(nb_ctx *ctx, const float *x, const float *m, i
     DeviceGuard g(ctx_device(ctx));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
-    const VjpVariant &vv = vjp_variant(ctx, n, gp != nullptr);
+    const VjpVariant *pick = &vjp_variant(ctx, n, gp != nullptr);
+    if (pick->mutual >= 0) {
+        st = run_vjp_mutual(ctx, pick->mutual, x, m, n, eps, ga, gp, gx, gm, s);
+        if (st != NB_ERR_OOM || ctx_ext(ctx).vjp_idx >= 0) return st;
+        pick = &vjp_variant(ctx, n, gp != nullptr);  // (now a direct shape)
+    }
+    const VjpVariant &vv = *pick;
     const int with_gp = gp ? 1 : 0;
     PairVariant shape{};
     shape.tile = vv.tile;

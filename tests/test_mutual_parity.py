@@ -132,3 +132,72 @@ def test_bounded_wait_reports_timeout_and_context_survives(nb, ctx, oracle_mod):
     finally:
         nb.nb_set_tile(ctx, 0, None)
     assert worst(a, p, *oracle_mod.force(x32, m32, eps)) <= TOL[0]
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 127, 129, 511, 512, 513, 1025, 2100])
+def test_vjp_tile_edges(nb, ctx, oracle_mod, n):
+    # The adjoint's mutual shapes at the edges of their tiles, with and without
+    # an upstream gradient on p, masses of both signs and zero among them: the
+    # measure and tolerance of test_vjp_parity.py.
+    import torch
+    from test_vjp_parity import rel_to_scale, vjp_term_scales
+    x32, m32, eps = particles(n, "tracers")
+    m32[::3] *= -1
+    rng = np.random.default_rng(n)
+    ga = rng.normal(size=(n, 3)).astype(np.float32)
+    gp = rng.normal(size=n).astype(np.float32)
+    dev = [torch.from_numpy(v).cuda() for v in (x32, m32, ga, gp)]
+    try:
+        for tile in [t for t in nb.nb_list_vjp_tiles() if t.packed & 64]:
+            nb.nb_set_vjp_tile(ctx, tile)
+            for with_gp in (True, False):
+                gx = torch.full((n, 3), float("nan"), device="cuda")
+                gm = torch.full((n,), float("nan"), device="cuda")
+                nb.nb_force_vjp(ctx, dev[0], dev[1], n, eps, dev[2], dev[3] if with_gp else None, gx, gm)
+                nb.nb_synchronize(ctx)
+                g0 = gp if with_gp else np.zeros_like(gp)
+                rgx, rgm = oracle_mod.force_vjp(x32, m32, eps, ga, g0)
+                sx, sm = vjp_term_scales(x32, np.abs(m32), eps, ga, g0)
+                one = np.finfo(np.float32).tiny
+                assert rel_to_scale(gx.cpu().numpy(), rgx, sx + one) <= 1e-5, (tile, with_gp)
+                assert rel_to_scale(gm.cpu().numpy(), rgm, sm + one) <= 1e-5, (tile, with_gp)
+    finally:
+        nb.nb_set_vjp_tile(ctx, None)
+
+
+def test_vjp_panels(nb, ctx):
+    # 200000 particles: the j-side sums exceed the bound on the scratch, so the
+    # rows run in panels. 128 particles, the first and last among them, against
+    # FP64 rows of the formulas in test_vjp_parity.py, with that file's measure
+    # and tolerance.
+    import torch
+    n = 200000
+    x32, m32, eps = particles(n, "spectrum")
+    rng = np.random.default_rng(3)
+    ga = rng.normal(size=(n, 3)).astype(np.float32)
+    gp = rng.normal(size=n).astype(np.float32)
+    x, m, gat, gpt = (torch.from_numpy(v).cuda() for v in (x32, m32, ga, gp))
+    gx, gm = torch.empty((n, 3), device="cuda"), torch.empty(n, device="cuda")
+    try:
+        nb.nb_set_vjp_tile(ctx, [t for t in nb.nb_list_vjp_tiles() if t.packed & 64][-1])
+        nb.nb_force_vjp(ctx, x, m, n, eps, gat, gpt, gx, gm)
+        nb.nb_synchronize(ctx)
+    finally:
+        nb.nb_set_vjp_tile(ctx, None)
+    rows = np.unique(np.concatenate([[0, n - 1], workloads.sample_rows(n, 126, 4)]))
+    for k in rows:
+        X, M, GA, GP = x32.astype(np.float64), m32.astype(np.float64), ga.astype(np.float64), gp.astype(np.float64)
+        r = X[k] - X
+        r2 = (r * r).sum(1)
+        y = 1 / np.sqrt(r2 + float(eps) ** 2)
+        y[k] = 0
+        rk, rl, rn = r @ GA[k], (r * GA).sum(1), np.sqrt(r2)
+        c = 3 * y ** 5 * (M[k] * rl - M * rk) - y ** 3 * (GP[k] * M + M[k] * GP)
+        want_x = c @ r + GA[k] * (M @ y ** 3) - M[k] * (y ** 3 @ GA)
+        want_m = GP @ y - rl @ y ** 3
+        na = np.linalg.norm(GA, axis=1)
+        sx = (M * (y ** 3 * na[k] + 3 * y ** 5 * abs(rk) * rn + abs(GP[k]) * y ** 3 * rn)
+              + M[k] * (y ** 3 * na + 3 * y ** 5 * abs(rl) * rn + abs(GP) * y ** 3 * rn)).sum()
+        sm = (abs(rl) * y ** 3 + abs(GP) * y).sum()
+        assert np.linalg.norm(gx[k].cpu().numpy() - want_x) <= 1e-5 * sx, k
+        assert abs(float(gm[k]) - want_m) <= 1e-5 * sm, k
