@@ -210,14 +210,18 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode);
  * do not start at 0, decrease, or do not end at n_total, and a non-empty
  * cluster whose eps is not > 0 with eps^2 a finite normal FP32 number, are
  * detected on the device; then nothing is read or written and the next
- * nb_synchronize returns NB_ERR_ARG. Work items are (cluster, block of 128 i-particles,
- * chunk of at most a quarter of its j-range), taken from a device queue by
- * the warps of one persistent launch, largest clusters first; each item is
- * summed by one warp in a fixed order and the chunks are added in chunk
- * order (bit-reproducible). The item list is kept in the context and reused
- * by the next call (batched force or batched leap-frog) while n_clusters,
- * n_total and the values of offsets and eps stay the same, which the device
- * checks on every call; any change makes a new list.
+ * nb_synchronize returns NB_ERR_ARG. Every unordered pair of a cluster of more
+ * than 128 particles is evaluated once, for both its particles. Work items are
+ * (cluster, block of 128 i-particles, part of the blocks it meets), taken from a
+ * device queue by the warps of one persistent launch; each item is summed by one
+ * warp in a fixed order and the partial sums are added in a fixed order
+ * (bit-reproducible), compensated in both modes. The plan (padded offsets, items'
+ * places) is kept in the context and reused by the next call (batched force or
+ * batched leap-frog) while n_clusters, n_total and the values of offsets stay the
+ * same, which the device checks on every call; any change makes a new one.
+ * Scratch, kept in the context: about 560 MiB, or 290 B per particle if that is
+ * more; where it cannot be allocated about 50 B per particle, every pair then
+ * being evaluated twice.
  */
 nb_status nb_force_batched(nb_ctx *ctx, const float *x, const float *m, const int64_t *offsets,
                            int64_t n_clusters, int64_t n_total, const float *eps,

@@ -1,256 +1,247 @@
 // nb_batched.cu -- Eq. (gravity) (Fujiwara & Nakasato, arXiv:0904.3659,
 // Section "Introduction") for many independent clusters in one persistent
-// launch, and the leap-frog of Section "Method" over such a batch.
+// launch, every unordered pair evaluated once, and the leap-frog of Section
+// "Method" over such a batch (nb_batched.cuh has the layout and the work split).
 //
-// Layout: the clusters, concatenated by the caller, are packed into a padded
-// copy in which every cluster starts on a multiple of kClusterPad particles
-// and is padded with inert entries (m = 0), so every j-tile and i-block lies
-// inside one cluster. Work item = (cluster, i-block); a one-block planning
-// kernel lists the items grouped by the cluster's padded size, largest first
-// (close to longest-processing-time order), and the pair kernel's CTAs pop
-// items from an atomic counter. Each item is summed entirely by one CTA in a
-// fixed order, so the results do not depend on which CTA pops what.
+// An evaluation is four launches: plan (padded offsets and blocks; a plan for the
+// same sizes, offsets and eps stands), pack (records and work items), pair kernel
+// (its warps pop items from an atomic counter), combine. Every sum has a fixed
+// order, so the results do not depend on which warp pops what.
 #include <algorithm>
 #include <cfloat>
 #include <climits>
 #include <cmath>
 
+#include "nb_batched.cuh"
 #include "nb_device.cuh"
 #include "nb_ext.h"
 #include "nb_internal.h"
-#include "nb_tile.cuh"
+#include "nb_mutual.cuh"
+#include "nb_triangle.cuh"
 
 namespace nbk {
 using namespace nbdev;
 
-constexpr int kClusterPad = 128;  // >= every batched i-block and j-tile
-// The batched kernels' i-block (32 lanes x 4 i) and j-tile sizes, fixed so
-// that the planner and the combine divide by constants (batch_prepare checks
-// every compiled shape against them).
-constexpr int kBatchIB = 128, kBatchJT = 128;
-static_assert(kClusterPad % kBatchIB == 0 && kClusterPad % kBatchJT == 0,
-              "i-blocks and j-tiles lie inside one padded cluster");
-constexpr int kPlanThreads = 1024;
-constexpr int kMaxChunks = 4;      // the j-range of an i-block is split into at most this many items
+constexpr int kBmPlanThreads = 1024;
+constexpr int kBmPlanNear = 8192;  // clusters whose first blocks the plan keeps in shared memory
+// Items per resident warp that the plan aims at: more of them even out the end of
+// the launch, fewer mean fewer partial sums.
+constexpr int kItemsPerWarp = 12;
+// Entries of j-side sums that bands above kMinBand may take (512 MiB).
+constexpr int64_t kPjEntries = (int64_t)32 << 20;
+constexpr int kBatchP = kBlock / 64;  // packed i-pairs per lane
 
-// Chunks an i-block of a cluster with ntiles j-tiles is split into.
-__host__ __device__ __forceinline__ int64_t chunks_of(int64_t ntiles) {
-    return ntiles < kMaxChunks ? ntiles : kMaxChunks;
-}
-
-struct BatchPlanArgs {
-    const int64_t *off;   // [C+1] caller's offsets
-    const float *eps;     // [C] caller's softening lengths
-    int64_t C;
-    int64_t n_total;      // the caller's particle count (offsets[C] must equal it)
-    int64_t cap_padded;   // capacity of the padded particle array
-    int64_t cap_items;    // capacity of the item list
-    int64_t *poff;        // [C+1] padded offsets (out)
-    int4 *items;          // [cap_items] (cluster, i-block, chunk, chunks) (out)
-    int64_t *ibase;       // [C] index of the cluster's first item (out)
-    int *nitems;          // item count (out)
-    int *err;             // set if the offsets do not fit the capacities
-    int64_t *planned_off; // [C+1] offsets of the plan in poff/items/ibase (in/out)
-    uint32_t *planned_eps;// [C] bits of its eps (in/out)
-    int replan;           // 1: the scratch holds no plan of this (C, n_total)
+struct BmBlock {  // a padded block
+    int cluster, b, nt;  // block b of the cluster's nt
+    int first;           // first item of its row
 };
 
-// Exclusive block-wide scan of one value per thread (kPlanThreads threads):
-// a shuffle scan within each warp, then one over the warps' totals. On
-// return smem[t] holds thread t's inclusive prefix and *total the block's sum.
-__device__ int64_t block_exclusive_scan(int64_t v, int64_t *smem, int64_t *total) {
-    constexpr int kWarps = kPlanThreads / 32;
-    static_assert(kWarps <= 32, "the warps' totals are scanned by one warp");
-    __shared__ int64_t wsum[kWarps];
+struct BmArgs {
+    const int64_t *off;    // [C + 1] caller's offsets
+    const float *eps;      // [C]
+    int64_t C, n_total;
+    int64_t cap_padded, cap_items;
+    int64_t *poff;         // [C + 1] padded offsets
+    int64_t *ibase;        // [C] the cluster's first item
+    BmBlock *block;        // [cap_padded / kBlock]
+    int4 *items;           // [cap_items] (cluster, i-block, first and end met tile)
+    int *nitems, *head;    // item count and queue head
+    BatchSplit *split;     // the batch's
+    int max_band;          // blocks per band at most
+    int64_t want_items;    // items wanted: kItemsPerWarp per resident warp
+    int *notes;            // [C] what the pack found of a cluster (MutualNote)
+    MPart *cp;             // [cap_padded][1 or 2]
+    float4 *pi;            // [item][kBlock] i-side sums
+    float4 *pj;            // j-side sums (batch_pj_entry)
+    int *err;
+    uint64_t wait_ns;
+    // What the plan in the scratch was made for: sizes and offsets. fresh: nothing.
+    int64_t *planned;  // [3] C (-1: none), n_total, want_items
+    int64_t *planned_off;
+    int fresh;
+    int64_t pi_len, pj_len;
+};
+
+__host__ __device__ inline int64_t padded_size(int64_t n) {
+    return n > 0 ? (n + kBlock - 1) / kBlock * kBlock : 0;
+}
+
+// Exclusive block-wide scan of one value per thread; *total the block's sum.
+__device__ int64_t bm_scan(int64_t v, int64_t *total) {
+    __shared__ int64_t wsum[kBmPlanThreads / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     int64_t x = v;
     for (int d = 1; d < 32; d <<= 1) {
         const int64_t y = __shfl_up_sync(0xffffffffu, x, d);
         if (lane >= d) x += y;
     }
+    __syncthreads();  // wsum of the scan before
     if (lane == 31) wsum[warp] = x;
     __syncthreads();
     if (warp == 0) {
-        int64_t w = lane < kWarps ? wsum[lane] : 0;
+        int64_t w = wsum[lane];
         for (int d = 1; d < 32; d <<= 1) {
             const int64_t y = __shfl_up_sync(0xffffffffu, w, d);
             if (lane >= d) w += y;
         }
-        if (lane < kWarps) wsum[lane] = w;
+        wsum[lane] = w;
     }
     __syncthreads();
-    const int64_t incl = x + (warp > 0 ? wsum[warp - 1] : 0);
-    smem[t] = incl;
-    *total = wsum[kWarps - 1];
-    __syncthreads();
-    return incl - v;
+    *total = wsum[kBmPlanThreads / 32 - 1];
+    return x + (warp > 0 ? wsum[warp - 1] : 0) - v;
 }
 
-__device__ __forceinline__ int size_class(int64_t psz) {
-    return psz > 0 ? 63 - __clzll((unsigned long long)psz) : -1;
-}
-
-__global__ void __launch_bounds__(kPlanThreads) batch_plan_kernel(const BatchPlanArgs P) {
-    __shared__ int64_t scan[kPlanThreads];
+// Offsets and eps checked, padded offsets, every cluster's first item and every
+// padded block's record (the items themselves are written by the pack's blocks).
+// Offsets must start at 0, never decrease and end at n_total, and a non-empty
+// cluster's eps must be > 0 with eps^2 a finite normal FP32 number; otherwise every
+// cluster is given zero size, so that no kernel reads or writes. A plan for the same
+// offsets stands (3 us; one is made in 25 us for 1024 clusters).
+__global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P) {
+    pdl_wait_then_release();
     const int t = threadIdx.x;
-    // The same offsets and eps as the plan already in the scratch (it was
-    // valid, or planned_off[0] would be -1): that plan stands.
-    if (!P.replan) {
-        int diff = 0;
-        for (int64_t c = t; c <= P.C; c += kPlanThreads) {
-            diff |= P.off[c] != P.planned_off[c];
-            if (c < P.C) diff |= __float_as_uint(P.eps[c]) != P.planned_eps[c];
-        }
-        if (!__syncthreads_or(diff)) return;
-    }
-    // Offsets must start at 0, never decrease and end at n_total, and every
-    // non-empty cluster's eps must be > 0 with eps^2 a finite normal FP32
-    // number (as for nb_force); otherwise every cluster is given zero size so
-    // no later kernel reads anything.
-    int bad = 0;
-    for (int64_t c = t; c < P.C; c += kPlanThreads) {
-        bad |= P.off[c + 1] < P.off[c];
-        if (P.off[c + 1] > P.off[c]) {
-            const float e = P.eps[c], e2 = e * e;
-            bad |= !(e > 0.f && e2 >= FLT_MIN && e2 <= FLT_MAX);  // also false for NaN
-        }
+    for (int64_t c = t; c < P.C; c += kBmPlanThreads) P.notes[c] = 0;
+    if (t == 0) *P.head = 0;
+    const int stands = !P.fresh && P.planned[0] == P.C && P.planned[1] == P.n_total && P.planned[2] == P.want_items;
+    int bad = 0, replan = !stands;
+    for (int64_t c = t; c < P.C; c += kBmPlanThreads) {
+        const int64_t o = P.off[c], end = P.off[c + 1];
+        const float e = P.eps[c], e2 = e * e;
+        if (stands) replan |= end != P.planned_off[c + 1];
+        bad |= end < o;
+        bad |= end > o && !(e > 0.f && e2 >= FLT_MIN && e2 <= FLT_MAX);  // also false for NaN
     }
     if (t == 0) bad |= (P.off[0] != 0) | (P.off[P.C] != P.n_total);
-    const bool valid = !__syncthreads_or(bad);
-    if (!valid) {
-        for (int64_t c = t; c <= P.C; c += kPlanThreads) P.poff[c] = 0;
+    if (!__syncthreads_or(bad | replan)) return;
+    if (__syncthreads_or(bad)) {
+        for (int64_t c = t; c <= P.C; c += kBmPlanThreads) P.poff[c] = 0;
         if (t == 0) {
             *P.nitems = 0;
-            P.planned_off[0] = -1;  // no valid plan in the scratch
+            P.planned[0] = -1;
             atomicOr(P.err, kErrBatchPlan);
         }
         return;
     }
-    // Padded offsets.
-    int64_t carry = 0;
-    for (int64_t base = 0; base < P.C; base += kPlanThreads) {
+    auto blocks = [&](int64_t c) { return c < P.C ? (int)(padded_size(P.off[c + 1] - P.off[c]) / kBlock) : 0; };
+    __shared__ int band;  // the longest cluster's blocks, as far as they may be one band
+    __shared__ int near[kBmPlanNear + 1];
+    if (t == 0) band = 1;
+    int longest = 1;
+    int64_t carry = 0, met = 0, nit = 0, total;
+    for (int64_t base = 0; base < P.C; base += kBmPlanThreads) {
         const int64_t c = base + t;
-        int64_t psz = 0;
-        if (c < P.C) {
-            const int64_t nc = P.off[c + 1] - P.off[c];
-            psz = nc > 0 ? (nc + kClusterPad - 1) / kClusterPad * kClusterPad : 0;
-        }
-        int64_t total;
-        const int64_t ex = block_exclusive_scan(psz, scan, &total);
-        if (c < P.C) P.poff[c] = carry + ex;
+        const int nt = blocks(c);
+        const int64_t ex = carry + bm_scan(nt, &total);
+        if (c < P.C) P.poff[c] = ex * kBlock;
+        if (c < kBmPlanNear) near[c] = (int)ex;
         carry += total;
+        longest = max(longest, min(nt, P.max_band));
     }
-    if (t == 0) P.poff[P.C] = carry;
-    const bool fits = carry <= P.cap_padded;
-    // Size classes present (one bit each), so the item pass below visits only those.
-    __shared__ unsigned long long present;
-    if (t == 0) present = 0ull;
+    for (int d = 16; d > 0; d >>= 1) longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, d));
+    if ((t & 31) == 0) atomicMax(&band, longest);
     __syncthreads();
-    unsigned long long mine = 0ull;
-    for (int64_t c = t; c < P.C; c += kPlanThreads) {
-        const int64_t nc = P.off[c + 1] - P.off[c];
-        const int64_t psz = nc > 0 ? (nc + kClusterPad - 1) / kClusterPad * kClusterPad : 0;
-        if (psz > 0) mine |= 1ull << size_class(psz);
+    for (int64_t base = 0; base < P.C; base += kBmPlanThreads) {
+        bm_scan(batch_met(band, blocks(base + t)), &total);
+        met += total;
     }
-    for (int d = 16; d > 0; d >>= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, d);
-    if ((t & 31) == 0 && mine) atomicOr(&present, mine);
-    __syncthreads();
-    const unsigned long long classes = present;
-    // Items, largest size class first; clusters in index order within a class,
-    // and (i-block, chunk) in order within a cluster.
-    int64_t nit = 0;
-    for (int cls = 62; cls >= 0 && fits; --cls) {
-        if (!((classes >> cls) & 1ull)) continue;
-        for (int64_t base = 0; base < P.C; base += kPlanThreads) {
-            const int64_t c = base + t;
-            int64_t cnt = 0, nch = 0;
-            if (c < P.C) {
-                const int64_t nc = P.off[c + 1] - P.off[c];
-                const int64_t psz = nc > 0 ? (nc + kClusterPad - 1) / kClusterPad * kClusterPad : 0;
-                if (size_class(psz) == cls) {
-                    nch = chunks_of(psz / kBatchJT);
-                    cnt = psz / kBatchIB * nch;
-                }
-            }
-            int64_t total;
-            const int64_t ex = block_exclusive_scan(cnt, scan, &total);
-            if (cnt) P.ibase[c] = nit + ex;
-            // Each warp writes the items of its threads' clusters, one
-            // cluster at a time with all 32 lanes (consecutive items, so the
-            // stores coalesce).
-            if (nit + total <= P.cap_items) {
-                const int lane = t & 31;
-                unsigned todo = __ballot_sync(0xffffffffu, cnt > 0);
-                while (todo) {
-                    const int src = __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    const int64_t first = nit + __shfl_sync(0xffffffffu, ex, src);
-                    const int ccnt = (int)__shfl_sync(0xffffffffu, cnt, src);  // <= 4 x i-blocks
-                    const int cn = (int)__shfl_sync(0xffffffffu, nch, src);
-                    const int cc = (int)(base + (t - lane) + src);
-                    for (int q = lane; q < ccnt; q += 32) {
-                        const int bi = q / cn;
-                        P.items[first + q] = make_int4(cc, bi, q - bi * cn, cn);
-                    }
-                }
-            }
-            nit += total;
+    const BatchSplit split = batch_split(band, met, P.want_items);
+    if (t == 0) {
+        P.poff[P.C] = carry * kBlock;
+        *P.split = split;
+    }
+    for (int64_t base = 0; base < P.C; base += kBmPlanThreads) {
+        const int64_t c = base + t;
+        const int nt = blocks(c);
+        const int64_t ex = bm_scan(nt > 0 ? split.first(nt, nt) : 0, &total);
+        if (c < P.C) P.ibase[c] = nit + ex;
+        nit += total;
+    }
+    const bool ok = carry * kBlock <= P.cap_padded && nit <= P.cap_items;
+    __syncthreads();  // poff, ibase, near
+    // Each padded block's cluster: the last one that starts at or before it.
+    for (int64_t s = t; ok && s < carry; s += kBmPlanThreads) {
+        int64_t lo = 0, hi = P.C;
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) / 2;
+            const int64_t at = P.C <= kBmPlanNear ? near[mid] : P.poff[mid] / kBlock;
+            if (at <= s) lo = mid;
+            else hi = mid;
         }
+        const int64_t b0 = P.C <= kBmPlanNear ? near[lo] : P.poff[lo] / kBlock;
+        const int nt = blocks(lo), b = (int)(s - b0);
+        P.block[s] = BmBlock{(int)lo, b, nt, (int)(P.ibase[lo] + split.first(nt, b))};
     }
-    const bool ok = fits && nit <= P.cap_items;
+    __syncthreads();  // poff is read above
     if (t == 0) {
         *P.nitems = ok ? (int)nit : 0;
         if (!ok) atomicOr(P.err, kErrBatchPlan);
+        P.planned[0] = ok ? P.C : -1;
+        P.planned[1] = P.n_total;
+        P.planned[2] = P.want_items;
     }
-    // Remember what this plan was made for (an unusable plan: nothing).
-    for (int64_t c = t; c <= P.C; c += kPlanThreads) {
-        P.planned_off[c] = ok ? P.off[c] : -1;
-        if (c < P.C) P.planned_eps[c] = __float_as_uint(P.eps[c]);
+    for (int64_t c = t; c <= P.C; c += kBmPlanThreads) {
+        if (!ok) P.poff[c] = 0;
+        P.planned_off[c] = P.off[c];
     }
 }
 
-// The cluster holding padded row s (0 <= s < poff[C]): the largest c with
-// poff[c] <= s (an empty cluster has poff[c] == poff[c + 1]).
-__device__ __forceinline__ int64_t padded_cluster(const int64_t *__restrict__ poff, int64_t C,
-                                                  int64_t s) {
-    int64_t lo = 0, hi = C - 1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) / 2;
-        if (poff[mid] <= s) lo = mid;
-        else hi = mid - 1;
+// One block of the pack: record r (and lo) of the block's particle, its notes,
+// and the items of the block's row.
+template <bool HL>
+__device__ __forceinline__ void bm_put(const BmArgs &A, const BmBlock &B, bool real, const MPart &r, const MPart &lo,
+                                       float hm0) {
+    const int t = threadIdx.x, c = B.cluster;
+    const BatchSplit split = *A.split;
+    const float eps = A.eps[c];
+    if (!(eps >= 1.f / kMutualRange && eps <= kMutualRange) && t == 0) atomicOr(&A.notes[c], (int)kNoteWide);
+    mutual_note(real, r, hm0, eps, &A.notes[c]);
+    MPart *dst = A.cp + ((int64_t)blockIdx.x * kBlock + t) * (HL ? kHLRecords : 1);
+    dst[0] = r;
+    if (HL) dst[1] = lo;
+    const int met = B.nt - B.b % split.band, q = split.items(met);
+    for (int k = t; k < q; k += kBlock) {
+        int v0, v1;
+        split.range(met, k, &v0, &v1);
+        if (B.nt == 1) {  // one item (cluster_weights)
+            v0 = 0;
+            v1 = k == 0 ? kBlockTiles : 0;
+        }
+        if (NB_IN(A.err, 60, (int64_t)B.first + k < A.cap_items)) A.items[B.first + k] = make_int4(c, B.b, v0, v1);
     }
-    return lo;
 }
 
-// The padded rows are processed in blocks of kClusterPad rows, each inside
-// one cluster: one CTA per block, one thread per row, so every row's loads
-// are in flight at once however the sizes are distributed. Blocks past
-// poff[C] (the capacity bound, or every block when the planner rejected the
-// offsets and left poff zero) do nothing.
-
-// Pack the padded rows (FP32 or FP64 source, rounded to FP32); rows past a
-// cluster's particles are inert (zero position and mass).
-template <typename T>
-__global__ void __launch_bounds__(kClusterPad) batch_pack_kernel(const T *__restrict__ x,
-                                                                 const float *__restrict__ m,
-                                                                 const int64_t *__restrict__ off,
-                                                                 const int64_t *__restrict__ poff,
-                                                                 int64_t C, JPart *__restrict__ jp) {
-    const int64_t s = (int64_t)blockIdx.x * kClusterPad;
-    if (s >= poff[C]) return;
-    const int64_t c = padded_cluster(poff, C, s);
-    const int64_t li = s - poff[c] + threadIdx.x, o = off[c], nc = off[c + 1] - o;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+// Pack padded rows from FP32 or FP64 positions (rounded to FP32). KICK: the kicks
+// (kick_back: the previous step's too) and the drift of the leap-frog first.
+template <typename T, bool KICK>
+__global__ void __launch_bounds__(kBlock) bm_pack_kernel(const BmArgs A, T *__restrict__ x, double *__restrict__ v,
+                                                         const float *__restrict__ a, const float *__restrict__ m,
+                                                         double dt, int kick_back) {
+    pdl_wait_then_release();
+    if ((int64_t)blockIdx.x * kBlock >= A.poff[A.C]) return;
+    const BmBlock B = A.block[blockIdx.x];
+    const int64_t c = B.cluster, li = (int64_t)B.b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
+    MPart r = mutual_padding();
     if (li < nc) {
         const int64_t i = o + li;
-        const float px = (float)x[3 * i], py = (float)x[3 * i + 1], pz = (float)x[3 * i + 2];
-        const float hm = -0.5f * m[i];
-        lo = make_float4(-px, -px, -py, -py);
-        hi = make_float4(-pz, -pz, hm, hm);
+        float q[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int64_t e = 3 * i + k;
+            T xc = x[e];
+            if constexpr (KICK) {
+                const double h = 0.5 * dt, g = -(double)a[e];
+                double vc = v[e];
+                if (kick_back) vc = vc + h * g;  // Eq. (3) of the previous step
+                vc = vc + h * g;                 // Eq. (1)
+                xc = xc + dt * vc;               // Eq. (2)
+                v[e] = vc;
+                x[e] = xc;
+            }
+            q[k] = (float)xc;
+        }
+        r = make_float4(-q[0], -q[1], -q[2], -0.5f * m[i]);
     }
-    float4 *dst = reinterpret_cast<float4 *>(jp + s + threadIdx.x);
-    dst[0] = lo;
-    dst[1] = hi;
+    bm_put<false>(A, B, li < nc, r, r, -0.5f * m[o]);
 }
 
 // Order-preserving map of an FP64 value's bits to a signed 64-bit integer
@@ -314,91 +305,118 @@ __global__ void __launch_bounds__(kFrameThreads) batch_frame_kernel(const double
     }
 }
 
-// Second pass: the padded rows as HL records (two JParts per particle, see
-// kHLRecords) in their cluster's frame; padding rows are inert (zero
-// position and mass). Each coordinate y = x - centre (|y| <= 2^E) is split
-// into h, y rounded to a multiple of the grid G (adding and subtracting
-// 1.5 * 2^52 G, whose unit in the last place is G, rounds to the nearest
-// multiple exactly), and the FP32 remainder l = fl32(y - h).
-__global__ void __launch_bounds__(kClusterPad) batch_pack_hl_kernel(const double *__restrict__ x,
-                                                                    const float *__restrict__ m,
-                                                                    const int64_t *__restrict__ off,
-                                                                    const int64_t *__restrict__ poff,
-                                                                    const double4 *__restrict__ frame,
-                                                                    int64_t C, JPart *__restrict__ jp) {
-    const int64_t s = (int64_t)blockIdx.x * kClusterPad;
-    if (s >= poff[C]) return;
-    const int64_t c = padded_cluster(poff, C, s);
-    const int64_t li = s - poff[c] + threadIdx.x, o = off[c], nc = off[c + 1] - o;
-    float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f}, hm = 0.f;
+// Compensated mode on FP64 state: HL records in the cluster's frame (centre of
+// its bounding box, grid; see kHLRecords and batch_pack_hl_kernel).
+__global__ void __launch_bounds__(kBlock) bm_pack_hl_kernel(const BmArgs A, const double *__restrict__ x,
+                                                            const float *__restrict__ m,
+                                                            const double4 *__restrict__ frame) {
+    pdl_wait_then_release();
+    if ((int64_t)blockIdx.x * kBlock >= A.poff[A.C]) return;
+    const BmBlock B = A.block[blockIdx.x];
+    const int64_t c = B.cluster, li = (int64_t)B.b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
+    MPart hi = mutual_padding(), lo = make_float4(0.f, 0.f, 0.f, 0.f);
     if (li < nc) {
         const double4 f = frame[c];
         const double cen[3] = {f.x, f.y, f.z};
-        const double magic = 6755399441055744.0 * f.w;  // 1.5 * 2^52 * G
+        const double magic = 6755399441055744.0 * f.w;  // 1.5 * 2^52 * grid
         const int64_t i = o + li;
+        float h[3], l[3];
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
             const double y = __dsub_rn(x[3 * i + k], cen[k]);
             const double yh = __dsub_rn(__dadd_rn(y, magic), magic);
             h[k] = (float)yh;
             l[k] = (float)__dsub_rn(y, yh);
         }
-        hm = -0.5f * m[i];
+        hi = make_float4(-h[0], -h[1], -h[2], -0.5f * m[i]);
+        lo = make_float4(-l[0], -l[1], -l[2], 0.f);
     }
-    float4 *dst = reinterpret_cast<float4 *>(jp + kHLRecords * (s + threadIdx.x));
-    dst[0] = make_float4(-h[0], -h[0], -h[1], -h[1]);
-    dst[1] = make_float4(-h[2], -h[2], hm, hm);
-    dst[2] = make_float4(-l[0], -l[0], -l[1], -l[1]);
-    dst[3] = make_float4(-l[2], -l[2], 0.f, 0.f);
+    bm_put<true>(A, B, li < nc, hi, lo, -0.5f * m[o]);
 }
 
-struct BatchArgs {
-    const JPart *jp;
-    const int64_t *off;
-    const int64_t *poff;
-    const float *eps;
-    const int4 *items;
-    const int *nitems;
-    int *counter;
-    float4 *partial;  // [item][words][ib]: one item's sums for its i-block
-    int *err;
-    uint64_t wait_ns;
-    int64_t cap_padded, cap_items, partial_len;  // extents (debug-build bounds checks)
+// A cluster of one block has no pairs to save: its sums are those of one evaluation
+// per (i, j), in one item, in the order of j, with the masses in the weights and
+// carried over its two tiles in FP32 (128 terms). Its particles are the heaviest of a
+// batch of clusters of equal mass, and their accelerations the least averaged.
+__device__ __forceinline__ int cluster_weights(const BmArgs &A, int c, int nt) {
+    return nt == 1 ? kWide : mutual_weights(__ldcg(A.notes + c));
+}
+
+// A group's particles on the first Q pairs of i-slots, for the i-side only; the
+// particles of slot `self` (-1: none) do not meet themselves. One code for every
+// kind of weights, w = (f y) y^2 with f = 1 where all masses are equal, so that the
+// kernel's loops stay in the instruction cache.
+template <int P, int Q, bool HL>
+__device__ __forceinline__ void one_sided_group(int weights, const MPart *__restrict__ T, int lane, int self,
+                                                const MutualI<P, HL> &I, float2 (&acc)[P][4], const float2 eps2) {
+    const bool equal = weights == kEqual, product = weights == kProduct;
+#pragma unroll 4
+    for (int t = 0; t < 32; ++t) {
+        const float4 h = T[HL ? 2 * t : t];
+        const float4 l = HL ? T[2 * t + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float hj = equal ? 1.f : h.w;
+        const int own = t == lane ? self : -1;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            float2 dx, dy, dz;
+            mutual_diff<P, HL>(I, q, h, l, dx, dy, dz);
+            float2 s = fma2(dx, dx, eps2);
+            s = fma2(dy, dy, s);
+            s = fma2(dz, dz, s);
+            float2 y = make_float2(rsqrt_sfu(s.x), rsqrt_sfu(s.y));
+            if (own == 2 * q) y.x = 0.f;
+            if (own == 2 * q + 1) y.y = 0.f;
+            const float2 f = product ? make_float2(__fmul_rn(I.hm[q].x, hj), __fmul_rn(I.hm[q].y, hj)) : splat2(hj);
+            const float2 p = mul2(f, y);
+            acc[q][3] = add2(acc[q][3], p);
+            const float2 w = mul2(p, mul2(y, y));
+            acc[q][0] = fma2(w, dx, acc[q][0]);
+            acc[q][1] = fma2(w, dy, acc[q][1]);
+            acc[q][2] = fma2(w, dz, acc[q][2]);
+        }
+    }
+}
+
+struct BmStage {
+    int item, cluster, iblock, tile, end;
+    int len;  // particles copied into the stage
+    int last;  // no particles of the cluster follow
 };
 
-struct StageMeta {
-    int item, cluster, iblock, jt, end;
-    int len;  // particles copied into the stage: JT, or the cluster's last, shorter tile
-};
+// One warp per CTA, persistent: lane 0 pops items and issues the 1-D bulk copies
+// of the tiles they meet, the warp consumes them. Later blocks of the band are met
+// as in mutual_kernel (nb_mutual.cu), each pair for both sides, the rest with
+// one_sided_group: in a row's own block both orders of a pair cost 24 operations
+// against 18 and the moves, but no chain through the lanes and no code of its own
+// (the mutual form there, with a loop for each slot, measured 62 against 57 us on
+// 1024 clusters of up to 512 particles, 663 against 667 us up to 4096).
+//
+// Bound by the register-file reads of the pair loop, and for small clusters by the
+// items' ends. 128 particles a block (4 per lane) against 256: half the padding and
+// half the own-block work, twice the j-side sums; 57 against 87 us up to 512, 667
+// against 687 up to 4096. Tiles of 64 against 128: 47 against 55 us up to 512.
+// Twelve warps' worth of registers (126 a lane: 16 resident); 12 items per warp
+// against 8: 669 against 678 us, against 4: 702.
+// Against one evaluation per (i, j): 1024 clusters up to 4096 particles 817 -> 685 us
+// (the pair kernel 777 -> 632; 904.8e6 unordered pairs, 66% of the FP32 lanes' issue
+// rate counting 18 operations a pair and the padding), 1024 up to 512 82 -> 58, 300
+// up to 2048 113 -> 85, a step of those on FP64 state 150 -> 121, 8 of 6000 to 20000
+// 730 -> 514.
+template <int STAGES, int MINB, int UNR, bool HL>
+__global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
+    constexpr int P = kBatchP;
+    constexpr int RS = HL ? kHLRecords : 1;
+    constexpr uint32_t TILE_BYTES = kTile * RS * sizeof(MPart);
 
-// HL: the particles are HL records (two JParts each, batch_pack_hl_kernel)
-// and each pair's x_i - x_j is formed by tile_pass_hl.
-// Warp-level persistent kernel: every warp of a CTA is an independent
-// worker with its own shared-memory stages, barriers and item stream. Lane 0
-// pops (cluster, i-block) items from the device queue, issues the 1-D bulk
-// copies of that cluster's j-tiles, and the whole warp consumes them. A work
-// item is 32 lanes x IPT i-particles (IPT/2 packed pairs per lane), so the
-// item equals the cluster padding and no CTA-wide barrier is needed.
-template <int WARPS, int IPT, int JT, int STAGES, bool COMP, bool HL>
-__global__ void __launch_bounds__(WARPS * 32) batched_pair_kernel(const BatchArgs A) {
-    constexpr int P = IPT / 2;
-    constexpr int IB = 32 * IPT;
-    constexpr int RS = HL ? kHLRecords : 1;  // JParts per particle
-    constexpr uint32_t TILE_BYTES = JT * RS * sizeof(JPart);
-    static_assert(kClusterPad % IB == 0 && kClusterPad % JT == 0, "tiles must divide the padding");
-    constexpr size_t WARP_BYTES = (size_t)STAGES * TILE_BYTES;
-
+    // Shared memory: [STAGES tiles][running sums, carries][barriers][stages][issue records]
     extern __shared__ __align__(128) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    JPart *tiles = reinterpret_cast<JPart *>(smem + warp * WARP_BYTES);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + WARPS * WARP_BYTES) + warp * STAGES;
-    StageMeta *meta =
-        reinterpret_cast<StageMeta *>(reinterpret_cast<uint64_t *>(smem + WARPS * WARP_BYTES) +
-                                      WARPS * STAGES) + warp * STAGES;
-    int *issued_at = reinterpret_cast<int *>(
-                         reinterpret_cast<StageMeta *>(reinterpret_cast<uint64_t *>(
-                                                           smem + WARPS * WARP_BYTES) +
-                                                       WARPS * STAGES) +
-                         WARPS * STAGES) + warp * STAGES;
+    const int lane = threadIdx.x;
+    MPart *tiles = reinterpret_cast<MPart *>(smem);
+    float2 *ssum = reinterpret_cast<float2 *>(smem + (size_t)STAGES * TILE_BYTES);
+    float2 *scmp = ssum + 4 * P * 32;
+    uint64_t *full = reinterpret_cast<uint64_t *>(scmp + 4 * P * 32);
+    BmStage *meta = reinterpret_cast<BmStage *>(full + STAGES);
+    int *issued_at = reinterpret_cast<int *>(meta + STAGES);
 
     if (lane == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -408,81 +426,100 @@ __global__ void __launch_bounds__(WARPS * 32) batched_pair_kernel(const BatchArg
         fence_mbar_init();
     }
     __syncwarp();
+    pdl_wait_then_release();
 
-    // Producer state (lane 0): walks the (item, j-tile) stream, popping items.
-    int p_item = -1, p_cluster = 0, p_b = 0, p_jt = 0, p_ntiles = 0, p_done = 0;
-    int64_t p_base = 0, p_nc = 0;
-    const int nitems = *A.nitems;
+    // Producer state (lane 0): walks the (item, tile) stream.
+    int p_item = -1, p_cluster = 0, p_b = 0, p_nt = 0, p_v = 0, p_end = 0, p_done = 0;
+    int64_t p_row0 = 0, p_nc = 0;
+    const int nitems = *A.nitems, band = A.split->band;
     auto produce = [&](int kk) {
         const int s = kk % STAGES;
-        if (!p_done && p_jt >= p_ntiles) {
-            const int it = atomicAdd(A.counter, 1);
-            if (it >= nitems || !NB_IN(A.err, 10, it < A.cap_items)) {
-                p_done = 1;
-            } else {
-                const int4 w = A.items[it];
-                p_item = it;
-                p_cluster = w.x;
-                p_b = w.y;
-                p_base = A.poff[w.x];
-                p_nc = A.off[w.x + 1] - A.off[w.x];
-                const int ntiles = (int)((A.poff[w.x + 1] - p_base) / JT);
-                // chunk w.z of w.w: tiles [w.z*ntiles/w.w, (w.z+1)*ntiles/w.w)
-                p_jt = (int)((int64_t)w.z * ntiles / w.w);
-                p_ntiles = (int)((int64_t)(w.z + 1) * ntiles / w.w);
+        BmStage mt;
+        int tile = 0;
+        for (;;) {  // the next tile that holds particles
+            if (p_v < p_end) {
+                tile = batch_met_tile(band, p_nt, p_b, p_v++);
+                if ((int64_t)tile * kTile < p_nc) break;
+                continue;
             }
+            const int it = p_done ? nitems : atomicAdd(A.head, 1);
+            if (it >= nitems || !NB_IN(A.err, 61, it < A.cap_items)) {
+                p_done = 1;
+                break;
+            }
+            const int4 w = A.items[it];
+            p_item = it;
+            p_cluster = w.x;
+            p_b = w.y;
+            p_v = w.z;
+            p_end = w.w;
+            p_row0 = A.poff[w.x];
+            p_nt = (int)((A.poff[w.x + 1] - p_row0) / kBlock);
+            p_nc = A.off[w.x + 1] - A.off[w.x];
         }
-        // The cluster's last tile stops at its last particle, rounded up to a
-        // multiple of 32: the padding rows beyond add nothing (zero mass).
-        const int64_t rem = p_nc - (int64_t)p_jt * JT;
-        const int len = rem >= JT ? JT : rem > 0 ? (int)((rem + 31) & ~(int64_t)31) : 32;
-        StageMeta mt;
-        mt.end = p_done;
+        if (!p_done && !NB_IN(A.err, 62, p_row0 + (int64_t)(tile + 1) * kTile <= A.cap_padded)) p_done = 1;
         mt.item = p_item;
         mt.cluster = p_cluster;
         mt.iblock = p_b;
-        mt.jt = p_jt;
-        mt.len = len;
+        mt.tile = tile;
+        // The cluster's last tile stops at its last particle, rounded up to 32.
+        const int64_t rem = p_nc - (int64_t)tile * kTile;
+        mt.len = rem >= kTile ? kTile : (int)((rem + 31) & ~(int64_t)31);
+        mt.last = rem <= kTile;
+        mt.end = p_done;
         meta[s] = mt;
-        if (!p_done && !NB_IN(A.err, 11, p_base + (int64_t)(p_jt + 1) * JT <= A.cap_padded))
-            p_done = 1;
         if (p_done) {
-            mt.end = 1;
-            meta[s] = mt;
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[s]))
-                         : "memory");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[s])) : "memory");
         } else {
             issued_at[s] = kk;
-            const uint32_t bytes = (uint32_t)len * RS * (uint32_t)sizeof(JPart);
+            const uint32_t bytes = (uint32_t)mt.len * RS * (uint32_t)sizeof(MPart);
             mbar_arrive_expect_tx(&full[s], bytes);
-            bulk_g2s(tiles + (size_t)s * JT * RS, A.jp + (p_base + (int64_t)p_jt * JT) * RS, bytes,
-                     &full[s]);
-            ++p_jt;
+            bulk_g2s(tiles + (size_t)s * kTile * RS, A.cp + (p_row0 + (int64_t)tile * kTile) * RS, bytes, &full[s]);
         }
     };
     if (lane == 0)
         for (int kk = 0; kk < STAGES - 1; ++kk) produce(kk);
 
-    float2 xi[P], yi[P], zi[P];
-    float2 lxi[P], lyi[P], lzi[P];  // HL: remainders of the i-particles' positions
-    float2 sum[P][4], cmp[P][4];
     const float2 zero2 = splat2(0.f);
-    int cur_item = -1, cur_cluster = 0, cur_b = 0;
+    MutualI<P, HL> I;
+    float2 acc[P][4];
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = zero2;
+    int cur_item = -1, weights = kEqual, b = 0, slots = 0, band_end = 0;
+    bool one_block = false;
+    float4 *pj = nullptr;  // the row's j-side entries, from its block b + 1 on
     float2 eps2 = zero2;
 
-    // The item's sums (and Kahan carries) for its i-block.
+    // Kahan: the true value is sum - carry. After every tile: the error against FP64
+    // stays below that of one evaluation per (i, j) (9.0e-8 against 1.01e-7 up to 4096
+    // particles a cluster; every 256 particles 9.9e-8 and no faster).
+    auto fold = [&]() {
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int k = (4 * q + r) * 32 + lane;
+                const float2 s0 = ssum[k];
+                const float2 y = add2(acc[q][r], neg2(scmp[k]));
+                const float2 v = add2(s0, y);
+                scmp[k] = add2(add2(v, neg2(s0)), neg2(y));
+                ssum[k] = v;
+                acc[q][r] = zero2;
+            }
+    };
     auto write_out = [&]() {
-        if (!NB_IN(A.err, 13, ((int64_t)cur_item + 1) * (COMP ? 2 : 1) * IB <= A.partial_len)) return;
-        float4 *dst = A.partial + (int64_t)cur_item * (COMP ? 2 : 1) * IB;
+        if (!NB_IN(A.err, 63, ((int64_t)cur_item + 1) * kBlock <= A.pi_len)) return;
+        float4 *dst = A.pi + (int64_t)cur_item * kBlock + lane;
 #pragma unroll
         for (int q = 0; q < P; ++q) {
-            const int i0 = (2 * q) * 32 + lane, i1 = i0 + 32;
-            dst[i0] = make_float4(sum[q][0].x, sum[q][1].x, sum[q][2].x, sum[q][3].x);
-            dst[i1] = make_float4(sum[q][0].y, sum[q][1].y, sum[q][2].y, sum[q][3].y);
-            if (COMP) {
-                dst[IB + i0] = make_float4(cmp[q][0].x, cmp[q][1].x, cmp[q][2].x, cmp[q][3].x);
-                dst[IB + i1] = make_float4(cmp[q][0].y, cmp[q][1].y, cmp[q][2].y, cmp[q][3].y);
-            }
+            float2 s[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                s[r] = add2(ssum[(4 * q + r) * 32 + lane], neg2(scmp[(4 * q + r) * 32 + lane]));
+            dst[64 * q] = make_float4(s[0].x, s[1].x, s[2].x, s[3].x);
+            dst[64 * q + 32] = make_float4(s[0].y, s[1].y, s[2].y, s[3].y);
         }
     };
 
@@ -497,147 +534,66 @@ __global__ void __launch_bounds__(WARPS * 32) batched_pair_kernel(const BatchArg
             bad = 1;
             break;
         }
-        const StageMeta mt = meta[s];
+        const BmStage mt = meta[s];
         if (mt.end) break;
         if (mt.item != cur_item) {
             if (cur_item >= 0) write_out();
             cur_item = mt.item;
-            cur_cluster = mt.cluster;
-            cur_b = mt.iblock;
-            eps2 = splat2(A.eps[cur_cluster] * A.eps[cur_cluster]);
-            const int64_t base = A.poff[cur_cluster] + (int64_t)cur_b * IB;
+            b = mt.iblock;
+            const float eps = A.eps[mt.cluster];
+            eps2 = splat2(eps * eps);
+            const int64_t row0 = A.poff[mt.cluster], nc = A.off[mt.cluster + 1] - A.off[mt.cluster];
+            const int nt = (int)((A.poff[mt.cluster + 1] - row0) / kBlock), s0 = b / band * band;
+            weights = cluster_weights(A, mt.cluster, nt);
+            one_block = nt == 1;
+            band_end = min(s0 + band, nt);
+            slots = (int)min((nc - (int64_t)b * kBlock + 31) / 32, (int64_t)(2 * P));
+            pj = A.pj + batch_pj_entry(band, row0, nt, b);
+            const float hm0 = A.cp[row0 * RS].w;
 #pragma unroll
             for (int q = 0; q < P; ++q) {
-                int64_t i0 = base + (2 * q) * 32 + lane, i1 = i0 + 32;
-                if (!NB_IN(A.err, 12, i1 < A.cap_padded)) i0 = i1 = 0;
-                const float4 A0 = reinterpret_cast<const float4 *>(A.jp + i0 * RS)[0];
-                const float4 B0 = reinterpret_cast<const float4 *>(A.jp + i0 * RS)[1];
-                const float4 A1 = reinterpret_cast<const float4 *>(A.jp + i1 * RS)[0];
-                const float4 B1 = reinterpret_cast<const float4 *>(A.jp + i1 * RS)[1];
-                xi[q] = make_float2(-A0.x, -A1.x);
-                yi[q] = make_float2(-A0.z, -A1.z);
-                zi[q] = make_float2(-B0.x, -B1.x);
-                if (HL) {
-                    const float4 C0 = reinterpret_cast<const float4 *>(A.jp + i0 * RS + 1)[0];
-                    const float4 D0 = reinterpret_cast<const float4 *>(A.jp + i0 * RS + 1)[1];
-                    const float4 C1 = reinterpret_cast<const float4 *>(A.jp + i1 * RS + 1)[0];
-                    const float4 D1 = reinterpret_cast<const float4 *>(A.jp + i1 * RS + 1)[1];
-                    lxi[q] = make_float2(-C0.x, -C1.x);
-                    lyi[q] = make_float2(-C0.z, -C1.z);
-                    lzi[q] = make_float2(-D0.x, -D1.x);
-                }
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    sum[q][r] = zero2;
-                    cmp[q][r] = zero2;
-                }
-            }
-        }
-        const JPart *T = tiles + (size_t)s * JT * RS;
-        float2 acc[P][4];
-#pragma unroll
-        for (int q = 0; q < P; ++q)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[q][r] = zero2;
-        const int ibase = cur_b * IB, jbase = mt.jt * JT;
-        int self0[P], self1[P];
-        if (jbase < ibase + IB && ibase < jbase + JT) {
-            if constexpr (JT == IB && JT == 128 && P == 2 && COMP) {
-                // The tile is the i-block itself: its 32-particle quarter k
-                // holds slot k of every lane (particle 32 k + lane), so each
-                // quarter runs the lane-diagonal form for its slot. (The
-                // compensated kernels only: with it, the plain kernel compiled
-                // to 96 instead of 112 registers and ran 7% slower; the
-                // compensated ones gained 2-3%.)
-#pragma unroll
-                for (int q = 0; q < P; ++q) self0[q] = self1[q] = lane;
-                // Quarters past a short last tile hold only padding: skipped.
+                int64_t i0 = row0 + (int64_t)b * kBlock + 64 * q + lane, i1 = i0 + 32;
+                if (!NB_IN(A.err, 64, i1 < A.cap_padded)) i0 = i1 = 0;
+                const float4 u = A.cp[i0 * RS], w = A.cp[i1 * RS];
+                I.x[q] = make_float2(-u.x, -w.x);
+                I.y[q] = make_float2(-u.y, -w.y);
+                I.z[q] = make_float2(-u.z, -w.z);
+                I.hm[q] = make_float2(u.w, w.w);
+                if (weights == kProduct)
+                    I.hm[q] = make_float2(mutual_scale(u.w, hm0, eps), mutual_scale(w.w, hm0, eps));
                 if constexpr (HL) {
-                    tile_pass_hl<P, 32, 4, true, true, 0>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0, self1);
-                    if (mt.len > 32)
-                        tile_pass_hl<P, 32, 4, true, true, 1>(T + 64, xi, yi, zi, lxi, lyi, lzi, acc, eps2,
-                                                              self0, self1);
-                    if (mt.len > 64)
-                        tile_pass_hl<P, 32, 4, true, true, 2>(T + 128, xi, yi, zi, lxi, lyi, lzi, acc, eps2,
-                                                              self0, self1);
-                    if (mt.len > 96)
-                        tile_pass_hl<P, 32, 4, true, true, 3>(T + 192, xi, yi, zi, lxi, lyi, lzi, acc, eps2,
-                                                              self0, self1);
-                } else {
-                    constexpr bool NW = kDefaultRefine != 0;
-                    tile_pass<P, 32, 4, true, kMixAll, NW, true, 0>(T, xi, yi, zi, acc, eps2, self0, self1);
-                    if (mt.len > 32)
-                        tile_pass<P, 32, 4, true, kMixAll, NW, true, 1>(T + 32, xi, yi, zi, acc, eps2, self0,
-                                                                        self1);
-                    if (mt.len > 64)
-                        tile_pass<P, 32, 4, true, kMixAll, NW, true, 2>(T + 64, xi, yi, zi, acc, eps2, self0,
-                                                                        self1);
-                    if (mt.len > 96)
-                        tile_pass<P, 32, 4, true, kMixAll, NW, true, 3>(T + 96, xi, yi, zi, acc, eps2, self0,
-                                                                        self1);
+                    const float4 ul = A.cp[i0 * RS + 1], wl = A.cp[i1 * RS + 1];
+                    I.lx[q] = make_float2(-ul.x, -wl.x);
+                    I.ly[q] = make_float2(-ul.y, -wl.y);
+                    I.lz[q] = make_float2(-ul.z, -wl.z);
                 }
-            } else {
 #pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    self0[q] = ibase + (2 * q) * 32 + lane - jbase;
-                    self1[q] = self0[q] + 32;
-                }
-                if (mt.len == JT) {
-                    if constexpr (HL)
-                        tile_pass_hl<P, JT, 1, true, true>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0,
-                                                           self1);
-                    else
-                        tile_pass<P, JT, 1, true, kMixAll, kDefaultRefine != 0>(T, xi, yi, zi, acc, eps2,
-                                                                                self0, self1);
-                } else {
-                    // A short last tile, in 32-particle pieces (self indices
-                    // relative to each piece).
-                    for (int o = 0; o < mt.len; o += 32) {
-                        if constexpr (HL)
-                            tile_pass_hl<P, 32, 1, true, true>(T + o * RS, xi, yi, zi, lxi, lyi, lzi, acc, eps2,
-                                                               self0, self1);
-                        else
-                            tile_pass<P, 32, 1, true, kMixAll, kDefaultRefine != 0>(T + o, xi, yi, zi, acc,
-                                                                                    eps2, self0, self1);
-#pragma unroll
-                        for (int q = 0; q < P; ++q) {
-                            self0[q] -= 32;
-                            self1[q] -= 32;
-                        }
-                    }
-                }
-            }
-        } else if (mt.len == JT) {
-            if constexpr (HL)
-                tile_pass_hl<P, JT, 4, false, true>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0,
-                                                    self1);
-            else
-                tile_pass<P, JT, 4, false, kMixAll, kDefaultRefine != 0>(T, xi, yi, zi, acc, eps2,
-                                                                         self0, self1);
-        } else {
-            // A short last tile, in 32-particle pieces.
-            for (int o = 0; o < mt.len; o += 32) {
-                if constexpr (HL)
-                    tile_pass_hl<P, 32, 4, false, true>(T + o * RS, xi, yi, zi, lxi, lyi, lzi, acc, eps2,
-                                                        self0, self1);
-                else
-                    tile_pass<P, 32, 4, false, kMixAll, kDefaultRefine != 0>(T + o, xi, yi, zi, acc, eps2,
-                                                                             self0, self1);
+                for (int r = 0; r < 4; ++r)
+                    ssum[(4 * q + r) * 32 + lane] = scmp[(4 * q + r) * 32 + lane] = zero2;
             }
         }
-#pragma unroll
-        for (int q = 0; q < P; ++q)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                if (COMP) {
-                    const float2 y = add2(acc[q][r], neg2(cmp[q][r]));
-                    const float2 t = add2(sum[q][r], y);
-                    cmp[q][r] = add2(add2(t, neg2(sum[q][r])), neg2(y));
-                    sum[q][r] = t;
-                } else {
-                    sum[q][r] = add2(sum[q][r], acc[q][r]);
+        const MPart *T = tiles + (size_t)s * kTile * RS;
+        const int groups = mt.len / 32, block = mt.tile / kBlockTiles;
+        if (block > b && block < band_end) {
+            float4 *dst = pj + ((int64_t)mt.tile * kTile - (int64_t)(b + 1) * kBlock) + lane;
+            if (NB_IN(A.err, 65, dst >= A.pj && dst + kTile - lane <= A.pj + A.pj_len))
+#pragma unroll 1
+                for (int g = 0; g < groups; ++g) {
+                    float ja[4];
+                    run_group<P, UNR, true, HL, kAny>(weights, T + g * 32 * RS, lane, I, acc, ja, eps2);
+                    dst[32 * g] = make_float4(ja[0], ja[1], ja[2], ja[3]);
                 }
+        } else {
+            const int g0 = block == b ? mt.tile % kBlockTiles * (kTile / 32) : -kTile;
+#pragma unroll 1
+            for (int g = 0; g < groups; ++g) {
+                const MPart *G = T + g * 32 * RS;
+                const int self = g0 < 0 ? -1 : g0 + g;
+                if (slots > 2) one_sided_group<P, P, HL>(weights, G, lane, self, I, acc, eps2);
+                else one_sided_group<P, 1, HL>(weights, G, lane, self, I, acc, eps2);
             }
+        }
+        if (!one_block || mt.last) fold();
     }
     if (!bad) {
         if (cur_item >= 0) write_out();
@@ -653,61 +609,88 @@ __global__ void __launch_bounds__(WARPS * 32) batched_pair_kernel(const BatchArg
     __syncwarp();
 }
 
-// Per particle: add the chunk sums of its (cluster, i-block) in chunk order
-// and remove the factors the pair sums carry (accel_scale, pot_scale of the
-// batched kernel's refine setting). One CTA per padded i-block of kBatchIB
-// rows (which divides kClusterPad, so the block lies inside one cluster), one
-// thread per particle.
-template <bool COMP>
-__global__ void batch_combine_kernel(const float4 *__restrict__ partial,
-                                     const int64_t *__restrict__ off, const int64_t *__restrict__ poff,
-                                     const int64_t *__restrict__ ibase, int64_t C,
-                                     float *__restrict__ a, float *__restrict__ p,
-                                     int64_t partial_len, int64_t n_total, int *err) {
-    // poff holds the validated padded sizes: all zero when the planner
-    // rejected the offsets, so nothing is written for an invalid batch, and
-    // a valid cluster's real size never exceeds its padded size.
-    constexpr int ib = kBatchIB;
-    const int64_t s = (int64_t)blockIdx.x * ib;
-    if (s >= poff[C]) return;
-    const int64_t c = padded_cluster(poff, C, s);
-    const int64_t psz = poff[c + 1] - poff[c];
-    const int64_t o = off[c];
-    const int64_t nc = off[c + 1] - o < psz ? off[c + 1] - o : psz;
-    const int64_t b = (s - poff[c]) / ib, w = threadIdx.x, li = b * ib + w;
+// Per particle: the j-side sums of the earlier rows of its band, in row order, then
+// the items of its own row, in chunk order; then the factors the weights left out.
+template <bool HL>
+__global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, float *__restrict__ a,
+                                                            float *__restrict__ p) {
+    pdl_wait_then_release();
+    constexpr int RS = HL ? kHLRecords : 1;
+    if ((int64_t)blockIdx.x * kBlock >= A.poff[A.C]) return;  // (zero when the plan rejected the offsets)
+    const BmBlock B = A.block[blockIdx.x];
+    const BatchSplit split = *A.split;
+    const int c = B.cluster, b = B.b, nt = B.nt;
+    const int64_t row0 = (int64_t)(blockIdx.x - b) * kBlock;
+    const int64_t li = (int64_t)b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
     if (li >= nc) return;
-    const int64_t nch = chunks_of(psz / kBatchJT);
-    const int64_t first = ibase[c] + b * nch;
     float S[4] = {0.f, 0.f, 0.f, 0.f}, E[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int64_t k = 0; k < nch; ++k) {
-        const int64_t base = (first + k) * (COMP ? 2 : 1) * ib + w;
-        if (!NB_IN(err, 14, base + (COMP ? ib : 0) < partial_len)) continue;
-        const float4 hi = partial[base];
-        const float h[4] = {hi.x, hi.y, hi.z, hi.w};
-        if (COMP) {
-            const float4 lo = partial[base + ib];
-            const float l[4] = {lo.x, lo.y, lo.z, lo.w};
+    constexpr int K = 8;  // loads in flight
+    const int s0 = b / split.band * split.band, len = min(s0 + split.band, nt) - s0;
+    const int64_t pj0 = batch_pj_entry(split.band, row0, nt, s0) + threadIdx.x;
+    for (int r = s0; r < b; r += K) {
+        float4 v[K];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                // TwoSum(S, h) then add the chunk's lost low part (h - l is its value)
-                const float t = __fadd_rn(S[q], h[q]);
-                const float bp = __fsub_rn(t, S[q]);
-                const float e = __fadd_rn(__fsub_rn(S[q], __fsub_rn(t, bp)), __fsub_rn(h[q], bp));
-                S[q] = t;
-                E[q] = __fadd_rn(E[q], __fsub_rn(e, l[q]));
-            }
-        } else {
+        for (int k = 0; k < K; ++k) {
+            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r + k >= b) continue;
+            const int64_t e = r + k - s0;  // rows before it in the band
+            const int64_t at = pj0 + (e * len - e * (e + 1) / 2 + (b - r - k - 1)) * kBlock;
+            if (NB_IN(A.err, 66, at < A.pj_len)) v[k] = __ldcg(A.pj + at);
+        }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) S[q] = __fadd_rn(S[q], h[q]);
+        for (int k = 0; k < K; ++k) {
+            if (r + k >= b) break;
+            const float h[4] = {-v[k].x, -v[k].y, -v[k].z, v[k].w};
+            comp_add(S, E, h);
         }
     }
-    const int64_t gi = o + li;
-    if (!NB_IN(err, 14, gi >= 0 && gi < n_total)) return;
-    constexpr float as = accel_scale(kDefaultRefine), ps = pot_scale(kDefaultRefine);
-    a[3 * gi + 0] = as * __fadd_rn(S[0], E[0]);
-    a[3 * gi + 1] = as * __fadd_rn(S[1], E[1]);
-    a[3 * gi + 2] = as * __fadd_rn(S[2], E[2]);
-    p[gi] = ps * __fadd_rn(S[3], E[3]);
+    const int met = nt - (b - s0), q = nt == 1 ? 1 : split.items(met);
+    for (int j = 0; j < q; j += K) {
+        float4 u[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            u[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j + k >= q) continue;
+            if (split.parts > 1) {  // a part past the last particle was not evaluated
+                int v0, v1;
+                split.range(met, j + k, &v0, &v1);
+                if ((int64_t)batch_met_tile(split.band, nt, b, v0) * kTile >= nc) continue;
+            }
+            const int64_t at = ((int64_t)B.first + j + k) * kBlock + threadIdx.x;
+            if (NB_IN(A.err, 67, at < A.pi_len)) u[k] = __ldcg(A.pi + at);
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (j + k >= q) break;
+            const float h[4] = {u[k].x, u[k].y, u[k].z, u[k].w};
+            comp_add(S, E, h);
+        }
+    }
+    float v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = -2.f * __fadd_rn(S[r], E[r]);
+    const float hm0 = A.cp[row0 * RS].w;
+    const int weights = cluster_weights(A, c, nt);
+    if (weights == kEqual) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] *= hm0;
+    } else if (weights == kProduct) {
+        const float d = mutual_scale(A.cp[((int64_t)blockIdx.x * kBlock + threadIdx.x) * RS].w, hm0, A.eps[c]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = __fdiv_rn(v[r], d);
+    }
+    const int64_t i = o + li;
+    if (!NB_IN(A.err, 68, i >= 0 && i < A.n_total)) return;
+    a[3 * i + 0] = v[0];
+    a[3 * i + 1] = v[1];
+    a[3 * i + 2] = v[2];
+    p[i] = v[3];
+}
+
+template <int S, bool HL>
+constexpr size_t bm_smem() {
+    return (size_t)S * (kTile * (HL ? kHLRecords : 1) * sizeof(MPart) + sizeof(uint64_t) + sizeof(BmStage) +
+                        sizeof(int)) + (size_t)2 * 4 * kBatchP * 32 * sizeof(float2);
 }
 
 // Leap-frog pieces that do not pack (the batched pack follows them).
@@ -724,86 +707,12 @@ __global__ void batch_kick_drift_kernel(double *__restrict__ x, double *__restri
     x[k] = x[k] + dt * vc;           // Eq. (2)
 }
 
-// Plain mode: the same kick and drift for the particles of one block of
-// kClusterPad padded rows, fused with the packing of the moved positions
-// (batch_pack_kernel<double>'s records), so the positions are read once.
-__global__ void __launch_bounds__(kClusterPad) batch_kick_drift_pack_kernel(
-    double *__restrict__ x, double *__restrict__ v, const float *__restrict__ a,
-    const float *__restrict__ m, const int64_t *__restrict__ off, const int64_t *__restrict__ poff,
-    int64_t C, double dt, int kick_back, JPart *__restrict__ jp) {
-    const int64_t s = (int64_t)blockIdx.x * kClusterPad;
-    if (s >= poff[C]) return;
-    const int64_t c = padded_cluster(poff, C, s);
-    const int64_t li = s - poff[c] + threadIdx.x, o = off[c], nc = off[c + 1] - o;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (li < nc) {
-        const int64_t i = o + li;
-        const double h = 0.5 * dt;
-        float q[3];
-        for (int k = 0; k < 3; ++k) {
-            const int64_t e = 3 * i + k;
-            const double g = -(double)a[e];
-            double vc = v[e];
-            if (kick_back) vc = vc + h * g;  // Eq. (3) of the previous step
-            vc = vc + h * g;                 // Eq. (1)
-            v[e] = vc;
-            const double xn = x[e] + dt * vc;  // Eq. (2)
-            x[e] = xn;
-            q[k] = (float)xn;
-        }
-        const float hm = -0.5f * m[i];
-        lo = make_float4(-q[0], -q[0], -q[1], -q[1]);
-        hi = make_float4(-q[2], -q[2], hm, hm);
-    }
-    float4 *dst = reinterpret_cast<float4 *>(jp + s + threadIdx.x);
-    dst[0] = lo;
-    dst[1] = hi;
-}
-
 __global__ void batch_kick_kernel(double *__restrict__ v, const float *__restrict__ a, int64_t n,
                                   double dt) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= 3 * n) return;
     v[k] = v[k] + (0.5 * dt) * (-(double)a[k]);  // Eq. (3)
 }
-
-// Registry of batched shapes.
-template <int W, int I, int J, int S, bool C, bool H>
-cudaError_t launch_batched(const BatchArgs &a, int grid, size_t smem, cudaStream_t st) {
-    batched_pair_kernel<W, I, J, S, C, H><<<grid, W * 32, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-struct BatchVariant {
-    int threads, ipt, jtile, stages;
-    bool comp, hl;
-    const void *kernel;
-    size_t smem;
-    cudaError_t (*launch)(const BatchArgs &, int, size_t, cudaStream_t);
-};
-
-template <int W, int S, int J, int RS>
-constexpr size_t batch_smem() {
-    return (size_t)W * S * (J * RS * sizeof(JPart) + sizeof(uint64_t) + sizeof(StageMeta) + sizeof(int));
-}
-
-// threads = warps x 32; ipt; jtile; stages; compensated; HL records
-#define NB_BVARIANT(W, I, J, S, C, H)                                                           \
-    {W * 32, I, J, S, C, H, (const void *)batched_pair_kernel<W, I, J, S, C, H>,                  \
-     batch_smem<W, S, J, H ? kHLRecords : 1>(), launch_batched<W, I, J, S, C, H>}
-
-// One warp per CTA (up to 18 resident per SM, bounded by shared memory):
-// 0.902 against 0.943 ms per plain evaluation of 1024 clusters with 4 warps
-// per CTA (16 resident), the compensated mode unchanged (0.958 ms); 2 stages
-// or 4 were slower (GB300, one process, interleaved).
-static const BatchVariant kBatch[] = {
-    NB_BVARIANT(1, 4, 128, 3, false, false),
-    NB_BVARIANT(1, 4, 128, 3, true, false),
-    // Compensated on FP64 state (HL records, 64 B per particle): 2 stages keep
-    // 13 one-warp CTAs per SM resident (3 stages: 9, bounded by shared memory).
-    NB_BVARIANT(1, 4, 128, 2, true, true),
-};
-#undef NB_BVARIANT
 
 }  // namespace nbk
 
@@ -812,144 +721,144 @@ using namespace nbx;
 
 namespace {
 
-enum BSlot : int {
-    B_JP = SLOT_BATCH_JP,
-    B_POFF = SLOT_BATCH_POFF,
-    B_ITEMS = SLOT_BATCH_ITEMS,
-    B_NITEMS = SLOT_BATCH_COUNT,
-    B_PART = SLOT_BATCH_PART,
-    B_IBASE = SLOT_BATCH_IBASE,
-    B_FRAME = SLOT_BATCH_FRAME,
-    B_PLANNED = SLOT_BATCH_PLANNED
+constexpr int kBmStages = 3;
+constexpr auto kBmPair = bm_pair_kernel<kBmStages, 12, 4, false>;
+constexpr auto kBmPairHL = bm_pair_kernel<kBmStages, 12, 4, true>;
+
+PairVariant bm_variant(bool hl) {
+    PairVariant v{};
+    v.tile.threads = 32;
+    v.kernel = (const void *)(hl ? kBmPairHL : kBmPair);
+    v.smem = hl ? bm_smem<kBmStages, true>() : bm_smem<kBmStages, false>();
+    return v;
+}
+
+struct BatchCall {
+    const int64_t *offsets;
+    int64_t C, n_total;
+    const float *eps;
+    bool hl;  // HL records (compensated mode on FP64 state)
 };
 
-void *bslot(nb_ctx *ctx, int k) { return ctx_ext(ctx).buf[k]; }
-
-nb_status bensure(nb_ctx *ctx, int k, size_t bytes) {
-    ExtState &s = ctx_ext(ctx);
-    cudaError_t e = ensure_buffer(&s.buf[k], &s.cap[k], bytes);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (batched)");
-    return NB_OK;
-}
-
-struct BatchPlanHost {
-    const BatchVariant *v;
-    int64_t n_total;
-    int64_t cap_padded, cap_items;
-    int grid;
+// Where a call's positions come from: FP32, or FP64 state with the leap-frog's
+// kicks and drift to be applied first (kick).
+struct BatchSource {
+    const float *x32;
+    double *x64, *v;
+    const float *a, *m;
+    double dt;
+    int kick, kick_back;
 };
 
-int batch_resident(const BatchVariant &v, int sm_count) {
-    if (v.smem > 48 * 1024)
-        cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.kernel, v.threads, v.smem) !=
-            cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    cudaGetLastError();
-    return per_sm * sm_count;
-}
-
-// Scratch for a batch, sized from (n_total, C) alone (offsets stay on the device).
-nb_status batch_prepare(nb_ctx *ctx, int64_t C, int64_t n_total, bool comp, bool hl,
-                        BatchPlanHost *out) {
-    const BatchVariant &v = kBatch[hl ? 2 : comp ? 1 : 0];
-    const int ib = 32 * v.ipt;  // one warp per work item
-    if (ib != kBatchIB || v.jtile != kBatchJT)
-        return fail(ctx, NB_ERR_ARG, "batched shape does not match the planner's block sizes");
-    out->v = &v;
-    out->n_total = n_total;
-    out->cap_padded = n_total + C * (int64_t)kClusterPad;
-    out->cap_items = kMaxChunks * (out->cap_padded / ib) + 1;
-    if (out->cap_items > 0x7fffffff || C > 0x7fffffff)
-        return fail(ctx, NB_ERR_ARG, "batch too large for 32-bit work items");
-    out->grid = batch_resident(v, ctx_sm_count(ctx));
-    nb_status st;
-    if ((st = bensure(ctx, B_JP, (size_t)out->cap_padded * (hl ? kHLRecords : 1) * sizeof(JPart))) !=
-        NB_OK)
-        return st;
-    if ((st = bensure(ctx, B_POFF, (size_t)(C + 1) * sizeof(int64_t))) != NB_OK) return st;
-    if ((st = bensure(ctx, B_ITEMS, (size_t)out->cap_items * sizeof(int4))) != NB_OK) return st;
-    if ((st = bensure(ctx, B_NITEMS, 2 * sizeof(int))) != NB_OK) return st;  // count, queue head
-    if ((st = bensure(ctx, B_IBASE, (size_t)std::max<int64_t>(C, 1) * sizeof(int64_t))) != NB_OK)
-        return st;
-    if ((st = bensure(ctx, B_PART, (size_t)out->cap_items * ib * sizeof(float4) * (comp ? 2 : 1))) !=
-        NB_OK)
-        return st;
-    return NB_OK;
-}
-
-nb_status batch_plan(nb_ctx *ctx, const int64_t *offsets, const float *eps, int64_t C,
-                     const BatchPlanHost &h, cudaStream_t st) {
-    BatchPlanArgs P{};
-    P.off = offsets;
-    P.eps = eps;
-    P.C = C;
-    P.n_total = h.n_total;
-    P.cap_padded = h.cap_padded;
-    P.cap_items = h.cap_items;
-    P.poff = static_cast<int64_t *>(bslot(ctx, B_POFF));
-    P.items = static_cast<int4 *>(bslot(ctx, B_ITEMS));
-    P.ibase = static_cast<int64_t *>(bslot(ctx, B_IBASE));
-    P.nitems = static_cast<int *>(bslot(ctx, B_NITEMS));
-    P.err = ctx_err_word(ctx);
-    // The previous plan is reused when the offsets and eps are the same
-    // values (checked on the device); it can only be in the scratch if the
-    // last plan was made for the same (C, n_total), which sized the scratch.
+nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     ExtState &es = ctx_ext(ctx);
-    nb_status rs = bensure(ctx, B_PLANNED, (size_t)(C + 1) * sizeof(int64_t) + (size_t)C * sizeof(uint32_t));
-    if (rs != NB_OK) return rs;
-    P.planned_off = static_cast<int64_t *>(bslot(ctx, B_PLANNED));
-    P.planned_eps = reinterpret_cast<uint32_t *>(P.planned_off + C + 1);
-    P.replan = !(es.plan_clusters == C && es.plan_total == h.n_total);
-    batch_plan_kernel<<<1, kPlanThreads, 0, st>>>(P);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        es.plan_clusters = es.plan_total = -1;
-        return cuda_fail(ctx, e, "batch plan launch");
-    }
-    es.plan_clusters = C;
-    es.plan_total = h.n_total;
-    return NB_OK;
-}
-
-// pack (already done by the caller of this helper) -> reset queue -> pair kernel
-nb_status batch_pair(nb_ctx *ctx, const int64_t *offsets, int64_t C, const float *eps, float *a,
-                     float *p, const BatchPlanHost &h, cudaStream_t st) {
-    int *nit = static_cast<int *>(bslot(ctx, B_NITEMS));
-    cudaError_t e = cudaMemsetAsync(nit + 1, 0, sizeof(int), st);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "queue reset");
-    BatchArgs A{};
-    A.jp = static_cast<const JPart *>(bslot(ctx, B_JP));
-    A.off = offsets;
-    A.poff = static_cast<const int64_t *>(bslot(ctx, B_POFF));
-    A.eps = eps;
-    A.items = static_cast<const int4 *>(bslot(ctx, B_ITEMS));
-    A.nitems = nit;
-    A.counter = nit + 1;
-    A.partial = static_cast<float4 *>(bslot(ctx, B_PART));
+    BmArgs A{};
+    A.off = k.offsets;
+    A.eps = k.eps;
+    A.C = k.C;
+    A.n_total = k.n_total;
+    A.cap_padded = k.n_total + k.C * (int64_t)kBlock;
+    const int64_t blocks = A.cap_padded / kBlock, most = padded_size(k.n_total) / kBlock;
+    A.want_items = small ? blocks : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k.hl));
+    A.cap_items = blocks + A.want_items + 1;  // at most one per row beyond the number wanted
+    if (A.cap_items > INT_MAX || k.C > INT_MAX) return fail(ctx, NB_ERR_ARG, "batch too large for 32-bit work items");
+    A.max_band = small ? 1 : (int)std::min(most, std::max<int64_t>(kMinBand, kPjEntries / (blocks * (kBlock / 2))));
+    const int64_t pj = (blocks + 1) * (kBlock / 2 * (A.max_band - 1));
+    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    // [planned sizes, item count, queue head, split][poff][ibase][planned offsets][notes][padded blocks]
+    const size_t b_off = al((size_t)(k.C + 1) * sizeof(int64_t)), b_c = al((size_t)k.C * sizeof(int));
+    const size_t b_blk = al((size_t)blocks * sizeof(BmBlock));
+    const size_t plan_before = es.cap[SLOT_BATCH_PLAN];
+    cudaError_t e = cudaSuccess;
+    auto need = [&](int slot, size_t bytes) {
+        if (e == cudaSuccess) e = ensure_buffer(&es.buf[slot], &es.cap[slot], bytes);
+    };
+    need(SLOT_BATCH_PLAN, 256 + 3 * b_off + b_c + b_blk);
+    if (es.cap[SLOT_BATCH_PLAN] != plan_before) es.batch_plan = false;
+    need(SLOT_BATCH_ITEMS, (size_t)A.cap_items * sizeof(int4));
+    need(SLOT_MUTUAL_CP, (size_t)A.cap_padded * (k.hl ? kHLRecords : 1) * sizeof(MPart));
+    need(SLOT_MUTUAL_PI, (size_t)A.cap_items * kBlock * sizeof(float4));
+    need(SLOT_MUTUAL_PJ, (size_t)pj * sizeof(float4));
+    if (k.hl) need(SLOT_BATCH_FRAME, (size_t)k.C * sizeof(double4));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (batched)");
+    unsigned char *plan = static_cast<unsigned char *>(es.buf[SLOT_BATCH_PLAN]);
+    A.planned = reinterpret_cast<int64_t *>(plan);
+    A.nitems = reinterpret_cast<int *>(plan + 64);
+    A.head = A.nitems + 1;
+    A.split = reinterpret_cast<BatchSplit *>(A.nitems + 2);
+    plan += 256;
+    A.poff = reinterpret_cast<int64_t *>(plan);
+    A.ibase = reinterpret_cast<int64_t *>(plan + b_off);
+    A.planned_off = reinterpret_cast<int64_t *>(plan + 2 * b_off);
+    A.notes = reinterpret_cast<int *>(plan + 3 * b_off);
+    A.block = reinterpret_cast<BmBlock *>(plan + 3 * b_off + b_c);
+    A.items = static_cast<int4 *>(es.buf[SLOT_BATCH_ITEMS]);
+    A.cp = static_cast<MPart *>(es.buf[SLOT_MUTUAL_CP]);
+    A.pi = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PI]);
+    A.pj = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PJ]);
     A.err = ctx_err_word(ctx);
     A.wait_ns = ctx_wait_ns(ctx);
-    A.cap_padded = h.cap_padded;
-    A.cap_items = h.cap_items;
-    A.partial_len = h.cap_items * (int64_t)(32 * h.v->ipt) * (h.v->comp ? 2 : 1);
+    A.pi_len = (int64_t)(es.cap[SLOT_MUTUAL_PI] / sizeof(float4));
+    A.pj_len = (int64_t)(es.cap[SLOT_MUTUAL_PJ] / sizeof(float4));
+    *out = A;
+    return NB_OK;
+}
+
+// Arguments of a call's kernels; allocates the scratch: up to 512 MiB (or 248 B per
+// particle, if that is more) of j-side sums and 60 MB of i-side sums, or, where that
+// cannot be had, no j-side sums (every pair evaluated twice) and 32 B per particle.
+nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
+    ExtState &es = ctx_ext(ctx);
+    const int64_t size = k.n_total + k.C * (int64_t)kBlock;
+    if (size <= es.batch_max_n) {
+        const nb_status st = bm_args(ctx, k, false, out);
+        if (st != NB_ERR_OOM) return st;
+        es.batch_max_n = size - 1;
+    }
+    return bm_args(ctx, k, true, out);
+}
+
+// One evaluation.
+nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource &src, float *a, float *p,
+                   cudaStream_t st) {
+    ExtState &es = ctx_ext(ctx);
+    A.fresh = !es.batch_plan;
+    cudaError_t e = launch_with_pdl(bm_plan_kernel, dim3(1), dim3(kBmPlanThreads), 0, st, A);
+    es.batch_plan = e == cudaSuccess;
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "batch plan launch");
+    const dim3 blocks((unsigned)(A.cap_padded / kBlock)), threads(kBlock);
+    double *const no_v = nullptr;
+    const float *const no_a = nullptr;
+    if (k.hl) {
+        double4 *frame = static_cast<double4 *>(es.buf[SLOT_BATCH_FRAME]);
+        if (src.kick) {
+            batch_kick_drift_kernel<<<(unsigned)((3 * k.n_total + 255) / 256), 256, 0, st>>>(
+                src.x64, src.v, src.a, k.n_total, src.dt, src.kick_back);
+            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+        }
+        batch_frame_kernel<<<(unsigned)k.C, kFrameThreads, 0, st>>>(src.x64, k.offsets, A.poff, frame);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "batched frame launch");
+        e = launch_with_pdl(bm_pack_hl_kernel, blocks, threads, 0, st, A, (const double *)src.x64, src.m,
+                            (const double4 *)frame);
+    } else if (src.x32) {
+        e = launch_with_pdl(bm_pack_kernel<const float, false>, blocks, threads, 0, st, A, src.x32, no_v, no_a, src.m,
+                            0.0, 0);
+    } else if (src.kick) {
+        e = launch_with_pdl(bm_pack_kernel<double, true>, blocks, threads, 0, st, A, src.x64, src.v, src.a, src.m,
+                            src.dt, src.kick_back);
+    } else {
+        e = launch_with_pdl(bm_pack_kernel<double, false>, blocks, threads, 0, st, A, src.x64, no_v, no_a, src.m, 0.0,
+                            0);
+    }
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "batched pack launch");
+    const PairVariant v = bm_variant(k.hl);
     {
         TimedLaunch t(ctx, 4, st);
-        e = h.v->launch(A, h.grid, h.v->smem, st);
+        e = launch_with_pdl(k.hl ? kBmPairHL : kBmPair, dim3((unsigned)resident_ctas(ctx, v)), dim3(32), v.smem, st, A);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batched pair kernel launch");
-    const int ib = 32 * h.v->ipt;
-    const unsigned nblk = (unsigned)((h.cap_padded + ib - 1) / ib);
-    if (h.v->comp)
-        batch_combine_kernel<true><<<nblk, ib, 0, st>>>(
-            A.partial, offsets, A.poff, static_cast<const int64_t *>(bslot(ctx, B_IBASE)), C, a, p,
-            A.partial_len, h.n_total, A.err);
-    else
-        batch_combine_kernel<false><<<nblk, ib, 0, st>>>(
-            A.partial, offsets, A.poff, static_cast<const int64_t *>(bslot(ctx, B_IBASE)), C, a, p,
-            A.partial_len, h.n_total, A.err);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "batched combine launch");
+    e = launch_with_pdl(k.hl ? bm_combine_kernel<true> : bm_combine_kernel<false>, blocks, threads, 0, st, A, a, p);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "batched combine launch");
     return NB_OK;
 }
 
@@ -972,17 +881,14 @@ nb_status nb_force_batched(nb_ctx *ctx, const float *x, const float *m, const in
     if (n_clusters == 0 || n_total == 0) return NB_OK;
     if (!x || !m || !offsets || !eps || !a || !p) return fail(ctx, NB_ERR_ARG, "NULL array pointer");
     DeviceGuard g(ctx_device(ctx));
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    BatchPlanHost h{};
-    if ((st = batch_prepare(ctx, n_clusters, n_total, mode == NB_COMPENSATED, false, &h)) != NB_OK)
-        return st;
-    if ((st = batch_plan(ctx, offsets, eps, n_clusters, h, s)) != NB_OK) return st;
-    batch_pack_kernel<float><<<(unsigned)(h.cap_padded / kClusterPad), kClusterPad, 0, s>>>(
-        x, m, offsets, static_cast<const int64_t *>(bslot(ctx, B_POFF)), n_clusters,
-        static_cast<JPart *>(bslot(ctx, B_JP)));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "batched pack launch");
-    return batch_pair(ctx, offsets, n_clusters, eps, a, p, h, s);
+    // One kernel for both modes: its sums are compensated.
+    const BatchCall call{offsets, n_clusters, n_total, eps, false};
+    BmArgs A;
+    if ((st = bm_prepare(ctx, call, &A)) != NB_OK) return st;
+    BatchSource src{};
+    src.x32 = x;
+    src.m = m;
+    return bm_force(ctx, call, A, src, a, p, static_cast<cudaStream_t>(stream));
 }
 
 nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const float *m,
@@ -999,45 +905,15 @@ nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const floa
         return fail(ctx, NB_ERR_ARG, "NULL array pointer");
     DeviceGuard g(ctx_device(ctx));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool hl = mode == NB_COMPENSATED;
-    BatchPlanHost h{};
-    if ((st = batch_prepare(ctx, n_clusters, n_total, hl, hl, &h)) != NB_OK) return st;
-    if ((st = batch_plan(ctx, offsets, eps, n_clusters, h, s)) != NB_OK) return st;
-    const int64_t *poff = static_cast<const int64_t *>(bslot(ctx, B_POFF));
-    JPart *jp = static_cast<JPart *>(bslot(ctx, B_JP));
-    const unsigned nb3 = (unsigned)((3 * n_total + 255) / 256);
+    const BatchCall call{offsets, n_clusters, n_total, eps, mode == NB_COMPENSATED};
+    BmArgs A;
+    if ((st = bm_prepare(ctx, call, &A)) != NB_OK) return st;
     cudaError_t e;
-
-    double4 *frame = nullptr;
-    if (hl) {
-        if ((st = bensure(ctx, B_FRAME, (size_t)n_clusters * sizeof(double4))) != NB_OK) return st;
-        frame = static_cast<double4 *>(bslot(ctx, B_FRAME));
-    }
-    const unsigned npack = (unsigned)(h.cap_padded / kClusterPad);
-    auto force = [&]() -> nb_status {
-        if (hl) {
-            batch_frame_kernel<<<(unsigned)n_clusters, kFrameThreads, 0, s>>>(x, offsets, poff, frame);
-            batch_pack_hl_kernel<<<npack, kClusterPad, 0, s>>>(x, m, offsets, poff, frame, n_clusters, jp);
-        } else {
-            batch_pack_kernel<double><<<npack, kClusterPad, 0, s>>>(x, m, offsets, poff, n_clusters, jp);
-        }
-        cudaError_t le = cudaGetLastError();
-        if (le != cudaSuccess) return cuda_fail(ctx, le, "batched pack launch");
-        return batch_pair(ctx, offsets, n_clusters, eps, a, p, h, s);
+    auto evaluate = [&](int kick, int kick_back) {
+        return bm_force(ctx, call, A, BatchSource{nullptr, x, v, a, m, dt, kick, kick_back}, a, p, s);
     };
-    auto step = [&](int kick_back) -> nb_status {
-        if (!hl) {  // kick, drift and pack in one pass, then the force
-            batch_kick_drift_pack_kernel<<<npack, kClusterPad, 0, s>>>(x, v, a, m, offsets, poff, n_clusters,
-                                                                       dt, kick_back, jp);
-            cudaError_t le = cudaGetLastError();
-            if (le != cudaSuccess) return cuda_fail(ctx, le, "leap-frog update launch");
-            return batch_pair(ctx, offsets, n_clusters, eps, a, p, h, s);
-        }
-        batch_kick_drift_kernel<<<nb3, 256, 0, s>>>(x, v, a, n_total, dt, kick_back);
-        cudaError_t le = cudaGetLastError();
-        if (le != cudaSuccess) return cuda_fail(ctx, le, "leap-frog update launch");
-        return force();
-    };
+    auto force = [&]() { return evaluate(0, 0); };
+    auto step = [&](int kick_back) { return evaluate(1, kick_back); };
 
     if (!a_valid && (st = force()) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
@@ -1067,7 +943,7 @@ nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const floa
         for (int k = 0; k < rest; ++k)
             if ((st = step(1)) != NB_OK) return st;
     }
-    batch_kick_kernel<<<nb3, 256, 0, s>>>(v, a, n_total, dt);
+    batch_kick_kernel<<<(unsigned)((3 * n_total + 255) / 256), 256, 0, s>>>(v, a, n_total, dt);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
     return NB_OK;
 }

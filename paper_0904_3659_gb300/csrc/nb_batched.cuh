@@ -1,0 +1,92 @@
+// nb_batched.cuh -- the work split of the batched kernels that evaluate
+// every unordered pair of a cluster once (nb_batched.cu).
+//
+// Clusters are padded to blocks of kBlock particles. Row b of a cluster is block b
+// on the i-side, held by one warp. In a band of consecutive blocks it meets its own
+// block and those of other bands for its own side, the later blocks of its band for
+// both sides. A band is as long as the batch's longest cluster (nothing is then met
+// twice but the own blocks), unless its j-side sums would take more than the scratch
+// set aside: one float4 per (row, particle of a later block of the band), at most
+// (band - 1) / 2 per particle whatever the sizes, which stay on the device.
+//
+// A row has nt - r blocks to meet (nt blocks in the cluster, r its place in the
+// band): its own, the later ones of the band, then the others. It is cut into items
+// of `chunk` consecutive blocks, or every block into `parts` items, whichever gives
+// the resident warps several items each.
+#pragma once
+
+#include <cstdint>
+
+namespace nbk {
+
+constexpr int kBlock = 128;  // particles per block: 4 per lane
+constexpr int kTile = 64;    // particles per copy
+constexpr int kBlockTiles = kBlock / kTile;
+constexpr int kMinBand = 32;  // blocks that a band may always have
+
+struct BatchSplit {
+    int band;          // blocks per band
+    int chunk, parts;  // one of them is 1
+    // Items of a row with t blocks to meet.
+    __host__ __device__ int items(int t) const { return (t + chunk - 1) / chunk * parts; }
+    // Items of rows with 1, 2 .. k blocks to meet together.
+    __host__ __device__ int64_t below(int64_t k) const {
+        const int64_t a = k / chunk;
+        return (chunk * (a * (a + 1) / 2) + (k - a * chunk) * (a + 1)) * parts;
+    }
+    // The first item of row b of a cluster of nt blocks, counted from the
+    // cluster's first (b = nt: their number).
+    __host__ __device__ int64_t first(int64_t nt, int64_t b) const {
+        const int64_t k = b / band, r = b - k * band, f = below(nt);
+        return (k ? k * (f - below(nt - band)) : 0) + (r ? f - below(nt - r) : 0);
+    }
+    // Item k of a row with t blocks to meet: the met tiles [*v0, *v1).
+    __host__ __device__ void range(int t, int k, int *v0, int *v1) const {
+        if (parts > 1) {
+            constexpr int n = kBlockTiles;
+            *v0 = k * (n / parts);
+            *v1 = *v0 + n / parts;
+            return;
+        }
+        const int q = items(t), each = t / q, more = t - each * q;  // the first `more` have one block more
+        *v0 = (k * each + (k < more ? k : more)) * kBlockTiles;
+        *v1 = *v0 + (each + (k < more)) * kBlockTiles;
+    }
+};
+
+// The split of a batch whose rows meet `met` blocks in all, for `want` items: at
+// most one item per row more.
+__host__ __device__ inline BatchSplit batch_split(int band, int64_t met, int64_t want) {
+    BatchSplit s{band, 1, 1};
+    if (met > want) s.chunk = (int)((met + want - 1) / want);
+    else while (2 * s.parts <= kBlockTiles && 2 * s.parts * met <= want) s.parts *= 2;
+    return s;
+}
+static_assert((kBlockTiles & (kBlockTiles - 1)) == 0, "parts hold equal numbers of tiles");
+
+// Blocks met by all rows of a cluster of nt blocks.
+__host__ __device__ inline int64_t batch_met(int band, int64_t nt) { return BatchSplit{band, 1, 1}.first(nt, nt); }
+
+// The v-th block that row b meets.
+__host__ __device__ inline int batch_met_block(int band, int nt, int b, int v) {
+    const int s0 = b / band * band, s1 = s0 + band < nt ? s0 + band : nt;
+    if (v < s1 - b) return b + v;
+    const int w = v - (s1 - b);
+    return w < s0 ? w : w - s0 + s1;
+}
+
+// The v-th tile that row b meets.
+__host__ __device__ inline int batch_met_tile(int band, int nt, int b, int v) {
+    return batch_met_block(band, nt, b, v / kBlockTiles) * kBlockTiles + v % kBlockTiles;
+}
+
+// The first j-side entry of row b (those of its band's later blocks' particles
+// follow) of a cluster whose first padded row is row0: kBlock (band - 1) / 2
+// entries are set aside per block.
+__host__ __device__ inline int64_t batch_pj_entry(int band, int64_t row0, int nt, int b) {
+    const int s0 = b / band * band, s1 = s0 + band < nt ? s0 + band : nt;
+    const int64_t r = b - s0, len = (int64_t)(s1 - s0) * kBlock;
+    return (row0 / kBlock + s0) * (kBlock / 2 * (band - 1)) + r * len - kBlock * (r * (r + 1) / 2);
+}
+
+}  // namespace nbk

@@ -17,18 +17,13 @@ enum ExtSlot : int {
     SLOT_P,             // potentials computed by nb_energy
     SLOT_ENERGY_BLK,    // energy block sums
     SLOT_ENERGY_OUT,    // energy result
-    SLOT_BATCH_JP,      // padded packed clusters
-    SLOT_BATCH_POFF,    // padded cluster offsets
-    SLOT_BATCH_ITEMS,   // batched work items
-    SLOT_BATCH_COUNT,   // item count and queue head
-    SLOT_BATCH_PART,    // per-item partial sums
-    SLOT_BATCH_IBASE,   // first item of each cluster
+    SLOT_BATCH_PLAN,    // batched: what the plan was made for, offsets and blocks
+    SLOT_BATCH_ITEMS,   // batched: work items
     SLOT_VJP_VP,        // packed VJP records
     SLOT_VJP_PART,      // VJP partial sums
     SLOT_HL_BOX,        // bounding-box partials of FP64 positions (HL packing)
     SLOT_ADJOINT,       // leap-frog adjoint: replayed state, position history, VJP operands
     SLOT_BATCH_FRAME,   // per-cluster HL frames (centre, grid) of the batched leap-frog
-    SLOT_BATCH_PLANNED, // the offsets and eps the current batched plan was made for
     SLOT_MUTUAL_CP,     // mutual kernels: packed particles
     SLOT_MUTUAL_PI,     //   segment sums of the i-side
     SLOT_MUTUAL_PJ,     //   j-side sums of a panel of rows
@@ -43,11 +38,11 @@ struct ExtState {
     void *buf[kSlots] = {};
     size_t cap[kSlots] = {};
     int vjp_idx = -1;  // VJP shape forced by nb_set_vjp_tile (-1: built-in)
-    // (n_clusters, n_total) of the batched plan in the scratch (-1: none).
-    int64_t plan_clusters = -1, plan_total = -1;
     // Largest n whose mutual scratch is known not to have failed to allocate:
     // above it the built-in choice is a direct shape.
     int64_t mutual_max_n = INT64_MAX, vjp_mutual_max_n = INT64_MAX;
+    int64_t batch_max_n = INT64_MAX;  // (padded particles; above it: the small scratch)
+    bool batch_plan = false;          // a plan was launched into SLOT_BATCH_PLAN
 };
 void ext_release(ExtState &s);
 

@@ -223,4 +223,31 @@ __device__ __forceinline__ void self_group(const MPart *__restrict__ T, int lane
     }
 }
 
+// The group functions for the kernel's form of the weights.
+template <int P, int UNR, bool POT, bool HL, int W>
+__device__ __forceinline__ void run_group(int weights, const MPart *G, int lane, const MutualI<P, HL> &I,
+                                          float2 (&acc)[P][4], float (&ja)[4], float2 eps2) {
+    if constexpr (W != kAny)
+        mutual_group<P, UNR, POT, HL, W>(G, lane, I, acc, ja, eps2);
+    else if (weights == kEqual)
+        mutual_group<P, UNR, POT, HL, kEqual>(G, lane, I, acc, ja, eps2);
+    else if (weights == kProduct)
+        mutual_group<P, UNR, POT, HL, kProduct>(G, lane, I, acc, ja, eps2);
+    else
+        mutual_group<P, 1, POT, HL, kWide>(G, lane, I, acc, ja, eps2);
+}
+
+template <int P, bool POT, bool HL, int W>
+__device__ __forceinline__ void run_self(int weights, const MPart *G, int lane, int self, const MutualI<P, HL> &I,
+                                         float2 (&acc)[P][4], float2 eps2) {
+    if constexpr (W != kAny)
+        self_group<P, POT, HL, W>(G, lane, self, I, acc, eps2);
+    else if (weights == kEqual)
+        self_group<P, POT, HL, kEqual>(G, lane, self, I, acc, eps2);
+    else if (weights == kProduct)
+        self_group<P, POT, HL, kProduct>(G, lane, self, I, acc, eps2);
+    else
+        self_group<P, POT, HL, kWide>(G, lane, self, I, acc, eps2);
+}
+
 }  // namespace nbk

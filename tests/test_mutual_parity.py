@@ -201,3 +201,109 @@ def test_vjp_panels(nb, ctx):
         sm = (abs(rl) * y ** 3 + abs(GP) * y).sum()
         assert np.linalg.norm(gx[k].cpu().numpy() - want_x) <= 1e-5 * sx, k
         assert abs(float(gm[k]) - want_m) <= 1e-5 * sm, k
+
+
+KINDS = ["equal", "spectrum", "tracers", "span", "equal_si", "spectrum_si"]
+BATCHES = {
+    # every edge of a group, a tile and a block; empty clusters among them
+    "edges": [1, 2, 31, 32, 33, 0, 63, 64, 65, 96, 127, 128, 129, 0, 191, 193, 255, 256, 257, 511, 513, 1000, 2049,
+              4097, 4500, 1, 160],
+    # blocks in several items, and one item per block
+    "few": [1, 33, 65, 300],
+    # several blocks per item
+    "many": list(range(1, 4200, 37)) * 3,
+}
+
+
+def batch(sizes):
+    """x, m, offsets, eps: the kinds of particles in turn."""
+    parts = [particles(n, KINDS[i % len(KINDS)]) if n else (np.zeros((0, 3), "f4"), np.zeros(0, "f4"), np.float32(1))
+             for i, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    return (np.concatenate([q[0] for q in parts]), np.concatenate([q[1] for q in parts]), off,
+            np.array([q[2] for q in parts], np.float32))
+
+
+def run_batch(nb, ctx, b, entry):
+    """The plain or compensated force, or the compensated one on FP64 state."""
+    import torch
+    x, m, off, eps = (torch.from_numpy(v).cuda() for v in b)
+    n = x.shape[0]
+    a = torch.full((n, 3), float("nan"), device="cuda")
+    p = torch.full((n,), float("nan"), device="cuda")
+    if entry == 2:
+        nb.nb_leapfrog_batched_step(ctx, x.double(), torch.zeros_like(x).double(), m, off, len(off) - 1, n, eps, a, p,
+                                    0.0, 0, False, nb.NB_COMPENSATED)
+    else:
+        nb.nb_force_batched(ctx, x, m, off, len(off) - 1, n, eps, a, p, entry)
+    nb.nb_synchronize(ctx)
+    return a.cpu().numpy(), p.cpu().numpy()
+
+
+@pytest.mark.parametrize("entry", [0, 1, 2])
+@pytest.mark.parametrize("sizes", BATCHES)
+def test_batched_edges_and_weights(nb, ctx, oracle_mod, sizes, entry):
+    b = batch(BATCHES[sizes])
+    a, p = run_batch(nb, ctx, b, entry)
+    x, m, off, eps = b
+    step = 7 if sizes == "many" else 1
+    for c in range(0, len(off) - 1, step):
+        lo, hi = off[c], off[c + 1]
+        if hi > lo:
+            ref = oracle_mod.force(x[lo:hi], m[lo:hi], eps[c])
+            assert worst(a[lo:hi], p[lo:hi], *ref) <= TOL[min(entry, 1)], (c, hi - lo, KINDS[c % len(KINDS)])
+    a2, p2 = run_batch(nb, ctx, b, entry)
+    assert a.tobytes() == a2.tobytes() and p.tobytes() == p2.tobytes()
+
+
+@pytest.mark.parametrize("entry", [0, 2])
+def test_batched_bands(nb, ctx, entry):
+    # A cluster whose blocks make more than one band, between two small ones:
+    # rows of it against FP64 sums, with the measure and tolerance of the mode.
+    sizes = [100, 100003, 64]
+    b = batch(sizes)
+    a, p = run_batch(nb, ctx, b, entry)
+    x, m, off, eps = b
+    lo, hi = off[1], off[2]
+    X, M, e2 = x[lo:hi].astype(np.float64), m[lo:hi].astype(np.float64), float(eps[1]) ** 2
+    rows = np.unique(np.concatenate([[0, sizes[1] - 1], workloads.sample_rows(sizes[1], 254, 4)]))
+    for k in rows:
+        d = X - X[k]
+        y = 1 / np.sqrt((d * d).sum(1) + e2)
+        y[k] = 0
+        t = (M * y ** 3)[:, None] * d
+        da = np.linalg.norm(a[lo + k].astype(np.float64) + t.sum(0))  # a is the sum over x_k - x_j
+        assert da <= TOL[min(entry, 1)] * np.linalg.norm(t, axis=1).sum(), k
+        assert abs(float(p[lo + k]) - M @ y) <= TOL[min(entry, 1)] * (M @ y), k
+
+
+def test_batched_far_and_nonfinite_particles_as_the_direct_kernels(nb, ctx):
+    sizes = [700, 1500, 90]
+    x, m, off, eps = batch(sizes)
+    for at in (off[0], off[1]):
+        x[at + 7] = (3e19, 0, 0)
+        x[at + 8] = (1e38, -1e38, 1e38)
+        x[at + 400] = (np.inf, 0, 0)
+        x[at + 640] = (0, np.nan, 0)
+        m[at + 3] = np.inf
+    for mode in (0, 1):
+        a, p = run_batch(nb, ctx, (x, m, off, eps), mode)
+        try:
+            nb.nb_set_tile(ctx, mode, [t for t in nb.nb_list_tiles(mode) if not t.fused and not t.packed & 64][0])
+            for c in range(len(sizes)):
+                s = slice(off[c], off[c + 1])
+                a0, p0 = run(nb, ctx, x[s], m[s], eps[c], mode)
+                assert np.array_equal(np.isnan(a0), np.isnan(a[s])) and np.array_equal(np.isnan(p0), np.isnan(p[s]))
+                assert np.array_equal(np.isinf(a0), np.isinf(a[s])) and np.array_equal(np.isinf(p0), np.isinf(p[s]))
+        finally:
+            nb.nb_set_tile(ctx, mode, None)
+
+
+def test_batched_small_batch_after_a_large_one(nb, ctx):
+    # The scratch holds the plan of another batch: results as on a fresh context.
+    small = batch([5, 200, 77])
+    with nb.Context(0) as fresh:
+        want = run_batch(nb, fresh, small, 0)
+    for sizes in (BATCHES["many"], [5, 200, 78], [200, 5, 77], [5, 200, 77]):
+        got = run_batch(nb, ctx, batch(sizes), 0)
+    assert got[0].tobytes() == want[0].tobytes() and got[1].tobytes() == want[1].tobytes()
