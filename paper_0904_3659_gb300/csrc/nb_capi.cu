@@ -293,7 +293,7 @@ int mutual_from_fp64(nb_ctx *ctx, int64_t n, bool comp) {
 // packed or to be packed from FP32 x, m. `jp` may be supplied by the caller
 // (already packed); else x, m are packed into the context's buffer.
 nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *prepacked,
-                    int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st) {
+                    int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st, bool only_p) {
     const PairVariant *vp = &choose_variant(ctx, n, comp);
     // The mutual kernels pack for themselves. The built-in choice falls back to
     // a direct shape when their scratch cannot be allocated.
@@ -311,7 +311,7 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *pr
     if ((prepacked || !p) && vp->tile.fused) vp = pair_variant(comp, pair_default_unfused_index(comp, n));
     // No potential wanted: the same shape without the potential term, if compiled.
     if (!p)
-        if (const PairVariant *tw = no_pot_twin(*vp)) vp = tw;
+        if (const PairVariant *tw = sums_twin(*vp, kSumA)) vp = tw;
     // The cluster form when its clusters do not all fit at once: the chunked
     // form of the same shape and split (partials through global memory).
     // Smaller clusters that fit would mean longer chunks: at N = 6144 the
@@ -386,7 +386,10 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *pr
     pa.partial_len = (int64_t)(ctx->partial_bytes / sizeof(float4));
     {
         TimedLaunch t(ctx, K_PAIR, st);
-        e = v.launch(pa, plan.grid, v.smem, st);
+        // Potential only: the same shape and work split without the rest, if compiled.
+        const PairVariant *tw = only_p ? sums_twin(v, kSumP) : nullptr;
+        if (tw) resident_ctas(ctx, *tw);  // (its shared memory allowed)
+        e = (tw ? *tw : v).launch(pa, plan.grid, v.smem, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "pair kernel launch");
 
@@ -414,8 +417,8 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *pr
 
 nb_status reserve_hl(nb_ctx *ctx, int64_t n) {
     size_t bytes = 0;
-    for (bool no_pot : {false, true}) {
-        const PairVariant &v = *hl_variant(n, no_pot);
+    for (PairSums sums : {kSumAll, kSumA}) {
+        const PairVariant &v = *hl_variant(n, sums);
         bytes = std::max(bytes, make_plan(v, n, resident_ctas(ctx, v)).partial_bytes);
     }
     cudaError_t e = ensure_buffer(&ctx->d_partial, &ctx->partial_bytes, bytes);
@@ -424,8 +427,8 @@ nb_status reserve_hl(nb_ctx *ctx, int64_t n) {
 }
 
 nb_status run_force_hl(nb_ctx *ctx, const JPart *jp, int64_t n, float eps, float *a, float *p,
-                       cudaStream_t st) {
-    const PairVariant &v = *hl_variant(n, p == nullptr);
+                       cudaStream_t st, bool only_p) {
+    const PairVariant &v = *hl_variant(n, p ? kSumAll : kSumA);
     const PairPlan plan = make_plan(v, n, resident_ctas(ctx, v));
     nb_status rs = reserve_hl(ctx, n);
     if (rs != NB_OK) return rs;
@@ -445,7 +448,9 @@ nb_status run_force_hl(nb_ctx *ctx, const JPart *jp, int64_t n, float eps, float
     cudaError_t e;
     {
         TimedLaunch t(ctx, K_PAIR, st);
-        e = v.launch(pa, plan.grid, v.smem, st);
+        const PairVariant &w = only_p ? *hl_variant(n, kSumP) : v;
+        if (only_p) resident_ctas(ctx, w);  // (its shared memory allowed)
+        e = w.launch(pa, plan.grid, w.smem, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "pair kernel launch (HL)");
     ReduceArgs ra{};
@@ -581,7 +586,7 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode) {
     // Every shape this context might pick for n (and the shapes' twins
     // without the potential): reserve for the largest.
     for (int k = 0; k < pair_variant_count(comp); ++k) {
-        const PairVariant *cands[2] = {pair_variant(comp, k), no_pot_twin(*pair_variant(comp, k))};
+        const PairVariant *cands[2] = {pair_variant(comp, k), sums_twin(*pair_variant(comp, k), kSumA)};
         for (const PairVariant *vp : cands) {
             if (!vp) continue;
             if (vp->mutual >= 0) {

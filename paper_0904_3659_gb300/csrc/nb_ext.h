@@ -84,15 +84,16 @@ const nbk::PairVariant &choose_variant(nb_ctx *ctx, int64_t n, bool comp);
 
 // Compensated path on FP64 state: pair kernel on HL records (two JParts per
 // particle, nbk::kHLRecords), then the compensated combine; p may be NULL
-// (the potential is then not summed).
+// (the potential is then not summed). only_p: a is zeroed, not summed.
 nb_status run_force_hl(nb_ctx *ctx, const nbk::JPart *jp, int64_t n, float eps, float *a, float *p,
-                       cudaStream_t st);
+                       cudaStream_t st, bool only_p = false);
 // Allocate the HL path's partial sums for n (before any graph capture).
 nb_status reserve_hl(nb_ctx *ctx, int64_t n);
 
 // pack (unless prepacked) -> pair -> combine, enqueued on st.
 nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const nbk::JPart *prepacked,
-                    int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st);
+                    int64_t n, float eps, float *a, float *p, bool comp, cudaStream_t st,
+                    bool only_p = false);
 
 // Mutual kernels (nb_mutual.cu). mutual_reserve allocates what n needs; the
 // records are then packed by run_mutual from x, m, or, with x NULL, by a kernel

@@ -190,11 +190,12 @@ struct PairVariant {
 
 // Registry of compiled variants (nb_pair.cu).
 // HL variants: compensated kernels on HL records (positions from FP64 state,
-// see kHLRecords); no_pot selects the twin that sums a_i only.
-const PairVariant *hl_variant(int64_t n, bool no_pot = false);
-// The twin of a plain packed shape that sums a_i only (12 FP32 operations
-// per pair), or nullptr if that shape has none.
-const PairVariant *no_pot_twin(const PairVariant &v);
+// see kHLRecords).
+enum PairSums : int { kSumAll = 0, kSumA = 1, kSumP = 2 };  // all, a_i only, the potential only
+const PairVariant *hl_variant(int64_t n, PairSums sums);
+// The twin of a plain packed shape with some of the sums only (kSumA: 12 FP32
+// operations per pair, kSumP: 8), or nullptr if that shape has none.
+const PairVariant *sums_twin(const PairVariant &v, PairSums sums);
 // The chunked form (fused = 1) of a single-launch shape, or nullptr.
 const PairVariant *chunked_twin(const PairVariant &v);
 int pair_variant_count(bool comp);

@@ -89,11 +89,14 @@ __global__ void pack_f32_kernel(const float *__restrict__ x, const float *__rest
 //                 particle, see kHLRecords): x_i - x_j is formed from the
 //                 exact difference of the grid parts plus the difference of
 //                 the remainders (tile_pass_hl)
-//   NP            no potential: only a_i is summed (12 FP32 operations per
-//                 pair); the potential slot of the partial sums stays zero.
+//   SUMS          kSumAll; kSumA: no potential, only a_i is summed (12 FP32
+//                 operations per pair); kSumP: only the potential (8). The slots
+//                 of the partial sums left out stay zero; the others are the
+//                 same bit for bit.
 template <int THREADS, int IPT, int JT, int STAGES, int UNR, int MINB, int REL, int ACCS, int MIX,
-          bool NEWTON, bool COMP, bool HL, bool NP = false>
+          bool NEWTON, bool COMP, bool HL, int SUMS = kSumAll>
 __global__ void __launch_bounds__(THREADS, MINB) pair_kernel(const PairArgs args) {
+    constexpr bool POT = SUMS != kSumA, ACC = SUMS != kSumP;
     static_assert(IPT % 2 == 0, "i-particles are processed in packed pairs");
     static_assert(!(HL && NEWTON), "the HL pass has no Newton step");
     constexpr int P = IPT / 2;
@@ -260,15 +263,15 @@ __global__ void __launch_bounds__(THREADS, MINB) pair_kernel(const PairArgs args
                 self1[q] = self0[q] + THREADS;
             }
             if constexpr (HL)
-                tile_pass_hl<P, JT, 1, true, !NP>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0, self1);
+                tile_pass_hl<P, JT, 1, true, POT, -1, ACC>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0, self1);
             else
-                tile_pass<P, JT, 1, true, MIX, NEWTON, !NP>(T, xi, yi, zi, acc, eps2, self0, self1);
+                tile_pass<P, JT, 1, true, MIX, NEWTON, POT, -1, ACC>(T, xi, yi, zi, acc, eps2, self0, self1);
         } else {
             if constexpr (HL)
-                tile_pass_hl<P, JT, UNR, false, !NP>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0,
-                                                     self1);
+                tile_pass_hl<P, JT, UNR, false, POT, -1, ACC>(T, xi, yi, zi, lxi, lyi, lzi, acc, eps2, self0,
+                                                              self1);
             else
-                tile_pass<P, JT, UNR, false, MIX, NEWTON, !NP>(T, xi, yi, zi, acc, eps2, self0, self1);
+                tile_pass<P, JT, UNR, false, MIX, NEWTON, POT, -1, ACC>(T, xi, yi, zi, acc, eps2, self0, self1);
         }
 
         if (REL == 1) {
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(THREADS, MINB) pair_kernel(const PairArgs args
 #pragma unroll
         for (int q = 0; q < P; ++q)
 #pragma unroll
-            for (int r = 0; r < (NP ? 3 : 4); ++r) {
+            for (int r = ACC ? 0 : 3; r < (POT ? 4 : 3); ++r) {
                 if (COMP) {
                     // Kahan: the running sum's lost low part is kept in cmp
                     // (true value = sum - cmp).
@@ -1024,9 +1027,9 @@ __global__ void fill_uniform_kernel(float *x, float *m, int64_t n, uint64_t seed
 // ---------------------------------------------------------------------------
 // Launchers and the registry of compiled shapes.
 template <int T, int I, int J, int S, int U, int M, int R, int A, int X, bool N, bool C, bool F,
-          bool NP = false>
+          int SUMS = kSumAll>
 static cudaError_t launch_pair(const PairArgs &a, int grid, size_t smem, cudaStream_t st) {
-    pair_kernel<T, I, J, S, U, M, R, A, X, N, C, F, NP><<<grid, T, smem, st>>>(a);
+    pair_kernel<T, I, J, S, U, M, R, A, X, N, C, F, SUMS><<<grid, T, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1095,12 +1098,13 @@ constexpr size_t pair_smem() {
      (const void *)pair_kernel<T, I, J, S, U, M, R, A, X, (N != 0), C, false>,                  \
      pair_smem<T, I, J, S, A, C>(), launch_pair<T, I, J, S, U, M, R, A, X, (N != 0), C, false>,  \
      nullptr}
-// Shapes without the potential (NP), for callers that need only a_i; H: HL records.
-#define NB_VARIANT_NP(T, I, J, S, U, M, R, A, X, C, H, NP)                                      \
+// Shapes with some of the sums only, for callers that need only a_i or only the
+// potential; H: HL records.
+#define NB_VARIANT_OF(T, I, J, S, U, M, R, A, X, C, H, SUMS)                                     \
     {{T, I, J, S, U, M, R, A, X, 0}, C,                                                         \
-     (const void *)pair_kernel<T, I, J, S, U, M, R, A, X, false, C, H, NP>,                     \
+     (const void *)pair_kernel<T, I, J, S, U, M, R, A, X, false, C, H, SUMS>,                     \
      pair_smem<T, I, J, S, A, C, H ? kHLRecords : 1>(),                                         \
-     launch_pair<T, I, J, S, U, M, R, A, X, false, C, H, NP>, nullptr}
+     launch_pair<T, I, J, S, U, M, R, A, X, false, C, H, SUMS>, nullptr}
 // Fused single-launch shapes: T threads (T / 32 warps sharing one i-block of
 // 32 I particles), J-particle warp tiles, one shared-memory block of
 // kFusedJmax particles (stages = 1).
@@ -1223,29 +1227,34 @@ static const PairVariant kComp[] = {
     NB_MUTUAL_ENTRY(32, 0, kMutualMid, true),
     NB_MUTUAL_ENTRY(128, 0, kMutualLarge, true),
 };
-// HL variants (compensated, positions from FP64 state as HL records), with
-// and without the potential, for large and for small n.
-static const PairVariant kHL[2][2] = {
-    {NB_VARIANT_NP(256, 4, 512, 3, 4, 1, 0, 0, 63, true, true, false),   // large n (the N = 2^16
-                                                                         // leap-frog: 1% faster than 256)
-     NB_VARIANT_NP(64, 4, 128, 4, 4, 1, 0, 0, 63, true, true, false)},   // small n
-    {NB_VARIANT_NP(256, 4, 512, 3, 4, 1, 0, 0, 63, true, true, true),
-     NB_VARIANT_NP(64, 4, 128, 4, 4, 1, 0, 0, 63, true, true, true)},
+// HL variants (compensated, positions from FP64 state as HL records), for large n
+// (the N = 2^16 leap-frog: 1% faster than with 256-particle tiles) and for small n,
+// with all sums, a_i only, the potential only.
+#define NB_HL_PAIR(SUMS)                                                \
+    {NB_VARIANT_OF(256, 4, 512, 3, 4, 1, 0, 0, 63, true, true, SUMS),   \
+     NB_VARIANT_OF(64, 4, 128, 4, 4, 1, 0, 0, 63, true, true, SUMS)}
+static const PairVariant kHL[3][2] = {NB_HL_PAIR(kSumAll), NB_HL_PAIR(kSumA), NB_HL_PAIR(kSumP)};
+// Twins of the built-in packed plain-mode shapes with a_i only (the integrator's
+// force from packed FP64 state, and nb_force with p NULL), and of a large-N shape
+// the tuner may pick; and with the potential only (the energy).
+static const PairVariant kOnlyA[] = {
+    NB_VARIANT_OF(256, 2, 128, 4, 4, 1, 0, 0, 63, false, false, kSumA),
+    NB_VARIANT_OF(64, 4, 128, 4, 4, 1, 0, 0, 63, false, false, kSumA),
+    NB_VARIANT_OF(256, 4, 256, 3, 4, 1, 0, 0, 63, false, false, kSumA),
+    NB_VARIANT_OF(128, 12, 256, 3, 4, 1, 0, 1, 63, false, false, kSumA),
+    NB_VARIANT_OF(256, 4, 1024, 3, 4, 1, 0, 0, 63, true, false, kSumA),
+    NB_VARIANT_OF(256, 4, 512, 3, 4, 1, 0, 0, 63, false, false, kSumA),
 };
-// No-potential twins of the built-in packed plain-mode shapes (the
-// integrator's force from packed FP64 state, and nb_force with p NULL), and
-// of a large-N shape the tuner may pick.
-static const PairVariant kNoPot[] = {
-    NB_VARIANT_NP(256, 2, 128, 4, 4, 1, 0, 0, 63, false, false, true),
-    NB_VARIANT_NP(64, 4, 128, 4, 4, 1, 0, 0, 63, false, false, true),
-    NB_VARIANT_NP(256, 4, 256, 3, 4, 1, 0, 0, 63, false, false, true),
-    NB_VARIANT_NP(128, 12, 256, 3, 4, 1, 0, 1, 63, false, false, true),
-    NB_VARIANT_NP(256, 4, 1024, 3, 4, 1, 0, 0, 63, true, false, true),
-    NB_VARIANT_NP(256, 4, 512, 3, 4, 1, 0, 0, 63, false, false, true),
+static const PairVariant kOnlyP[] = {
+    NB_VARIANT_OF(256, 2, 128, 4, 4, 1, 0, 0, 63, false, false, kSumP),
+    NB_VARIANT_OF(64, 4, 128, 4, 4, 1, 0, 0, 63, false, false, kSumP),
+    NB_VARIANT_OF(256, 4, 512, 3, 4, 1, 0, 0, 63, false, false, kSumP),
+    NB_VARIANT_OF(256, 4, 1024, 3, 4, 1, 0, 0, 63, true, false, kSumP),
 };
-static_assert(kDefaultRefine == 0, "the no-potential and HL shapes have no Newton step");
+static_assert(kDefaultRefine == 0, "the shapes with some of the sums and the HL shapes have no Newton step");
 #undef NB_VARIANT
-#undef NB_VARIANT_NP
+#undef NB_VARIANT_OF
+#undef NB_HL_PAIR
 #undef NB_FUSED
 #undef NB_FUSED_SK
 #undef NB_FUSED_CL
@@ -1253,9 +1262,7 @@ static_assert(kDefaultRefine == 0, "the no-potential and HL shapes have no Newto
 
 static int pair_variant_index(bool comp, const nb_tile &t);
 
-const PairVariant *hl_variant(int64_t n, bool no_pot) {
-    return &kHL[no_pot ? 1 : 0][n >= (int64_t)1 << 15 ? 0 : 1];
-}
+const PairVariant *hl_variant(int64_t n, PairSums sums) { return &kHL[sums][n >= (int64_t)1 << 15 ? 0 : 1]; }
 
 const PairVariant *chunked_twin(const PairVariant &v) {
     nb_tile t = v.tile;
@@ -1264,11 +1271,15 @@ const PairVariant *chunked_twin(const PairVariant &v) {
     return k >= 0 ? pair_variant(v.comp, k) : nullptr;
 }
 
-const PairVariant *no_pot_twin(const PairVariant &v) {
-    if (v.tile.fused) return nullptr;
-    for (const PairVariant &w : kNoPot)
-        if (w.comp == v.comp && same_tile(w.tile, v.tile)) return &w;
+template <size_t N>
+static const PairVariant *twin_in(const PairVariant (&list)[N], const PairVariant &v) {
+    for (const PairVariant &w : list)
+        if (!v.tile.fused && w.comp == v.comp && same_tile(w.tile, v.tile)) return &w;
     return nullptr;
+}
+
+const PairVariant *sums_twin(const PairVariant &v, PairSums sums) {
+    return sums == kSumAll ? nullptr : sums == kSumA ? twin_in(kOnlyA, v) : twin_in(kOnlyP, v);
 }
 
 int pair_variant_count(bool comp) {

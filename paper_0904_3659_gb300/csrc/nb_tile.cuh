@@ -27,7 +27,8 @@ using namespace nbdev;
 // results). Mixing trades issue slots (packed: one per two lanes) against
 // the lower sustained pipe rate of packed instructions.
 // POT = false leaves the potential out (acc[q][3] untouched): 12 FP32
-// operations per pair, for callers that need only a_i (the integrator).
+// operations per pair, for callers that need only a_i (the integrator). ACC =
+// false leaves the accelerations out: 8 operations, for the energy.
 enum : int { kMixD = 1, kMixS = 2, kMixN = 4, kMixQ = 8, kMixW = 16, kMixA = 32, kMixAll = 63 };
 
 template <bool PK>
@@ -49,7 +50,7 @@ __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) {
 // slot DK of the thread meets itself, at jj == self0[0] (the lane), and the
 // mask costs one compare and one select per j instead of two of each per
 // pair.
-template <int P, int JT, int UNR, bool DIAG, int MIX, bool NEWTON, bool POT = true, int DK = -1>
+template <int P, int JT, int UNR, bool DIAG, int MIX, bool NEWTON, bool POT = true, int DK = -1, bool ACC = true>
 __device__ __forceinline__ void tile_pass(const JPart *__restrict__ T, const float2 (&xi)[P],
                                           const float2 (&yi)[P], const float2 (&zi)[P],
                                           float2 (&acc)[P][4], const float2 eps2,
@@ -91,8 +92,10 @@ __device__ __forceinline__ void tile_pass(const JPart *__restrict__ T, const flo
                 if (jj == self0[q]) hm.x = 0.f;
                 if (jj == self1[q]) hm.y = 0.f;
             }
-            const float2 qv = vmul<PQ>(hm, u);
+            // (packed, a product used once would be fused into the sum: other bits)
+            const float2 qv = vmul<PQ && ACC>(hm, u);
             if (POT) acc[q][3] = vadd<PQ>(acc[q][3], qv);
+            if (!ACC) continue;
             const float2 u2 = vmul<PW>(u, u);
             const float2 w = vmul<PW>(qv, u2);
             acc[q][0] = vfma<PA>(w, dx, acc[q][0]);
@@ -131,9 +134,10 @@ __device__ __forceinline__ void tile_pass_diag32(int k, int lane, const JPart *_
 // component of x_i - x_j is then (h_i - h_j) + (l_i - l_j): one rounding of
 // the exact difference (up to the remainders' own rounding, far below it),
 // so close pairs keep their relative accuracy wherever they sit. 6 FP32
-// operations per pair more than tile_pass (19, or 18 without the potential).
+// operations per pair more than tile_pass (19, or 18 without the potential, 14
+// without the accelerations).
 // DK >= 0: the lane-diagonal form, as for tile_pass.
-template <int P, int JT, int UNR, bool DIAG, bool POT, int DK = -1>
+template <int P, int JT, int UNR, bool DIAG, bool POT, int DK = -1, bool ACC = true>
 __device__ __forceinline__ void tile_pass_hl(const JPart *__restrict__ T, const float2 (&xi)[P],
                                              const float2 (&yi)[P], const float2 (&zi)[P],
                                              const float2 (&lxi)[P], const float2 (&lyi)[P],
@@ -170,8 +174,9 @@ __device__ __forceinline__ void tile_pass_hl(const JPart *__restrict__ T, const 
                 if (jj == self0[q]) hm.x = 0.f;
                 if (jj == self1[q]) hm.y = 0.f;
             }
-            const float2 qv = mul2(hm, u);
+            const float2 qv = vmul<ACC>(hm, u);  // (as in tile_pass)
             if (POT) acc[q][3] = add2(acc[q][3], qv);
+            if (!ACC) continue;
             const float2 w = mul2(qv, mul2(u, u));
             acc[q][0] = fma2(w, dx, acc[q][0]);
             acc[q][1] = fma2(w, dy, acc[q][1]);
