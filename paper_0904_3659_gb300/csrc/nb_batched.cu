@@ -666,19 +666,13 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
             comp_add(S, E, h);
         }
     }
-    float v[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) v[r] = -2.f * __fadd_rn(S[r], E[r]);
     const float hm0 = A.cp[row0 * RS].w;
     const int weights = cluster_weights(A, c, nt);
-    if (weights == kEqual) {
+    const float hm = A.cp[((int64_t)blockIdx.x * kBlock + threadIdx.x) * RS].w;
+    const float f = weights == kProduct ? mutual_scale(hm, hm0, A.eps[c]) : hm0;
+    float v[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] *= hm0;
-    } else if (weights == kProduct) {
-        const float d = mutual_scale(A.cp[((int64_t)blockIdx.x * kBlock + threadIdx.x) * RS].w, hm0, A.eps[c]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = __fdiv_rn(v[r], d);
-    }
+    for (int r = 0; r < 4; ++r) v[r] = mutual_result(weights, S[r], E[r], f);
     const int64_t i = o + li;
     if (!NB_IN(A.err, 68, i >= 0 && i < A.n_total)) return;
     a[3 * i + 0] = v[0];

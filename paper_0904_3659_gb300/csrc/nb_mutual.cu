@@ -359,17 +359,10 @@ __global__ void __launch_bounds__(32 * kCombineWarps) mutual_combine_kernel(cons
     // holds -m/2), 1 / (c m_i) (kProduct), -2 (kWide).
     const int weights = *A.weights;
     const int rs = O.hl ? kHLRecords : 1;
+    const float hm0 = A.cp[0].w, f = weights == kProduct ? mutual_scale(A.cp[i * rs].w, hm0, A.eps) : hm0;
     float v[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) v[r] = -2.f * __fadd_rn(S[r], E[r]);
-    if (weights == kEqual) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] *= A.cp[0].w;
-    } else if (weights == kProduct) {
-        const float c = mutual_scale(A.cp[i * rs].w, A.cp[0].w, A.eps);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = __fdiv_rn(v[r], c);
-    }
+    for (int r = 0; r < 4; ++r) v[r] = mutual_result(weights, S[r], E[r], f);
     if (O.a) {
         O.a[3 * i + 0] = v[0];
         O.a[3 * i + 1] = v[1];
