@@ -73,12 +73,13 @@ __global__ void kick_drift_pack_kernel(double *__restrict__ x, double *__restric
 
 // The same for the mutual kernels' records (nb_mutual.cuh): one thread per
 // padded particle, in blocks of nbx::kMutualPackThreads. KICK: the kicks and the
-// drift first (kick_back as above), else the positions as they are.
+// drift first (kick_back as above; xh, if given, records the moved positions), else
+// the positions as they are.
 template <bool KICK>
 __global__ void mutual_pack_f64_kernel(double *__restrict__ x, double *__restrict__ v,
                                        const float *__restrict__ a, const float *__restrict__ m, int64_t n,
                                        int64_t npad, double dt, int kick_back, float eps, MPart *__restrict__ cp,
-                                       int *__restrict__ notes) {
+                                       int *__restrict__ notes, double *__restrict__ xh) {
     pdl_wait_then_release();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     MPart r = mutual_padding();
@@ -96,6 +97,7 @@ __global__ void mutual_pack_f64_kernel(double *__restrict__ x, double *__restric
                 xc = xc + dt * vc;               // Eq. (2)
                 v[3 * i + c] = vc;
                 x[3 * i + c] = xc;
+                if (xh) xh[3 * i + c] = xc;
             }
             q[c] = (float)xc;
         }
@@ -103,6 +105,29 @@ __global__ void mutual_pack_f64_kernel(double *__restrict__ x, double *__restric
     }
     mutual_note(i < n, r, -0.5f * m[0], eps, notes);
     if (i < npad) cp[i] = r;
+}
+
+// The same for the single-launch kernels, which read FP32 positions: one thread per
+// component.
+template <bool KICK>
+__global__ void round_f64_kernel(double *__restrict__ x, double *__restrict__ v, const float *__restrict__ a,
+                                 int64_t n, double dt, int kick_back, float *__restrict__ x32,
+                                 double *__restrict__ xh) {
+    pdl_wait_then_release();
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= 3 * n) return;
+    double xc = x[k];
+    if (KICK) {
+        const double h = 0.5 * dt, g = -(double)a[k];
+        double vc = v[k];
+        if (kick_back) vc = vc + h * g;  // Eq. (3) of the previous step
+        vc = vc + h * g;                 // Eq. (1)
+        xc = xc + dt * vc;               // Eq. (2)
+        v[k] = vc;
+        x[k] = xc;
+        if (xh) xh[k] = xc;
+    }
+    x32[k] = (float)xc;
 }
 
 // Order-preserving map of an FP64 value's bits to a signed 64-bit integer (its
@@ -116,11 +141,12 @@ constexpr int kBoxBlocks = 512;  // most partial boxes
 
 // Compensated mode on the mutual kernels: kicks and drift (if kick; kick_back as
 // above), and one partial bounding box of the moved positions per block (lo x,
-// y, z, hi x, y, z as keys).
+// y, z, hi x, y, z as keys). xh as above.
 __global__ void __launch_bounds__(256) kick_drift_box_kernel(double *__restrict__ x, double *__restrict__ v,
                                                              const float *__restrict__ a, int64_t n, double dt,
                                                              int kick, int kick_back,
-                                                             long long *__restrict__ box) {
+                                                             long long *__restrict__ box,
+                                                             double *__restrict__ xh) {
     __shared__ long long s[8][6];
     pdl_wait_then_release();
     const double h = 0.5 * dt;
@@ -137,6 +163,7 @@ __global__ void __launch_bounds__(256) kick_drift_box_kernel(double *__restrict_
                 xc = xc + dt * vc;               // Eq. (2)
                 v[3 * i + c] = vc;
                 x[3 * i + c] = xc;
+                if (xh) xh[3 * i + c] = xc;
             }
             const long long k = box_key(__double_as_longlong(xc));
             lo[c] = min(lo[c], k);
@@ -178,6 +205,7 @@ __global__ void kick_drift_kernel(double *__restrict__ x, double *__restrict__ v
 
 __global__ void kick_kernel(double *__restrict__ v, const float *__restrict__ a, int64_t n,
                             double dt) {
+    pdl_wait_then_release();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= 3 * n) return;
     v[k] = v[k] + (0.5 * dt) * (-(double)a[k]);  // Eq. (3)
@@ -458,6 +486,7 @@ unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1
 // the direct kernels (`mutual` NULL). Decided once per call.
 struct Evaluator {
     const MutualShape *mutual = nullptr;
+    bool single = false;  // plain mode: nb_force's single-launch shape on rounded positions
     bool comp = false;
     bool only_p = false;  // direct kernels: a is zeroed, not summed
 };
@@ -467,6 +496,8 @@ struct Evaluator {
 nb_status choose_evaluator(nb_ctx *ctx, int64_t n, bool comp, bool pot, Evaluator *ev) {
     ev->comp = comp;
     ev->mutual = nullptr;
+    if ((ev->single = !comp && single_from_fp64(n) && choose_variant(ctx, n, false).tile.fused))
+        return ensure_slot(ctx, S_P, (size_t)n * sizeof(float));  // (for a NULL p: these shapes sum it)
     const int size = mutual_from_fp64(ctx, n, comp);
     if (size < 0) return NB_OK;
     const MutualShape &s = mutual_shape(size, pot, comp);
@@ -499,11 +530,12 @@ nb_status reserve_hl_state(nb_ctx *ctx, int64_t n) {
 
 // The same through the mutual kernels, after kicks and drift (if kick).
 nb_status step_hl_mutual(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
-                         int64_t n, float eps, double dt, int kick, int kick_back, cudaStream_t st) {
+                         int64_t n, float eps, double dt, int kick, int kick_back, cudaStream_t st,
+                         double *xh = nullptr) {
     long long *box = static_cast<long long *>(slot(ctx, S_BOX));
     const int nbox = (int)std::min<int64_t>(kBoxBlocks, (n + 255) / 256);
     cudaError_t e = launch_with_pdl(kick_drift_box_kernel, dim3((unsigned)nbox), dim3(256), 0, st, x, v,
-                                    (const float *)a, n, dt, kick, kick_back, box);
+                                    (const float *)a, n, dt, kick, kick_back, box, xh);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
     const int64_t npad = mutual_npad(*ev.mutual, n);
     e = launch_with_pdl(mutual_hl_pack_kernel, dim3((unsigned)mutual_pack_blocks(npad)), dim3(kMutualPackThreads), 0,
@@ -530,6 +562,20 @@ nb_status force_hl(nb_ctx *ctx, const Evaluator &ev, const double *x, const floa
     return run_force_hl(ctx, jp, n, eps, a, p, st, ev.only_p);
 }
 
+// Plain mode through nb_force's single-launch shapes, after kicks and drift (KICK):
+// two launches a step against three, and no partial sums through global memory (us
+// per step, against the mutual kernels: N = 1000 6.5 / 13.6, 4096 13.7 / 22.3, 9728
+// 44.9 / 48.0; unequal masses 44.8 / 52.6).
+template <bool KICK>
+nb_status force_single(nb_ctx *ctx, double *x, double *v, const float *m, float *a, float *p, int64_t n, float eps,
+                       double dt, int kick_back, cudaStream_t st, double *xh) {
+    float *x32 = static_cast<float *>(slot(ctx, S_JP));
+    const cudaError_t e = launch_with_pdl(round_f64_kernel<KICK>, dim3(blocks_for(3 * n, 128)), dim3(128), 0, st, x, v,
+                                          (const float *)a, n, dt, kick_back, x32, xh);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+    return run_force(ctx, x32, m, nullptr, n, eps, a, p ? p : static_cast<float *>(slot(ctx, S_P)), false, st);
+}
+
 // Plain mode: Eq. (gravity) at the FP64 positions as they are.
 nb_status force_plain(nb_ctx *ctx, const Evaluator &ev, double *x, const float *m, int64_t n, float eps, float *a,
                       float *p, cudaStream_t st) {
@@ -539,46 +585,48 @@ nb_status force_plain(nb_ctx *ctx, const Evaluator &ev, double *x, const float *
         const int64_t npad = mutual_npad(*ev.mutual, n);
         e = launch_with_pdl(mutual_pack_f64_kernel<false>, dim3((unsigned)mutual_pack_blocks(npad)),
                             dim3(kMutualPackThreads), 0, st, x, (double *)nullptr, (const float *)nullptr, m, n, npad,
-                            0.0, 0, eps, mutual_records(ctx), mutual_notes(ctx));
+                            0.0, 0, eps, mutual_records(ctx), mutual_notes(ctx), (double *)nullptr);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
         return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
     }
+    if (ev.single) return force_single<false>(ctx, x, nullptr, m, a, p, n, eps, 0.0, 0, st, nullptr);
     pack_f64_kernel<<<blocks_for(padded(n), 256), 256, 0, st>>>(x, m, n, padded(n), jp);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
     return run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, st, ev.only_p);
 }
 
+// Copy the positions to xh (if given).
+nb_status record(nb_ctx *ctx, double *xh, const double *x, int64_t n, cudaStream_t s) {
+    if (!xh) return NB_OK;
+    const cudaError_t e = cudaMemcpyAsync(xh, x, (size_t)3 * n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    return e == cudaSuccess ? NB_OK : cuda_fail(ctx, e, "position history copy");
+}
+
 // Plain mode, one step but its last kick: fused kicks, drift and packing, then
 // the force.
 nb_status step_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
-                     int64_t n, float eps, double dt, int kick_back, cudaStream_t st) {
+                     int64_t n, float eps, double dt, int kick_back, cudaStream_t st, double *xh) {
     JPart *jp = static_cast<JPart *>(slot(ctx, S_JP));
     cudaError_t e;
+    if (ev.single) return force_single<true>(ctx, x, v, m, a, p, n, eps, dt, kick_back, st, xh);
     if (ev.mutual) {
         const int64_t npad = mutual_npad(*ev.mutual, n);
         e = launch_with_pdl(mutual_pack_f64_kernel<true>, dim3((unsigned)mutual_pack_blocks(npad)),
                             dim3(kMutualPackThreads), 0, st, x, v, (const float *)a, m, n, npad, dt, kick_back, eps,
-                            mutual_records(ctx), mutual_notes(ctx));
+                            mutual_records(ctx), mutual_notes(ctx), xh);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
         return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
     }
     kick_drift_pack_kernel<<<blocks_for(padded(n), 256), 256, 0, st>>>(x, v, a, m, n, padded(n), dt, kick_back, jp);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+    if (nb_status rs; (rs = record(ctx, xh, x, n, st)) != NB_OK) return rs;
     return run_force(ctx, nullptr, nullptr, jp, n, eps, a, p, false, st);
-}
-
-// With x_hist set, copy the positions after step t (t = 0 for the entry
-// positions) into x_hist[t] ([nsteps + 1][n][3] FP64): the adjoint's replay.
-nb_status record(nb_ctx *ctx, double *x_hist, int t, const double *x, int64_t n, cudaStream_t s) {
-    if (!x_hist) return NB_OK;
-    const cudaError_t e = cudaMemcpyAsync(x_hist + (size_t)t * 3 * n, x, (size_t)3 * n * sizeof(double),
-                                          cudaMemcpyDeviceToDevice, s);
-    return e == cudaSuccess ? NB_OK : cuda_fail(ctx, e, "position history copy");
 }
 
 // The compensated leap-frog: every force evaluation packs the FP64 positions
 // as HL records (force_hl). Steps after the first are replayed from a graph,
-// unless the positions of every step are recorded (x_hist).
+// unless the positions of every step are recorded (x_hist, [nsteps + 1][n][3] FP64,
+// the entry positions first: the adjoint's replay).
 nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
                       int64_t n, float eps, double dt, int nsteps, int a_valid, cudaStream_t s,
                       double *x_hist) {
@@ -586,17 +634,19 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
     if (st != NB_OK) return st;
     cudaError_t e;
     if (!a_valid && (st = force_hl(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
-    if ((st = record(ctx, x_hist, 0, x, n, s)) != NB_OK) return st;
+    if ((st = record(ctx, x_hist, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
     const unsigned nb3 = blocks_for(3 * n, 256);
-    auto step = [&](int kick_back) -> nb_status {
-        if (ev.mutual) return step_hl_mutual(ctx, ev, x, v, m, a, p, n, eps, dt, 1, kick_back, s);
+    auto step = [&](int kick_back, int t = 0) -> nb_status {
+        double *const xh = x_hist ? x_hist + (size_t)t * 3 * n : nullptr;
+        if (ev.mutual) return step_hl_mutual(ctx, ev, x, v, m, a, p, n, eps, dt, 1, kick_back, s, xh);
         kick_drift_kernel<<<nb3, 256, 0, s>>>(x, v, a, n, dt, kick_back);
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return cuda_fail(ctx, le, "leap-frog update launch");
+        if (nb_status rs; (rs = record(ctx, xh, x, n, s)) != NB_OK) return rs;
         return force_hl(ctx, ev, x, m, n, eps, a, p, s);
     };
-    if ((st = step(0)) != NB_OK || (st = record(ctx, x_hist, 1, x, n, s)) != NB_OK) return st;
+    if ((st = step(0, 1)) != NB_OK) return st;
     const int rest = nsteps - 1;
     if (rest >= 2 && s != nullptr && !x_hist) {
         cudaGraph_t graph = nullptr;
@@ -620,11 +670,10 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     } else {
         for (int k = 0; k < rest; ++k)
-            if ((st = step(1)) != NB_OK || (st = record(ctx, x_hist, k + 2, x, n, s)) != NB_OK)
-                return st;
+            if ((st = step(1, k + 2)) != NB_OK) return st;
     }
-    kick_kernel<<<nb3, 256, 0, s>>>(v, a, n, dt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
+    e = launch_with_pdl(kick_kernel, dim3(nb3), dim3(256), 0, s, v, (const float *)a, n, dt);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
     return NB_OK;
 }
 
@@ -637,12 +686,15 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
     cudaError_t e;
     nb_status st;
     if (!a_valid && (st = force_plain(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
-    if ((st = record(ctx, x_hist, 0, x, n, s)) != NB_OK) return st;
+    if ((st = record(ctx, x_hist, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
+    auto step = [&](int kick_back, int t) {
+        return step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, kick_back, s,
+                          x_hist ? x_hist + (size_t)t * 3 * n : nullptr);
+    };
 
     // Step 0: front kick + drift + pack, force.
-    if ((st = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 0, s)) != NB_OK) return st;
-    if ((st = record(ctx, x_hist, 1, x, n, s)) != NB_OK) return st;
+    if ((st = step(0, 1)) != NB_OK) return st;
 
     // Steps 1 .. nsteps-1: the same kernels with the same arguments each
     // step, so they are captured once into a graph and replayed (not on the
@@ -654,7 +706,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
         e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture begin");
         const bool timing = ctx_set_timing(ctx, false);  // no event nodes in the graph
-        nb_status cst = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 1, s);
+        nb_status cst = step(1, 0);
         ctx_set_timing(ctx, timing);
         e = cudaStreamEndCapture(s, &graph);
         if (cst != NB_OK) {
@@ -670,13 +722,11 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     } else {
         for (int k = 0; k < rest; ++k)
-            if ((st = step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, 1, s)) != NB_OK ||
-                (st = record(ctx, x_hist, k + 2, x, n, s)) != NB_OK)
-                return st;
+            if ((st = step(1, k + 2)) != NB_OK) return st;
     }
     // Final back kick, Eq. (3).
-    kick_kernel<<<blocks_for(3 * n, 256), 256, 0, s>>>(v, a, n, dt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
+    e = launch_with_pdl(kick_kernel, dim3(blocks_for(3 * n, 256)), dim3(256), 0, s, v, (const float *)a, n, dt);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
     return NB_OK;
 }
 

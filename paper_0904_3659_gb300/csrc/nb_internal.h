@@ -208,6 +208,8 @@ int pair_default_unfused_index(bool comp, int64_t n);
 int pair_mutual_index(bool comp, int64_t n);
 // The mutual shape for n FP64 positions (leap-frog, energy), or -1.
 int mutual_size_from_fp64(int64_t n);
+// Whether a single-launch shape serves FP64 state rounded to FP32 (plain mode).
+bool single_from_fp64(int64_t n);
 // Whether the tuner times the fused (single-launch, small-n) shapes at n.
 bool fused_candidate(int64_t n);
 

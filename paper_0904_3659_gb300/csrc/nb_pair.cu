@@ -1386,13 +1386,16 @@ int pair_mutual_index(bool comp, int64_t n) {
     return -1;
 }
 
-// From FP64 positions the mutual shapes are the fastest at every size (leap-frog
-// without the potential, equal masses, us per step against the direct kernels:
-// n = 256 16.8 / 22.3, 4096 26 / 31.5, 20011 141 / 191; compensated: 24 / 43.5,
-// 34 / 56, 190 / 290).
+// From FP64 positions the mutual shapes are faster than the packed direct ones at
+// every size (leap-frog without the potential, equal masses, us per step: n = 256
+// 13.0 / 22.3, 4096 22.3 / 31.5, 20011 141 / 191; compensated: 18.6 / 43.5, 29.6 / 56,
+// 190 / 290). In plain mode the single-launch cluster shapes, on positions rounded to
+// FP32, are faster yet as far as they are nb_force's choice (9728: 44.9 / 48.0).
 int mutual_size_from_fp64(int64_t n) {
     return n < kMutualMidN ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
 }
+
+bool single_from_fp64(int64_t n) { return n <= kClusterMaxN; }
 
 PairPlan make_plan(const PairVariant &v, int64_t n, int resident_ctas) {
     PairPlan p{};

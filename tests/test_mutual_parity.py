@@ -307,3 +307,40 @@ def test_batched_small_batch_after_a_large_one(nb, ctx):
     for sizes in (BATCHES["many"], [5, 200, 78], [200, 5, 77], [5, 200, 77]):
         got = run_batch(nb, ctx, batch(sizes), 0)
     assert got[0].tobytes() == want[0].tobytes() and got[1].tobytes() == want[1].tobytes()
+
+
+@pytest.mark.parametrize("with_p", [False, True])
+@pytest.mark.parametrize("n", [1, 33, 1000, 9728, 9729])
+def test_plain_leapfrog_at_the_edge_of_the_single_launch_shapes(nb, ctx, n, with_p):
+    # Three steps against the same steps with nb_force at the rounded positions: the
+    # accelerations differ by at most 2e-5 of their scale (1e-5 each), so v by dt 3
+    # times that and x by 3 dt times as much again; once up to 9728 (one kernel) by
+    # the FP64 rounding alone. On a stream too, where the steps are replayed.
+    import torch
+    x32, m32, eps = particles(n, "spectrum")
+    m = torch.from_numpy(m32).cuda()
+    dt = 1.0 / 64
+    x = torch.from_numpy(x32.astype(np.float64)).cuda() * (1 + 1e-9)
+    v = torch.zeros_like(x)
+    a, p = torch.empty((n, 3), device="cuda"), torch.empty(n, device="cuda")
+
+    def force(x):
+        nb.nb_force(ctx, x.float(), m, n, eps, a, p, 0)
+        return a.double()
+
+    wx, wv, g = x.clone(), v.clone(), force(x)
+    for _ in range(3):
+        wv -= 0.5 * dt * g
+        wx += dt * wv
+        g = force(wx)
+        wv -= 0.5 * dt * g
+    scale = float(g.abs().max())
+    rel = 1e-14 if n <= 9728 else 2e-5
+    nb.nb_synchronize(ctx)
+    for stream in (None, torch.cuda.Stream()):
+        gx, gv = x.clone(), v.clone()
+        torch.cuda.synchronize()
+        nb.nb_leapfrog_step(ctx, gx, gv, m, a, p if with_p else None, n, eps, dt, 3, 0, 0, stream)
+        nb.nb_synchronize(ctx, stream)
+        assert float((gv - wv).abs().max()) <= 3 * dt * rel * scale + 1e-15
+        assert float((gx - wx).abs().max()) <= 9 * dt * dt * rel * scale + 1e-14
