@@ -111,11 +111,24 @@ int *mutual_notes(nb_ctx *ctx);
 nb_status run_mutual(nb_ctx *ctx, const nbk::MutualShape &s, const float *x, const float *m, int64_t n, float eps,
                      float *a, float *p, cudaStream_t st);
 
-// nb_force_vjp on the mutual kernels (nb_vjp_mutual.cu); gp may be NULL.
-// NB_ERR_OOM when the scratch cannot be allocated (nothing is enqueued then).
+// A step of the leap-frog's adjoint around its VJP of Eq. (gravity), all FP64: the
+// operands are x and la with the back kick's share -dt/2 lv (first: the force at the
+// start of a trajectory, la alone), and the result enters lx and lm, then the drift
+// and the front kick lv and la (first: la is cleared).
+struct VjpState {
+    const double *x;
+    double *lx, *lv, *la, *lm;
+    double dt;
+    int first;
+};
 
+// nb_force_vjp on the mutual kernels (nb_vjp_mutual.cu); gp may be NULL. With a
+// state: from and to its arrays, not x, ga, gp, gx, gm. NB_ERR_OOM when the scratch
+// cannot be allocated (nothing is enqueued then).
 nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, int64_t n, float eps, const float *ga,
-                         const float *gp, float *gx, float *gm, cudaStream_t st);
+                         const float *gp, float *gx, float *gm, cudaStream_t st, const VjpState *state = nullptr);
+// The size argument for n without an upstream gradient on p, -1 for a direct shape.
+int vjp_mutual_size(nb_ctx *ctx, int64_t n);
 
 struct DeviceGuard {
     int prev = -1;

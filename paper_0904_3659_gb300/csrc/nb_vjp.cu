@@ -538,6 +538,8 @@ const VjpVariant &vjp_variant(nb_ctx *ctx, int64_t n, bool with_gp) {
 
 }  // namespace
 
+int nbx::vjp_mutual_size(nb_ctx *ctx, int64_t n) { return vjp_variant(ctx, n, false).mutual; }
+
 extern "C" nb_status nb_force_vjp(nb_ctx *ctx, const float *x, const float *m, int64_t n, float eps,
                                   const float *ga, const float *gp, float *gx, float *gm,
                                   void *stream) {

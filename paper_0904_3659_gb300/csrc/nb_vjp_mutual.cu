@@ -43,6 +43,28 @@ __global__ void vjp_mutual_pack_kernel(const float *__restrict__ x, const float 
     cp[kVmRecords * i + 1] = v;
 }
 
+// The same from the leap-frog adjoint's state.
+__global__ void vjp_mutual_pack_state_kernel(const nbx::VjpState s, const float *__restrict__ m, int64_t n,
+                                             int64_t npad, float4 *__restrict__ cp) {
+    pdl_wait_then_release();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= npad) return;
+    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+    if (i < n) {
+        float x[3], g[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double l = s.la[3 * i + c];
+            x[c] = (float)s.x[3 * i + c];
+            g[c] = (float)(s.first ? l : l + (-((0.5 * s.dt) * s.lv[3 * i + c])));
+        }
+        u = make_float4(-x[0], -x[1], -x[2], m[i]);
+        v = make_float4(g[0], g[1], g[2], 0.f);
+    }
+    cp[kVmRecords * i] = u;
+    cp[kVmRecords * i + 1] = v;
+}
+
 struct VmArgs {
     const float4 *cp;      // [npad][2]
     float4 *pi;            // [grid + rows][4][ib]: sums (R, S), (V, G), their carries
@@ -59,6 +81,7 @@ struct VmArgs {
 
 struct VmOut {
     float *gx, *gm;
+    nbx::VjpState adj;     // (adj.lx: the results go there)
     float4 *state;         // [n][4] sums and carries between panels
     int64_t n;
     int ib, jt, last;
@@ -429,10 +452,26 @@ __global__ void __launch_bounds__(32 * kVmCombineWarps) vjp_mutual_combine_kerne
     const float4 u = A.cp[kVmRecords * i], g = A.cp[kVmRecords * i + 1];
     const float Sm = __fadd_rn(S[3], E[3]), gv[3] = {g.x, g.y, g.z};
 #pragma unroll
-    for (int c = 0; c < 3; ++c)  // gx = R + ga S - m V
-        O.gx[3 * i + c] = __fadd_rn(__fadd_rn(S[c], E[c]),
-                                    __fmaf_rn(-u.w, __fadd_rn(S[4 + c], E[4 + c]), __fmul_rn(gv[c], Sm)));
-    O.gm[i] = __fadd_rn(S[7], E[7]);
+    for (int c = 0; c < 3; ++c) {  // gx = R + ga S - m V
+        const float gx = __fadd_rn(__fadd_rn(S[c], E[c]),
+                                   __fmaf_rn(-u.w, __fadd_rn(S[4 + c], E[4 + c]), __fmul_rn(gv[c], Sm)));
+        if (!O.adj.lx) {
+            O.gx[3 * i + c] = gx;
+            continue;
+        }
+        const double x = O.adj.lx[3 * i + c] + (double)gx;
+        O.adj.lx[3 * i + c] = x;
+        double a = 0.0;
+        if (!O.adj.first) {
+            const double v = O.adj.lv[3 * i + c] + O.adj.dt * x;
+            O.adj.lv[3 * i + c] = v;
+            a = -((0.5 * O.adj.dt) * v);
+        }
+        O.adj.la[3 * i + c] = a;
+    }
+    const float gm = __fadd_rn(S[7], E[7]);
+    if (O.adj.lx) O.adj.lm[i] = O.adj.lm[i] + (double)gm;
+    else O.gm[i] = gm;
 }
 
 template <int WARPS, int P, int JT, int STAGES>
@@ -476,7 +515,7 @@ using namespace nbk;
 namespace nbx {
 
 nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, int64_t n, float eps, const float *ga,
-                         const float *gp, float *gx, float *gm, cudaStream_t st) {
+                         const float *gp, float *gx, float *gm, cudaStream_t st, const VjpState *state) {
     const VmShape &s = kVmShapes[size][gp ? 1 : 0];
     PairVariant v{};
     v.tile.threads = s.threads;
@@ -525,10 +564,12 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     A.npad = npad;
     A.pi_len = (int64_t)(es.cap[SLOT_MUTUAL_PI] / sizeof(float4));
     A.pj_len = (int64_t)(es.cap[SLOT_MUTUAL_PJ] / sizeof(float4));
-    VmOut O{gx, gm, static_cast<float4 *>(es.buf[SLOT_MUTUAL_STATE]), n, s.ib, s.jt, 0};
+    VmOut O{gx,   gm,   state ? *state : VjpState{}, static_cast<float4 *>(es.buf[SLOT_MUTUAL_STATE]), n, s.ib,
+            s.jt, 0};
 
-    e = launch_with_pdl(vjp_mutual_pack_kernel, dim3((unsigned)((npad + 127) / 128)), dim3(128), 0, st, x, m, ga, gp,
-                        n, npad, cp);
+    const dim3 pack((unsigned)((npad + 127) / 128));
+    e = state ? launch_with_pdl(vjp_mutual_pack_state_kernel, pack, dim3(128), 0, st, *state, m, n, npad, cp)
+              : launch_with_pdl(vjp_mutual_pack_kernel, pack, dim3(128), 0, st, x, m, ga, gp, n, npad, cp);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "vjp pack launch");
     for (int64_t r0 = 0; r0 < T.nib;) {
         const int64_t r1 = T.panel_end(r0, most);
