@@ -247,6 +247,18 @@ __global__ void adj_drift_kick_kernel(double *__restrict__ lx, double *__restric
     if (k < n) lm[k] = lm[k] + (double)gm[k];
 }
 
+// The copies that a segment's replay works on, and the first recorded positions.
+__global__ void adj_copy_kernel(const double *__restrict__ x, const double *__restrict__ v,
+                                const float *__restrict__ a, int64_t n3, double *__restrict__ xw,
+                                double *__restrict__ vw, float *__restrict__ aw, double *__restrict__ hist) {
+    pdl_wait_then_release();
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= n3) return;
+    xw[k] = hist[k] = x[k];
+    vw[k] = v[k];
+    if (a) aw[k] = a[k];
+}
+
 // The force at the start of a trajectory, a_0 = F(x_0): VJP operands from
 // the adjoint of a_0, then its result folded into lx, lm (la cleared).
 __global__ void adj_first_operands_kernel(const double *__restrict__ la,
@@ -625,8 +637,8 @@ nb_status step_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, con
 
 // The compensated leap-frog: every force evaluation packs the FP64 positions
 // as HL records (force_hl). Steps after the first are replayed from a graph,
-// unless the positions of every step are recorded (x_hist, [nsteps + 1][n][3] FP64,
-// the entry positions first: the adjoint's replay).
+// unless the positions after every step are recorded (x_hist, [nsteps][n][3] FP64:
+// the adjoint's replay).
 nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, const float *m, float *a, float *p,
                       int64_t n, float eps, double dt, int nsteps, int a_valid, cudaStream_t s,
                       double *x_hist) {
@@ -634,10 +646,9 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
     if (st != NB_OK) return st;
     cudaError_t e;
     if (!a_valid && (st = force_hl(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
-    if ((st = record(ctx, x_hist, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
     const unsigned nb3 = blocks_for(3 * n, 256);
-    auto step = [&](int kick_back, int t = 0) -> nb_status {
+    auto step = [&](int kick_back, int t) -> nb_status {
         double *const xh = x_hist ? x_hist + (size_t)t * 3 * n : nullptr;
         if (ev.mutual) return step_hl_mutual(ctx, ev, x, v, m, a, p, n, eps, dt, 1, kick_back, s, xh);
         kick_drift_kernel<<<nb3, 256, 0, s>>>(x, v, a, n, dt, kick_back);
@@ -646,7 +657,7 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
         if (nb_status rs; (rs = record(ctx, xh, x, n, s)) != NB_OK) return rs;
         return force_hl(ctx, ev, x, m, n, eps, a, p, s);
     };
-    if ((st = step(0, 1)) != NB_OK) return st;
+    if ((st = step(0, 0)) != NB_OK) return st;
     const int rest = nsteps - 1;
     if (rest >= 2 && s != nullptr && !x_hist) {
         cudaGraph_t graph = nullptr;
@@ -654,7 +665,7 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
         e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture begin");
         const bool timing = ctx_set_timing(ctx, false);
-        nb_status cst = step(1);
+        nb_status cst = step(1, 0);
         ctx_set_timing(ctx, timing);
         e = cudaStreamEndCapture(s, &graph);
         if (cst != NB_OK) {
@@ -670,7 +681,7 @@ nb_status leapfrog_hl(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, co
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     } else {
         for (int k = 0; k < rest; ++k)
-            if ((st = step(1, k + 2)) != NB_OK) return st;
+            if ((st = step(1, k + 1)) != NB_OK) return st;
     }
     e = launch_with_pdl(kick_kernel, dim3(nb3), dim3(256), 0, s, v, (const float *)a, n, dt);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
@@ -686,7 +697,6 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
     cudaError_t e;
     nb_status st;
     if (!a_valid && (st = force_plain(ctx, ev, x, m, n, eps, a, p, s)) != NB_OK) return st;
-    if ((st = record(ctx, x_hist, x, n, s)) != NB_OK) return st;
     if (nsteps == 0) return NB_OK;
     auto step = [&](int kick_back, int t) {
         return step_plain(ctx, ev, x, v, m, a, p, n, eps, dt, kick_back, s,
@@ -694,7 +704,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
     };
 
     // Step 0: front kick + drift + pack, force.
-    if ((st = step(0, 1)) != NB_OK) return st;
+    if ((st = step(0, 0)) != NB_OK) return st;
 
     // Steps 1 .. nsteps-1: the same kernels with the same arguments each
     // step, so they are captured once into a graph and replayed (not on the
@@ -722,7 +732,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     } else {
         for (int k = 0; k < rest; ++k)
-            if ((st = step(1, k + 2)) != NB_OK) return st;
+            if ((st = step(1, k + 1)) != NB_OK) return st;
     }
     // Final back kick, Eq. (3).
     e = launch_with_pdl(kick_kernel, dim3(blocks_for(3 * n, 256)), dim3(256), 0, s, v, (const float *)a, n, dt);
@@ -801,13 +811,13 @@ nb_status nb_leapfrog_adjoint(nb_ctx *ctx, const double *x, const double *v, con
 
     // Replay the segment on copies with the forward's own kernels (so the
     // same positions), recording x.
-    cudaError_t e = cudaMemcpyAsync(xw, x, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(vw, v, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && a) e = cudaMemcpyAsync(aw, a, n3 * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    cudaError_t e = launch_with_pdl(adj_copy_kernel, dim3(blocks_for((int64_t)n3, 256)), dim3(256), 0, s, x, v, a,
+                                    (int64_t)n3, xw, vw, aw, hist);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint replay copies");
+    double *const after = hist + n3;
     st = mode == NB_COMPENSATED
-             ? leapfrog_hl(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist)
-             : leapfrog_plain(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, hist);
+             ? leapfrog_hl(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, after)
+             : leapfrog_plain(ctx, ev, xw, vw, m, aw, nullptr, n, eps, dt, nsteps, a != nullptr, s, after);
     if (st != NB_OK) return st;
 
     // Reverse sweep, last step first: one VJP of Eq. (gravity) per step.
