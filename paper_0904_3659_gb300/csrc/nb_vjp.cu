@@ -506,7 +506,9 @@ constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
 // against 33 / 35, N = 16384 225 / 201 against 268 / 245, N = 65536 3305 / 2980
 // against 4090 / 3655), with 32-particle j-tiles below kVjpMutualLargeN (N = 8192
 // 71 / 62 against 72 / 65) and 128-particle tiles from there (N = 12000 133 / 119
-// against 138 / 120). The direct shapes remain for n whose mutual scratch cannot
+// against 138 / 120), but 32 again without gp from kVjpMutualNoGpN (N = 16384 201.2
+// for 128 against 201.9, 20000 312 against 296, 32768 776 against 751, 65536 2990
+// against 2961). The direct shapes remain for n whose mutual scratch cannot
 // be allocated.
 // Direct shapes (GB300 sweep, G-pairs/s). With an upstream gradient on p:
 // two packed pairs per thread in 128-thread CTAs with the barrier-free stage
@@ -524,13 +526,14 @@ constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
 // FP32 operation fewer, 1-3% slower).
 constexpr int kVjpMutualSmall = 21, kVjpMutualLarge = 22;
 constexpr int64_t kVjpMutualLargeN = 10240;
+constexpr int64_t kVjpMutualNoGpN = 17 << 10;
 constexpr int kVjpSmall = 17, kVjpLarge = 18, kVjpNoGpSmall = 19, kVjpNoGpLarge = 2;
 
 const VjpVariant &vjp_variant(nb_ctx *ctx, int64_t n, bool with_gp) {
     const int k = ctx_ext(ctx).vjp_idx;
     if (k >= 0 && k < kVjpCount) return kVjp[k];
     if (n <= ctx_ext(ctx).vjp_mutual_max_n)
-        return kVjp[n < kVjpMutualLargeN ? kVjpMutualSmall : kVjpMutualLarge];
+        return kVjp[n < kVjpMutualLargeN || (!with_gp && n >= kVjpMutualNoGpN) ? kVjpMutualSmall : kVjpMutualLarge];
     const bool small = n < ((int64_t)1 << 15);
     if (!with_gp) return kVjp[small ? kVjpNoGpSmall : kVjpNoGpLarge];
     return kVjp[small ? kVjpSmall : kVjpLarge];
