@@ -60,14 +60,14 @@ def alu_peak(sm_count, sm_mhz, ops) -> float:
     return sm_count * sm_mhz * 1e6 * FP32_LANES_PER_SM / ops / 1e9
 
 
-# DRAM bytes (read + write) of one launch of the large-N plain pair kernel
-# (256 threads x 4 i, 1024-particle tiles), from an ncu capture of that
-# kernel alone on a Plummer sphere of N = 131072 (4.215 MB read, 0 written).
-# The kernel reads each j-tile from L2 after its first touch, so DRAM traffic
-# grows with N, not N^2; the bench reports it scaled to its N, and null for
-# any other tile shape.
-PROFILED_TILE = (256, 4, 1024, 3, 4, 1, 0, 0, 63, 0, 0)
-PROFILED_DRAM_BYTES, PROFILED_N = 4.215e6, 131072
+# DRAM bytes (read + write) of one launch of the large-N mutual pair kernel (4
+# warps x 8 i per lane, 128-particle tiles), from an ncu capture of that kernel
+# alone on a Plummer sphere of N = 131072 (2.2 MB read, 93.4 MB written: the
+# j-side sums, one float4 per 1024 pairs, less what is still in L2 at the end).
+# They grow with N^2; the bench reports them scaled to its N, and null for any
+# other tile shape.
+PROFILED_TILE = (128, 8, 128, 3, 4, 3, 0, 1, 82, 0, 0)
+PROFILED_DRAM_BYTES, PROFILED_N = 9.56e7, 131072
 
 
 # --------------------------------------------------------------------------
@@ -493,8 +493,8 @@ def extra_adjoint(nb, ctx, dev, torch, plain_rate, oracle_ref=False):
     for _ in range(reps):
         nb.nb_force(ctx, x, mt, n, eps, a, p)
     f1.record()
-    # The trajectory adjoint's case: no upstream gradient on p (26 instead of
-    # 28 FP32 operations per pair).
+    # The trajectory adjoint's case: no upstream gradient on p (34 instead of
+    # 38 FP32 operations per unordered pair).
     for _ in range(3):
         nb.nb_force_vjp(ctx, x, mt, n, eps, ga, None, gx, gm)
     g0, g1 = _events(torch)
@@ -779,9 +779,9 @@ def run_ours(args):
         "kernels_ms_per_step": {k: v[0] / args.steps for k, v in plain_k.items()},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G-int/s",
                      "frac": achieved / peak,
-                     "traffic": (PROFILED_DRAM_BYTES * n / PROFILED_N
+                     "traffic": (PROFILED_DRAM_BYTES * (n / PROFILED_N) ** 2
                                  if plain_tile == PROFILED_TILE else None),
-                     "traffic_note": "DRAM bytes per launch, ncu capture at N=131072 scaled by N",
+                     "traffic_note": "DRAM bytes per step of the pair kernel, ncu capture at N=131072 scaled by N^2",
                      "basis": (f"{sm_count} SMs x {sm_max_mhz:.0f} MHz x {FP32_LANES_PER_SM} FP32 "
                                f"lanes / {ops} FP32 ops per interaction "
                                f"(+{MUFU_PER_INT} MUFU rsqrt, not binding); sm_max_mhz of "
