@@ -286,7 +286,7 @@ int mutual_from_fp64(nb_ctx *ctx, int64_t n, bool comp) {
         // (a single-launch shape leaves it to the built-in choice)
         if (!v.tile.fused || v.mutual >= 0) return v.mutual;
     }
-    return n <= ctx->ext.mutual_max_n ? mutual_size_from_fp64(n) : -1;
+    return n <= ctx->ext.mutual_max_n ? mutual_size_from_fp64(n, comp) : -1;
 }
 
 // Enqueue pack -> pair -> combine for one system of n particles already

@@ -207,7 +207,7 @@ int pair_default_unfused_index(bool comp, int64_t n);
 // The built-in mutual shape for n, or -1 (see nb_mutual.cu).
 int pair_mutual_index(bool comp, int64_t n);
 // The mutual shape for n FP64 positions (leap-frog, energy), or -1.
-int mutual_size_from_fp64(int64_t n);
+int mutual_size_from_fp64(int64_t n, bool comp);
 // Whether a single-launch shape serves FP64 state rounded to FP32 (plain mode).
 bool single_from_fp64(int64_t n);
 // Whether the tuner times the fused (single-launch, small-n) shapes at n.

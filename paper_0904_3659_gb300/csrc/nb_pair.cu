@@ -1355,6 +1355,10 @@ constexpr int64_t kFusedMaxN = (int64_t)3 << 13;
 // 745 / 836).
 constexpr int64_t kMutualMinN = (int64_t)13 << 10;
 constexpr int64_t kMutualMidN = kFusedMaxN;
+// On two-word positions one kernel per form pays earlier (leap-frog step with the
+// potential, equal / unequal masses / with tracers: N = 16384 139 / 149 / 156 us
+// against 142 / 148 / 171, N = 20011 194 / 207 / 218 against 199 / 207 / 242).
+constexpr int64_t kMutualMidHLN = (int64_t)9 << 11;
 constexpr int64_t kMutualLargeN = (int64_t)5 << 13;
 
 bool fused_candidate(int64_t n) { return n < (int64_t)1 << 16; }
@@ -1391,8 +1395,8 @@ int pair_mutual_index(bool comp, int64_t n) {
 // 13.0 / 22.3, 4096 22.3 / 31.5, 20011 141 / 191; compensated: 18.6 / 43.5, 29.6 / 56,
 // 190 / 290). In plain mode the single-launch cluster shapes, on positions rounded to
 // FP32, are faster yet as far as they are nb_force's choice (9728: 44.9 / 48.0).
-int mutual_size_from_fp64(int64_t n) {
-    return n < kMutualMidN ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
+int mutual_size_from_fp64(int64_t n, bool comp) {
+    return n < (comp ? kMutualMidHLN : kMutualMidN) ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
 }
 
 bool single_from_fp64(int64_t n) { return n <= kClusterMaxN; }
