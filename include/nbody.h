@@ -211,7 +211,7 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode);
  * cluster whose eps is not > 0 with eps^2 a finite normal FP32 number, are
  * detected on the device; then nothing is read or written and the next
  * nb_synchronize returns NB_ERR_ARG. Every unordered pair of a cluster of more
- * than 128 particles is evaluated once, for both its particles. Work items are
+ * than 256 particles is evaluated once, for both its particles. Work items are
  * (cluster, block of 128 i-particles, part of the blocks it meets), taken from a
  * device queue by the warps of one persistent launch; each item is summed by one
  * warp in a fixed order and the partial sums are added in a fixed order

@@ -198,14 +198,10 @@ __device__ __forceinline__ void bm_put(const BmArgs &A, const BmBlock &B, bool r
     MPart *dst = A.cp + ((int64_t)blockIdx.x * kBlock + t) * (HL ? kHLRecords : 1);
     dst[0] = r;
     if (HL) dst[1] = lo;
-    const int met = B.nt - B.b % split.band, q = split.items(met);
+    const int met = B.nt - B.b % cluster_band(split.band, B.nt), q = split.items(met);
     for (int k = t; k < q; k += kBlock) {
         int v0, v1;
-        split.range(met, k, &v0, &v1);
-        if (B.nt == 1) {  // one item (cluster_weights)
-            v0 = 0;
-            v1 = k == 0 ? kBlockTiles : 0;
-        }
+        split.range(B.nt, met, k, &v0, &v1);
         if (NB_IN(A.err, 60, (int64_t)B.first + k < A.cap_items)) A.items[B.first + k] = make_int4(c, B.b, v0, v1);
     }
 }
@@ -216,7 +212,7 @@ template <typename T, bool KICK>
 __global__ void __launch_bounds__(kBlock) bm_pack_kernel(const BmArgs A, T *__restrict__ x, double *__restrict__ v,
                                                          const float *__restrict__ a, const float *__restrict__ m,
                                                          double dt, int kick_back) {
-    pdl_wait_then_release();
+    pdl_wait();
     if ((int64_t)blockIdx.x * kBlock >= A.poff[A.C]) return;
     const BmBlock B = A.block[blockIdx.x];
     const int64_t c = B.cluster, li = (int64_t)B.b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
@@ -262,6 +258,7 @@ __global__ void __launch_bounds__(kFrameThreads) batch_frame_kernel(const double
                                                                     const int64_t *__restrict__ poff,
                                                                     double4 *__restrict__ frame) {
     __shared__ long long s[6][kFrameThreads / 32];
+    pdl_wait();
     const int64_t c = blockIdx.x;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t o = off[c], psz = poff[c + 1] - poff[c];
@@ -310,7 +307,7 @@ __global__ void __launch_bounds__(kFrameThreads) batch_frame_kernel(const double
 __global__ void __launch_bounds__(kBlock) bm_pack_hl_kernel(const BmArgs A, const double *__restrict__ x,
                                                             const float *__restrict__ m,
                                                             const double4 *__restrict__ frame) {
-    pdl_wait_then_release();
+    pdl_wait();
     if ((int64_t)blockIdx.x * kBlock >= A.poff[A.C]) return;
     const BmBlock B = A.block[blockIdx.x];
     const int64_t c = B.cluster, li = (int64_t)B.b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
@@ -334,12 +331,12 @@ __global__ void __launch_bounds__(kBlock) bm_pack_hl_kernel(const BmArgs A, cons
     bm_put<true>(A, B, li < nc, hi, lo, -0.5f * m[o]);
 }
 
-// A cluster of one block has no pairs to save: its sums are those of one evaluation
-// per (i, j), in one item, in the order of j, with the masses in the weights and
-// carried over its two tiles in FP32 (128 terms). Its particles are the heaviest of a
-// batch of clusters of equal mass, and their accelerations the least averaged.
+// The sums of a cluster of kDirectBlocks blocks or fewer are those of one evaluation
+// per (i, j): the masses in the weights, a block's j in order in one FP32 sum of 128
+// terms, the blocks' sums compensated. Their particles are the heaviest of a batch of
+// clusters of equal mass and their accelerations the least averaged.
 __device__ __forceinline__ int cluster_weights(const BmArgs &A, int c, int nt) {
-    return nt == 1 ? kWide : mutual_weights(__ldcg(A.notes + c));
+    return nt <= kDirectBlocks ? kWide : mutual_weights(__ldcg(A.notes + c));
 }
 
 // A group's particles on the first Q pairs of i-slots, for the i-side only; the
@@ -399,9 +396,9 @@ struct BmStage {
 // against 8: 669 against 678 us, against 4: 702.
 // Against one evaluation per (i, j): 1024 clusters up to 4096 particles 817 -> 685 us
 // (the pair kernel 777 -> 632; 904.8e6 unordered pairs, 66% of the FP32 lanes' issue
-// rate counting 18 operations a pair and the padding), 1024 up to 512 82 -> 58, 300
-// up to 2048 113 -> 85, a step of those on FP64 state 150 -> 121, 8 of 6000 to 20000
-// 730 -> 514.
+// rate counting 18 operations a pair and the padding), 1024 up to 512 82 -> 63, 300
+// up to 2048 113 -> 87, a step of those on FP64 state 150 -> 120, 8 of 6000 to 20000
+// 730 -> 510.
 template <int STAGES, int MINB, int UNR, bool HL>
 __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
     constexpr int P = kBatchP;
@@ -426,7 +423,9 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
         fence_mbar_init();
     }
     __syncwarp();
-    pdl_wait_then_release();
+    // (No release: the combine's blocks, resident early, slow small batches: 40 clusters
+    // up to 1024 27.6 -> 23.5 us, 32 compensated steps of 40 up to 512 1022 -> 919.)
+    pdl_wait();
 
     // Producer state (lane 0): walks the (item, tile) stream.
     int p_item = -1, p_cluster = 0, p_b = 0, p_nt = 0, p_v = 0, p_end = 0, p_done = 0;
@@ -488,7 +487,7 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc[q][r] = zero2;
     int cur_item = -1, weights = kEqual, b = 0, slots = 0, band_end = 0;
-    bool one_block = false;
+    bool direct = false;
     float4 *pj = nullptr;  // the row's j-side entries, from its block b + 1 on
     float2 eps2 = zero2;
 
@@ -543,10 +542,10 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
             const float eps = A.eps[mt.cluster];
             eps2 = splat2(eps * eps);
             const int64_t row0 = A.poff[mt.cluster], nc = A.off[mt.cluster + 1] - A.off[mt.cluster];
-            const int nt = (int)((A.poff[mt.cluster + 1] - row0) / kBlock), s0 = b / band * band;
+            const int nt = (int)((A.poff[mt.cluster + 1] - row0) / kBlock), cb = cluster_band(band, nt), s0 = b / cb * cb;
             weights = cluster_weights(A, mt.cluster, nt);
-            one_block = nt == 1;
-            band_end = min(s0 + band, nt);
+            direct = nt <= kDirectBlocks;
+            band_end = min(s0 + cb, nt);
             slots = (int)min((nc - (int64_t)b * kBlock + 31) / 32, (int64_t)(2 * P));
             pj = A.pj + batch_pj_entry(band, row0, nt, b);
             const float hm0 = A.cp[row0 * RS].w;
@@ -593,7 +592,7 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
                 else one_sided_group<P, 1, HL>(weights, G, lane, self, I, acc, eps2);
             }
         }
-        if (!one_block || mt.last) fold();
+        if (!direct || mt.last || mt.tile % kBlockTiles == kBlockTiles - 1) fold();
     }
     if (!bad) {
         if (cur_item >= 0) write_out();
@@ -625,7 +624,7 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
     if (li >= nc) return;
     float S[4] = {0.f, 0.f, 0.f, 0.f}, E[4] = {0.f, 0.f, 0.f, 0.f};
     constexpr int K = 8;  // loads in flight
-    const int s0 = b / split.band * split.band, len = min(s0 + split.band, nt) - s0;
+    const int cb = cluster_band(split.band, nt), s0 = b / cb * cb, len = min(s0 + cb, nt) - s0;
     const int64_t pj0 = batch_pj_entry(split.band, row0, nt, s0) + threadIdx.x;
     for (int r = s0; r < b; r += K) {
         float4 v[K];
@@ -644,7 +643,7 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
             comp_add(S, E, h);
         }
     }
-    const int met = nt - (b - s0), q = nt == 1 ? 1 : split.items(met);
+    const int met = nt - (b - s0), q = split.items(met);
     for (int j = 0; j < q; j += K) {
         float4 u[K];
 #pragma unroll
@@ -653,8 +652,8 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
             if (j + k >= q) continue;
             if (split.parts > 1) {  // a part past the last particle was not evaluated
                 int v0, v1;
-                split.range(met, j + k, &v0, &v1);
-                if ((int64_t)batch_met_tile(split.band, nt, b, v0) * kTile >= nc) continue;
+                split.range(nt, met, j + k, &v0, &v1);
+                if (v0 == v1 || (int64_t)batch_met_tile(split.band, nt, b, v0) * kTile >= nc) continue;
             }
             const int64_t at = ((int64_t)B.first + j + k) * kBlock + threadIdx.x;
             if (NB_IN(A.err, 67, at < A.pi_len)) u[k] = __ldcg(A.pi + at);
@@ -687,10 +686,16 @@ constexpr size_t bm_smem() {
                         sizeof(int)) + (size_t)2 * 4 * kBatchP * 32 * sizeof(float2);
 }
 
-// Leap-frog pieces that do not pack (the batched pack follows them).
+// Leap-frog pieces that do not pack (the batched pack follows them). The notes and
+// the queue head are cleared as the plan does: the steps after a call's first
+// evaluation run without one.
 __global__ void batch_kick_drift_kernel(double *__restrict__ x, double *__restrict__ v,
                                         const float *__restrict__ a, int64_t n, double dt,
-                                        int kick_back) {
+                                        int kick_back, int *__restrict__ notes, int64_t C, int *__restrict__ head) {
+    pdl_wait_then_release();
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += gridDim.x * (int64_t)blockDim.x)
+        notes[c] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *head = 0;
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= 3 * n) return;
     const double h = 0.5 * dt, g = -(double)a[k];
@@ -703,6 +708,7 @@ __global__ void batch_kick_drift_kernel(double *__restrict__ x, double *__restri
 
 __global__ void batch_kick_kernel(double *__restrict__ v, const float *__restrict__ a, int64_t n,
                                   double dt) {
+    pdl_wait_then_release();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= 3 * n) return;
     v[k] = v[k] + (0.5 * dt) * (-(double)a[k]);  // Eq. (3)
@@ -812,13 +818,17 @@ nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
     return bm_args(ctx, k, true, out);
 }
 
-// One evaluation.
-nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource &src, float *a, float *p,
+// One evaluation. `planned`: this call has made one before, so its plan is there (on
+// FP64 state in compensated mode; 32 steps of 300 clusters 4070 -> 4010 us).
+nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource &src, bool planned, float *a, float *p,
                    cudaStream_t st) {
     ExtState &es = ctx_ext(ctx);
-    A.fresh = !es.batch_plan;
-    cudaError_t e = launch_with_pdl(bm_plan_kernel, dim3(1), dim3(kBmPlanThreads), 0, st, A);
-    es.batch_plan = e == cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (!(planned && k.hl && src.kick)) {
+        A.fresh = !es.batch_plan;
+        e = launch_with_pdl(bm_plan_kernel, dim3(1), dim3(kBmPlanThreads), 0, st, A);
+        es.batch_plan = e == cudaSuccess;
+    }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch plan launch");
     const dim3 blocks((unsigned)(A.cap_padded / kBlock)), threads(kBlock);
     double *const no_v = nullptr;
@@ -826,12 +836,13 @@ nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource 
     if (k.hl) {
         double4 *frame = static_cast<double4 *>(es.buf[SLOT_BATCH_FRAME]);
         if (src.kick) {
-            batch_kick_drift_kernel<<<(unsigned)((3 * k.n_total + 255) / 256), 256, 0, st>>>(
-                src.x64, src.v, src.a, k.n_total, src.dt, src.kick_back);
-            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
+            e = launch_with_pdl(batch_kick_drift_kernel, dim3((unsigned)((3 * k.n_total + 255) / 256)), dim3(256), 0, st,
+                                src.x64, src.v, src.a, k.n_total, src.dt, src.kick_back, A.notes, k.C, A.head);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
         }
-        batch_frame_kernel<<<(unsigned)k.C, kFrameThreads, 0, st>>>(src.x64, k.offsets, A.poff, frame);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "batched frame launch");
+        e = launch_with_pdl(batch_frame_kernel, dim3((unsigned)k.C), dim3(kFrameThreads), 0, st,
+                            (const double *)src.x64, k.offsets, (const int64_t *)A.poff, frame);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "batched frame launch");
         e = launch_with_pdl(bm_pack_hl_kernel, blocks, threads, 0, st, A, (const double *)src.x64, src.m,
                             (const double4 *)frame);
     } else if (src.x32) {
@@ -882,7 +893,7 @@ nb_status nb_force_batched(nb_ctx *ctx, const float *x, const float *m, const in
     BatchSource src{};
     src.x32 = x;
     src.m = m;
-    return bm_force(ctx, call, A, src, a, p, static_cast<cudaStream_t>(stream));
+    return bm_force(ctx, call, A, src, false, a, p, static_cast<cudaStream_t>(stream));
 }
 
 nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const float *m,
@@ -903,8 +914,12 @@ nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const floa
     BmArgs A;
     if ((st = bm_prepare(ctx, call, &A)) != NB_OK) return st;
     cudaError_t e;
+    bool planned = false;
     auto evaluate = [&](int kick, int kick_back) {
-        return bm_force(ctx, call, A, BatchSource{nullptr, x, v, a, m, dt, kick, kick_back}, a, p, s);
+        const nb_status rs = bm_force(ctx, call, A, BatchSource{nullptr, x, v, a, m, dt, kick, kick_back}, planned, a,
+                                      p, s);
+        planned = true;
+        return rs;
     };
     auto force = [&]() { return evaluate(0, 0); };
     auto step = [&](int kick_back) { return evaluate(1, kick_back); };
@@ -937,8 +952,9 @@ nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const floa
         for (int k = 0; k < rest; ++k)
             if ((st = step(1)) != NB_OK) return st;
     }
-    batch_kick_kernel<<<(unsigned)((3 * n_total + 255) / 256), 256, 0, s>>>(v, a, n_total, dt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
+    e = launch_with_pdl(batch_kick_kernel, dim3((unsigned)((3 * n_total + 255) / 256)), dim3(256), 0, s, v,
+                        (const float *)a, n_total, dt);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "kick launch");
     return NB_OK;
 }
 

@@ -23,6 +23,11 @@ constexpr int kBlock = 128;  // particles per block: 4 per lane
 constexpr int kTile = 64;    // particles per copy
 constexpr int kBlockTiles = kBlock / kTile;
 constexpr int kMinBand = 32;  // blocks that a band may always have
+// Clusters of up to so many blocks are evaluated per (i, j), every block by every row
+// (a band of one block): they have few pairs to save (cluster_weights, nb_batched.cu).
+constexpr int kDirectBlocks = 2;
+
+__host__ __device__ inline int cluster_band(int band, int64_t nt) { return nt <= kDirectBlocks ? 1 : band; }
 
 struct BatchSplit {
     int band;          // blocks per band
@@ -37,15 +42,18 @@ struct BatchSplit {
     // The first item of row b of a cluster of nt blocks, counted from the
     // cluster's first (b = nt: their number).
     __host__ __device__ int64_t first(int64_t nt, int64_t b) const {
-        const int64_t k = b / band, r = b - k * band, f = below(nt);
-        return (k ? k * (f - below(nt - band)) : 0) + (r ? f - below(nt - r) : 0);
+        const int cb = cluster_band(band, nt);
+        const int64_t k = b / cb, r = b - k * cb, f = below(nt);
+        return (k ? k * (f - below(nt - cb)) : 0) + (r ? f - below(nt - r) : 0);
     }
-    // Item k of a row with t blocks to meet: the met tiles [*v0, *v1).
-    __host__ __device__ void range(int t, int k, int *v0, int *v1) const {
+    // Item k of a row of a cluster of nt blocks, t of them to meet: the met tiles
+    // [*v0, *v1). Blocks of the smallest clusters are not parted.
+    __host__ __device__ void range(int nt, int t, int k, int *v0, int *v1) const {
         if (parts > 1) {
             constexpr int n = kBlockTiles;
             *v0 = k * (n / parts);
             *v1 = *v0 + n / parts;
+            if (nt <= kDirectBlocks) *v1 = k % parts ? *v0 : *v0 + n;
             return;
         }
         const int q = items(t), each = t / q, more = t - each * q;  // the first `more` have one block more
@@ -69,6 +77,7 @@ __host__ __device__ inline int64_t batch_met(int band, int64_t nt) { return Batc
 
 // The v-th block that row b meets.
 __host__ __device__ inline int batch_met_block(int band, int nt, int b, int v) {
+    band = cluster_band(band, nt);
     const int s0 = b / band * band, s1 = s0 + band < nt ? s0 + band : nt;
     if (v < s1 - b) return b + v;
     const int w = v - (s1 - b);

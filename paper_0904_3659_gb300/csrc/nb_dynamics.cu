@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) kick_drift_box_kernel(double *__restrict_
                                                              long long *__restrict__ box,
                                                              double *__restrict__ xh) {
     __shared__ long long s[8][6];
-    pdl_wait_then_release();
+    pdl_wait();
     const double h = 0.5 * dt;
     long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
     for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)

@@ -80,7 +80,12 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
     int *issued_at = reinterpret_cast<int *>(full + STAGES);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    pdl_wait_then_release();  // the packed particles are ready
+    // The packed particles are ready. The combine's blocks, resident early, slow the
+    // kernel down at small n (compensated step, N = 4096 32.0 -> 30.1 us, N = 16384
+    // 140 -> 139); with a kernel per form the next one is released (N = 65536 1287
+    // against 1294 us).
+    if (W == kAny) pdl_wait();
+    else pdl_wait_then_release();
     const int weights = mutual_weights(__ldcg(A.notes) | (A.wide_eps ? kNoteWide : 0));
     if (W != kAny && W != weights) return;
     const int64_t c = blockIdx.x;

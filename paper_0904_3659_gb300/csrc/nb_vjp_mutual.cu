@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) vjp_mutual_kernel(const VmAr
         fence_mbar_init();
     }
     __syncthreads();
-    pdl_wait_then_release();
+    pdl_wait();  // (no release: the combine's blocks, resident early, cost 1-2%)
 
     int64_t pb = b, pt = t;  // thread 0: the next tile to copy
     auto issue = [&](int kk) {
