@@ -43,11 +43,14 @@ using MPart = float4;
 //            operations (14 without the potential).
 //  kProduct  w = ((c m_i m_j) y) y^2, one weight for both sides; the combine
 //            divides by a particle's own c m_i. 18 operations. c is a power of
-//            two (mutual_scale) that keeps w inside FP32's range for masses
-//            within 2^28 of the first one and distances up to 2^39 eps.
+//            two (product_scale) that keeps every product and sum inside FP32's
+//            range for masses within a factor of the first one and distances up to
+//            a multiple of eps that depend on eps (2^28 and 2^34 up to eps = 1, 2^15
+//            and 2^21 at eps = 2^40).
 //  kWide     w_i = ((-m_j/2) y) y^2, w_j = ((-m_i/2) y) y^2: 19 operations, for
-//            everything else (massless particles, positions or softening
-//            outside [2^-40, 2^40], infinities and NaN).
+//            everything else (massless particles, wider ranges of masses or
+//            distances, positions or softening outside [2^-40, 2^40],
+//            infinities and NaN).
 // One weight for both sides also means fewer registers read. Measured at N =
 // 131072, G-interactions/s: kEqual 3450, kProduct 3090, and 2830-2980 for the
 // form w_i = (-m_j/2) y^3, w_j = (-m_i/2) y^3, also 18 operations.
@@ -65,18 +68,36 @@ __device__ __forceinline__ int mutual_weights(int notes) {
     return notes & kNoteNoProduct ? kWide : kProduct;
 }
 
-// kProduct: times 2^-e0 twice, e0 the exponent of the first mass, and 2^60
-// eps^3 rounded down to a power of two, applied to an i-particle's -m_i/2.
-// With |m| within 2^28 of the first and r <= 2^39 eps, w lies in [2^-117, 2^117].
-__device__ __forceinline__ float mutual_scale(float hm, float hm0, float eps) {
-    const int e0 = ilogbf(hm0), e = ilogbf(eps);
-    return ldexpf(hm, 60 + 3 * e - 2 * e0);
+// kProduct's ranges. With e the exponent of eps and e0 that of the first particle's
+// -m/2, every -m/2 lies within 2^+-ratio of the first one's, every coordinate within
+// 2^(reach - 2) eps, so every distance below 2^reach eps, and c = 2^(shift - 2 e0).
+// The products and sums are then bounded by
+//   c m_i              2^(t - ratio) .. 2^(t + ratio + 1) with t = shift - e0
+//   c m_i m_j          2^(shift - 2 ratio) .. 2^(shift + 2 ratio + 2)
+//   c m_i m_j y        2^(shift - e + 2 ratio + 2), 2^31 of them by 2^(shift - e + 2 ratio + 33)
+//   w = c m_i m_j y^3  2^(shift - 3 e - 2 ratio - 3 reach - 3) .. 2^(shift - 3 e + 2 ratio + 2)
+//   w d                2^(shift - 2 e + 2 ratio + 1), 2^31 of them by 2^(shift - 2 e + 2 ratio + 32)
+// For the products to be normal numbers and the sums to be finite, 4 ratio + 3 reach
+// may be 214 - max(2 e, 3 e - 33, 0): where eps > 1 masses and distances give up as
+// many powers of two each. What room `shift` has goes to the range of the first mass.
+struct ProductScale {
+    int ratio, reach, shift;
+    bool fits;  // c m_i is a normal number
+};
+__host__ __device__ constexpr ProductScale product_scale(int e0, int e) {
+    const auto lesser = [](int a, int b) { return a < b ? a : b; };
+    const auto greater = [](int a, int b) { return a > b ? a : b; };
+    const int less = (greater(greater(2 * e, 3 * e - 33), 0) + 6) / 7, ratio = 28 - less, reach = 34 - less;
+    const int least = greater(3 * e + 2 * ratio + 3 * reach - 122, 2 * ratio - 126);
+    const int most = 94 - 2 * ratio + lesser(lesser(e, 2 * e + 1), lesser(3 * e + 31, 31));
+    const int shift = greater(least, lesser(e0, most)), t = shift - e0;
+    return {ratio, reach, shift, t - ratio >= -126 && t + ratio <= 126};
 }
-// Whether that scale stays in range for every such mass.
-__device__ __forceinline__ bool mutual_scale_fits(float hm0, float eps) {
-    if (!(fabsf(hm0) >= 1e-37f && fabsf(hm0) <= 1e37f)) return false;  // zero, subnormal, infinite, NaN
-    const int t = 60 + 3 * ilogbf(eps) - ilogbf(hm0);
-    return t >= -95 && t <= 95;
+
+// c m_i of an i-particle's -m_i/2.
+__device__ __forceinline__ float mutual_scale(float hm, float hm0, float eps) {
+    const int e0 = ilogbf(hm0);
+    return ldexpf(hm, product_scale(e0, ilogbf(eps)).shift - 2 * e0);
 }
 
 // Padding records: no mass, and so far away that s overflows to infinity and y
@@ -92,9 +113,11 @@ __device__ __forceinline__ void mutual_note(bool real, const MPart &v, float hm0
         const float r = fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))), m = fabsf(v.w), m0 = fabsf(hm0);
         if (!(r <= kMutualRange) || v.x != v.x || v.y != v.y || v.z != v.z) k |= kNoteWide;
         if (__float_as_uint(v.w) != __float_as_uint(hm0) || !(m <= 1.7e38f)) k |= kNoteUnequal;
-        if (!(r <= eps * 137438953472.f)) k |= kNoteNoProduct;  // 2^37 eps per coordinate
-        if (!(m >= m0 * 3.7252903e-9f && m * 3.7252903e-9f <= m0)) k |= kNoteNoProduct;  // 2^-28
-        if (!mutual_scale_fits(hm0, eps)) k |= kNoteNoProduct;
+        const bool normal = m0 >= 1e-37f && m0 <= 1e37f;  // not zero, subnormal, infinite, NaN
+        const ProductScale q = product_scale(normal ? ilogbf(hm0) : 0, ilogbf(eps));
+        if (!normal || !q.fits || !(r <= ldexpf(eps, q.reach - 2)) ||
+            !(m >= ldexpf(m0, -q.ratio) && ldexpf(m, -q.ratio) <= m0))
+            k |= kNoteNoProduct;
     }
     const int any = __syncthreads_or(k & kNoteUnequal) * kNoteUnequal |
                     (__syncthreads_or(k & kNoteNoProduct) ? kNoteNoProduct : 0) |
