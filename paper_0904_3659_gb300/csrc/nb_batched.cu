@@ -55,8 +55,8 @@ struct BmArgs {
     float4 *pj;            // j-side sums (batch_pj_entry)
     int *err;
     uint64_t wait_ns;
-    // What the plan in the scratch was made for: sizes and offsets. fresh: nothing.
-    int64_t *planned;  // [3] C (-1: none), n_total, want_items
+    // What the plan in the scratch was made for. fresh: nothing.
+    BatchKey *planned;
     int64_t *planned_off;
     int fresh;
     int64_t pi_len, pj_len;
@@ -102,7 +102,8 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
     const int t = threadIdx.x;
     for (int64_t c = t; c < P.C; c += kBmPlanThreads) P.notes[c] = 0;
     if (t == 0) *P.head = 0;
-    const int stands = !P.fresh && P.planned[0] == P.C && P.planned[1] == P.n_total && P.planned[2] == P.want_items;
+    const BatchKey key{P.C, P.n_total, P.want_items, P.max_band};
+    const int stands = !P.fresh && same_plan(*P.planned, key);
     int bad = 0, replan = !stands;
     for (int64_t c = t; c < P.C; c += kBmPlanThreads) {
         const int64_t o = P.off[c], end = P.off[c + 1];
@@ -117,7 +118,7 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
         for (int64_t c = t; c <= P.C; c += kBmPlanThreads) P.poff[c] = 0;
         if (t == 0) {
             *P.nitems = 0;
-            P.planned[0] = -1;
+            P.planned->clusters = -1;
             atomicOr(P.err, kErrBatchPlan);
         }
         return;
@@ -175,9 +176,8 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
     if (t == 0) {
         *P.nitems = ok ? (int)nit : 0;
         if (!ok) atomicOr(P.err, kErrBatchPlan);
-        P.planned[0] = ok ? P.C : -1;
-        P.planned[1] = P.n_total;
-        P.planned[2] = P.want_items;
+        *P.planned = key;
+        if (!ok) P.planned->clusters = -1;
     }
     for (int64_t c = t; c <= P.C; c += kBmPlanThreads) {
         if (!ok) P.poff[c] = 0;
@@ -765,7 +765,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.max_band = small ? 1 : (int)std::min(most, std::max<int64_t>(kMinBand, kPjEntries / (blocks * (kBlock / 2))));
     const int64_t pj = (blocks + 1) * (kBlock / 2 * (A.max_band - 1));
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    // [planned sizes, item count, queue head, split][poff][ibase][planned offsets][notes][padded blocks]
+    // [the plan's key, item count, queue head, split][poff][ibase][planned offsets][notes][padded blocks]
     const size_t b_off = al((size_t)(k.C + 1) * sizeof(int64_t)), b_c = al((size_t)k.C * sizeof(int));
     const size_t b_blk = al((size_t)blocks * sizeof(BmBlock));
     const size_t plan_before = es.cap[SLOT_BATCH_PLAN];
@@ -782,7 +782,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     if (k.hl) need(SLOT_BATCH_FRAME, (size_t)k.C * sizeof(double4));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (batched)");
     unsigned char *plan = static_cast<unsigned char *>(es.buf[SLOT_BATCH_PLAN]);
-    A.planned = reinterpret_cast<int64_t *>(plan);
+    A.planned = reinterpret_cast<BatchKey *>(plan);
     A.nitems = reinterpret_cast<int *>(plan + 64);
     A.head = A.nitems + 1;
     A.split = reinterpret_cast<BatchSplit *>(A.nitems + 2);

@@ -29,6 +29,16 @@ constexpr int kDirectBlocks = 2;
 
 __host__ __device__ inline int cluster_band(int band, int64_t nt) { return nt <= kDirectBlocks ? 1 : band; }
 
+// What a plan depends on besides the offsets. A plan made for longer bands than a
+// call has scratch for must not stand: its j-side sums would go past their buffer.
+struct BatchKey {
+    int64_t clusters, n_total, want_items, max_band;  // clusters -1: no plan
+};
+__host__ __device__ inline bool same_plan(const BatchKey &a, const BatchKey &b) {
+    return a.clusters == b.clusters && a.n_total == b.n_total && a.want_items == b.want_items &&
+           a.max_band == b.max_band;
+}
+
 struct BatchSplit {
     int band;          // blocks per band
     int chunk, parts;  // one of them is 1
