@@ -776,9 +776,9 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     need(SLOT_BATCH_PLAN, 256 + 3 * b_off + b_c + b_blk);
     if (es.cap[SLOT_BATCH_PLAN] != plan_before) es.batch_plan = false;
     need(SLOT_BATCH_ITEMS, (size_t)A.cap_items * sizeof(int4));
-    need(SLOT_MUTUAL_CP, (size_t)A.cap_padded * (k.hl ? kHLRecords : 1) * sizeof(MPart));
-    need(SLOT_MUTUAL_PI, (size_t)A.cap_items * kBlock * sizeof(float4));
-    need(SLOT_MUTUAL_PJ, (size_t)pj * sizeof(float4));
+    need(SLOT_BATCH_CP, (size_t)A.cap_padded * (k.hl ? kHLRecords : 1) * sizeof(MPart));
+    need(SLOT_BATCH_PI, (size_t)A.cap_items * kBlock * sizeof(float4));
+    need(SLOT_BATCH_PJ, (size_t)pj * sizeof(float4));
     if (k.hl) need(SLOT_BATCH_FRAME, (size_t)k.C * sizeof(double4));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (batched)");
     unsigned char *plan = static_cast<unsigned char *>(es.buf[SLOT_BATCH_PLAN]);
@@ -793,13 +793,13 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.notes = reinterpret_cast<int *>(plan + 3 * b_off);
     A.block = reinterpret_cast<BmBlock *>(plan + 3 * b_off + b_c);
     A.items = static_cast<int4 *>(es.buf[SLOT_BATCH_ITEMS]);
-    A.cp = static_cast<MPart *>(es.buf[SLOT_MUTUAL_CP]);
-    A.pi = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PI]);
-    A.pj = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PJ]);
+    A.cp = static_cast<MPart *>(es.buf[SLOT_BATCH_CP]);
+    A.pi = static_cast<float4 *>(es.buf[SLOT_BATCH_PI]);
+    A.pj = static_cast<float4 *>(es.buf[SLOT_BATCH_PJ]);
     A.err = ctx_err_word(ctx);
     A.wait_ns = ctx_wait_ns(ctx);
-    A.pi_len = (int64_t)(es.cap[SLOT_MUTUAL_PI] / sizeof(float4));
-    A.pj_len = (int64_t)(es.cap[SLOT_MUTUAL_PJ] / sizeof(float4));
+    A.pi_len = (int64_t)(es.cap[SLOT_BATCH_PI] / sizeof(float4));
+    A.pj_len = (int64_t)(es.cap[SLOT_BATCH_PJ] / sizeof(float4));
     *out = A;
     return NB_OK;
 }

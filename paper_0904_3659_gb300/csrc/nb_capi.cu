@@ -300,7 +300,7 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *pr
     if (vp->mutual >= 0) {
         if (!prepacked) {
             const MutualShape &s = mutual_shape(vp->mutual, p != nullptr, false);
-            const nb_status rs = mutual_reserve(ctx, s, n);
+            const nb_status rs = mutual_reserve(ctx, s, n, kMutualForce);
             if (rs == NB_OK) return run_mutual(ctx, s, x, m, n, eps, a, p, st);
             if (rs != NB_ERR_OOM || shape_is_chosen(ctx, n, comp)) return rs;
         }
@@ -412,6 +412,28 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const JPart *pr
         e = launch_reduce(ra, v.comp, st);  // the combine matches the kernel's running sums
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "combine kernel launch");
+    return NB_OK;
+}
+
+nb_status reserve_direct(nb_ctx *ctx, int64_t n, bool comp) {
+    size_t jp = 0, part = 0;
+    int64_t nib = 0;
+    // Every direct shape this context might pick for n (and the shapes' twins
+    // without the potential): reserve for the largest.
+    for (int k = 0; k < pair_variant_count(comp); ++k) {
+        const PairVariant *cands[2] = {pair_variant(comp, k), sums_twin(*pair_variant(comp, k), kSumA)};
+        for (const PairVariant *vp : cands) {
+            if (!vp || vp->mutual >= 0) continue;
+            const PairPlan plan = make_plan(*vp, n, resident_ctas(ctx, *vp));
+            jp = std::max(jp, (size_t)plan.npad * sizeof(JPart));
+            part = std::max(part, plan.partial_bytes);
+            if (vp->tile.fused) nib = std::max(nib, plan.nib);
+        }
+    }
+    cudaError_t e = ensure_buffer(&ctx->d_jp, &ctx->jp_bytes, jp);
+    if (e == cudaSuccess) e = ensure_buffer(&ctx->d_partial, &ctx->partial_bytes, part);
+    if (e == cudaSuccess && nib > 0) e = ensure_counters(ctx, nib);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (direct shapes)");
     return NB_OK;
 }
 
@@ -581,33 +603,16 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode) {
     if (n == 0) return NB_OK;
     DeviceGuard g(ctx->device);
     const bool comp = mode == NB_COMPENSATED;
-    size_t jp = 0, part = 0;
-    int64_t nib = 0;
-    // Every shape this context might pick for n (and the shapes' twins
-    // without the potential): reserve for the largest.
     for (int k = 0; k < pair_variant_count(comp); ++k) {
-        const PairVariant *cands[2] = {pair_variant(comp, k), sums_twin(*pair_variant(comp, k), kSumA)};
-        for (const PairVariant *vp : cands) {
-            if (!vp) continue;
-            if (vp->mutual >= 0) {
-                // Without this scratch the built-in choice is a direct shape.
-                for (bool pot : {true, false}) {
-                    const nb_status rs = mutual_reserve(ctx, mutual_shape(vp->mutual, pot, false), n);
-                    if (rs != NB_OK && rs != NB_ERR_OOM) return rs;
-                }
-                continue;
-            }
-            const PairPlan plan = make_plan(*vp, n, resident_ctas(ctx, *vp));
-            jp = std::max(jp, (size_t)plan.npad * sizeof(JPart));
-            part = std::max(part, plan.partial_bytes);
-            if (vp->tile.fused) nib = std::max(nib, plan.nib);
+        const int mutual = pair_variant(comp, k)->mutual;
+        if (mutual < 0) continue;
+        // Without this scratch the built-in choice is a direct shape.
+        for (bool pot : {true, false}) {
+            const nb_status rs = mutual_reserve(ctx, mutual_shape(mutual, pot, false), n, kMutualForce);
+            if (rs != NB_OK && rs != NB_ERR_OOM) return rs;
         }
     }
-    cudaError_t e = ensure_buffer(&ctx->d_jp, &ctx->jp_bytes, jp);
-    if (e == cudaSuccess) e = ensure_buffer(&ctx->d_partial, &ctx->partial_bytes, part);
-    if (e == cudaSuccess && nib > 0) e = ensure_counters(ctx, nib);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "nb_reserve");
-    return NB_OK;
+    return reserve_direct(ctx, n, comp);
 }
 
 nb_status nb_force_host(nb_ctx *ctx, const float *x, const float *m, int64_t n, float eps, float *a,

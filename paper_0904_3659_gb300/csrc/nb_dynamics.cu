@@ -513,7 +513,7 @@ nb_status choose_evaluator(nb_ctx *ctx, int64_t n, bool comp, bool pot, Evaluato
     const int size = mutual_from_fp64(ctx, n, comp);
     if (size < 0) return NB_OK;
     const MutualShape &s = mutual_shape(size, pot, comp);
-    const nb_status st = mutual_reserve(ctx, s, n);
+    const nb_status st = mutual_reserve(ctx, s, n, kMutualFp64);
     if (st == NB_OK) ev->mutual = &s;
     return st == NB_ERR_OOM ? NB_OK : st;
 }
@@ -551,7 +551,7 @@ nb_status step_hl_mutual(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
     if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
     const int64_t npad = mutual_npad(*ev.mutual, n);
     e = launch_with_pdl(mutual_hl_pack_kernel, dim3((unsigned)mutual_pack_blocks(npad)), dim3(kMutualPackThreads), 0,
-                        st, (const double *)x, m, n, npad, (const long long *)box, nbox, eps, mutual_records(ctx),
+                        st, (const double *)x, m, n, npad, (const long long *)box, nbox, eps, mutual_records(ctx, kMutualFp64),
                         mutual_notes(ctx));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "HL pack launch");
     return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
@@ -597,7 +597,7 @@ nb_status force_plain(nb_ctx *ctx, const Evaluator &ev, double *x, const float *
         const int64_t npad = mutual_npad(*ev.mutual, n);
         e = launch_with_pdl(mutual_pack_f64_kernel<false>, dim3((unsigned)mutual_pack_blocks(npad)),
                             dim3(kMutualPackThreads), 0, st, x, (double *)nullptr, (const float *)nullptr, m, n, npad,
-                            0.0, 0, eps, mutual_records(ctx), mutual_notes(ctx), (double *)nullptr);
+                            0.0, 0, eps, mutual_records(ctx, kMutualFp64), mutual_notes(ctx), (double *)nullptr);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "pack launch");
         return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
     }
@@ -625,7 +625,7 @@ nb_status step_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v, con
         const int64_t npad = mutual_npad(*ev.mutual, n);
         e = launch_with_pdl(mutual_pack_f64_kernel<true>, dim3((unsigned)mutual_pack_blocks(npad)),
                             dim3(kMutualPackThreads), 0, st, x, v, (const float *)a, m, n, npad, dt, kick_back, eps,
-                            mutual_records(ctx), mutual_notes(ctx), xh);
+                            mutual_records(ctx, kMutualFp64), mutual_notes(ctx), xh);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
         return run_mutual(ctx, *ev.mutual, nullptr, nullptr, n, eps, a, p, st);
     }
@@ -745,7 +745,7 @@ nb_status leapfrog_plain(nb_ctx *ctx, const Evaluator &ev, double *x, double *v,
 nb_status reserve_leapfrog(nb_ctx *ctx, int64_t n, nb_mode mode) {
     nb_status st;
     if ((st = reserve_force(ctx, n, mode == NB_COMPENSATED)) != NB_OK) return st;
-    return nb_reserve(ctx, n, mode);
+    return reserve_direct(ctx, n, mode == NB_COMPENSATED);
 }
 
 }  // namespace

@@ -24,14 +24,27 @@ enum ExtSlot : int {
     SLOT_HL_BOX,        // bounding-box partials of FP64 positions (HL packing)
     SLOT_ADJOINT,       // leap-frog adjoint: replayed state, position history, VJP operands
     SLOT_BATCH_FRAME,   // per-cluster HL frames (centre, grid) of the batched leap-frog
-    SLOT_MUTUAL_CP,     // mutual kernels: packed particles
-    SLOT_MUTUAL_PI,     //   segment sums of the i-side
-    SLOT_MUTUAL_PJ,     //   j-side sums of a panel of rows
-    SLOT_MUTUAL_ROWS,   //   first and last CTA of each row
-    SLOT_MUTUAL_STATE,  //   sums carried from panel to panel
-    SLOT_MUTUAL_NOTES,  //   the form of the weights, and what the pack found
-    SLOT_COUNT
+    SLOT_BATCH_CP,      // batched: packed particles
+    SLOT_BATCH_PI,      //   sums of the i-side
+    SLOT_BATCH_PJ,      //   sums of the j-side
+    SLOT_MUTUAL_NOTES,  // mutual kernels: the form of the weights, and what the pack found
+    SLOT_MUTUAL,        //   the other scratch of each user (mutual_slot)
+    SLOT_COUNT = SLOT_MUTUAL + 15
 };
+
+// The calls that run mutual kernels, each with scratch of its own: a captured nb_force
+// must find its buffers where they were, whatever the other calls need meanwhile.
+enum MutualUser : int { kMutualForce = 0, kMutualFp64 = 1, kMutualVjp = 2 };
+enum MutualPart : int {
+    kPartCp = 0,  // packed particles
+    kPartPi,      // segment sums of the i-side
+    kPartPj,      // j-side sums of a panel of rows
+    kPartRows,    // first and last CTA of each row
+    kPartState,   // sums carried from panel to panel
+    kMutualParts
+};
+inline int mutual_slot(MutualUser user, MutualPart part) { return SLOT_MUTUAL + kMutualParts * user + part; }
+static_assert(SLOT_COUNT == SLOT_MUTUAL + 3 * kMutualParts, "every part of every user");
 
 struct ExtState {
     static constexpr int kSlots = SLOT_COUNT;
@@ -87,6 +100,8 @@ const nbk::PairVariant &choose_variant(nb_ctx *ctx, int64_t n, bool comp);
 // (the potential is then not summed). only_p: a is zeroed, not summed.
 nb_status run_force_hl(nb_ctx *ctx, const nbk::JPart *jp, int64_t n, float eps, float *a, float *p,
                        cudaStream_t st, bool only_p = false);
+// Allocate what the direct shapes need for n, whichever is picked.
+nb_status reserve_direct(nb_ctx *ctx, int64_t n, bool comp);
 // Allocate the HL path's partial sums for n (before any graph capture).
 nb_status reserve_hl(nb_ctx *ctx, int64_t n);
 
@@ -96,8 +111,8 @@ nb_status run_force(nb_ctx *ctx, const float *x, const float *m, const nbk::JPar
                     bool only_p = false);
 
 // Mutual kernels (nb_mutual.cu). mutual_reserve allocates what n needs; the
-// records are then packed by run_mutual from x, m, or, with x NULL, by a kernel
-// of the caller's (mutual_pack_blocks blocks of kMutualPackThreads) into
+// records are then packed by run_mutual from x, m, or, with x NULL (the calls on FP64
+// state, kMutualFp64), by a kernel of the caller's (mutual_pack_blocks blocks of kMutualPackThreads) into
 // mutual_records, with mutual_note on mutual_notes. a or p may be NULL.
 constexpr int kMutualPackThreads = 128;
 inline int64_t mutual_pack_blocks(int64_t npad) { return (npad + kMutualPackThreads - 1) / kMutualPackThreads; }
@@ -105,8 +120,8 @@ inline int64_t mutual_pack_blocks(int64_t npad) { return (npad + kMutualPackThre
 // the built-in one, or for a plain call the one forced or tuned.
 int mutual_from_fp64(nb_ctx *ctx, int64_t n, bool comp);
 int64_t mutual_npad(const nbk::MutualShape &s, int64_t n);
-nb_status mutual_reserve(nb_ctx *ctx, const nbk::MutualShape &s, int64_t n);
-float4 *mutual_records(nb_ctx *ctx);
+nb_status mutual_reserve(nb_ctx *ctx, const nbk::MutualShape &s, int64_t n, MutualUser user);
+float4 *mutual_records(nb_ctx *ctx, MutualUser user);
 int *mutual_notes(nb_ctx *ctx);
 nb_status run_mutual(nb_ctx *ctx, const nbk::MutualShape &s, const float *x, const float *m, int64_t n, float eps,
                      float *a, float *p, cudaStream_t st);

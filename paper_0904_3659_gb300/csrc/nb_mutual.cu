@@ -480,8 +480,12 @@ int64_t panel_tiles(const MutualShape &s) { return (int64_t)(kMutualPartialBytes
 
 int64_t mutual_npad(const MutualShape &s, int64_t n) { return round_up(std::max<int64_t>(n, 1), s.ib); }
 
-nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n) {
+nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n, MutualUser user) {
     ExtState &es = ctx_ext(ctx);
+    auto need = [&](MutualPart part, size_t bytes) {
+        const int k = mutual_slot(user, part);
+        return ensure_buffer(&es.buf[k], &es.cap[k], bytes);
+    };
     const Triangle T = triangle(s, n);
     int64_t pj = 1, rows = 1;
     bool panels = false;
@@ -494,16 +498,11 @@ nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n) {
     }
     const int64_t pi = (most_resident(ctx, s) + rows) * 2 * s.ib;
     const size_t records = s.hl ? kHLRecords : 1;
-    cudaError_t e = ensure_buffer(&es.buf[SLOT_MUTUAL_CP], &es.cap[SLOT_MUTUAL_CP],
-                                  (size_t)mutual_npad(s, n) * records * sizeof(MPart));
-    if (e == cudaSuccess)
-        e = ensure_buffer(&es.buf[SLOT_MUTUAL_PI], &es.cap[SLOT_MUTUAL_PI], (size_t)pi * sizeof(float4));
-    if (e == cudaSuccess)
-        e = ensure_buffer(&es.buf[SLOT_MUTUAL_PJ], &es.cap[SLOT_MUTUAL_PJ], (size_t)pj * sizeof(float4));
-    if (e == cudaSuccess)
-        e = ensure_buffer(&es.buf[SLOT_MUTUAL_ROWS], &es.cap[SLOT_MUTUAL_ROWS], (size_t)2 * T.nib * sizeof(int));
-    if (e == cudaSuccess && panels)
-        e = ensure_buffer(&es.buf[SLOT_MUTUAL_STATE], &es.cap[SLOT_MUTUAL_STATE], (size_t)n * 2 * sizeof(float4));
+    cudaError_t e = need(kPartCp, (size_t)mutual_npad(s, n) * records * sizeof(MPart));
+    if (e == cudaSuccess) e = need(kPartPi, (size_t)pi * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartPj, (size_t)pj * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartRows, (size_t)2 * T.nib * sizeof(int));
+    if (e == cudaSuccess && panels) e = need(kPartState, (size_t)n * 2 * sizeof(float4));
     if (e == cudaSuccess && !es.buf[SLOT_MUTUAL_NOTES]) {
         e = ensure_buffer(&es.buf[SLOT_MUTUAL_NOTES], &es.cap[SLOT_MUTUAL_NOTES], 2 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(es.buf[SLOT_MUTUAL_NOTES], 0, 2 * sizeof(int));
@@ -514,26 +513,30 @@ nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n) {
     return cuda_fail(ctx, e, "scratch allocation (mutual pair sums)");
 }
 
-MPart *mutual_records(nb_ctx *ctx) { return static_cast<MPart *>(ctx_ext(ctx).buf[SLOT_MUTUAL_CP]); }
+MPart *mutual_records(nb_ctx *ctx, MutualUser user) {
+    return static_cast<MPart *>(ctx_ext(ctx).buf[mutual_slot(user, kPartCp)]);
+}
 int *mutual_notes(nb_ctx *ctx) { return static_cast<int *>(ctx_ext(ctx).buf[SLOT_MUTUAL_NOTES]); }
 
 nb_status run_mutual(nb_ctx *ctx, const MutualShape &s, const float *x, const float *m, int64_t n, float eps,
                      float *a, float *p, cudaStream_t st) {
+    const MutualUser user = x ? kMutualForce : kMutualFp64;
     cudaError_t e;
     if (x) {
         TimedLaunch t(ctx, 0, st);
         const int64_t npad = mutual_npad(s, n);
         e = launch_with_pdl(mutual_pack_f32_kernel, dim3((unsigned)mutual_pack_blocks(npad)),
-                            dim3(kMutualPackThreads), 0, st, x, m, n, npad, mutual_records(ctx), eps, mutual_notes(ctx));
+                            dim3(kMutualPackThreads), 0, st, x, m, n, npad, mutual_records(ctx, user), eps, mutual_notes(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "pack kernel launch");
     }
     ExtState &es = ctx_ext(ctx);
     const Triangle T = triangle(s, n);
     MutualArgs A{};
-    A.cp = mutual_records(ctx);
-    A.pi = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PI]);
-    A.pj = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PJ]);
-    A.row_first = static_cast<int *>(es.buf[SLOT_MUTUAL_ROWS]);
+    auto part = [&](MutualPart k) { return es.buf[mutual_slot(user, k)]; };
+    A.cp = mutual_records(ctx, user);
+    A.pi = static_cast<float4 *>(part(kPartPi));
+    A.pj = static_cast<float4 *>(part(kPartPj));
+    A.row_first = static_cast<int *>(part(kPartRows));
     A.row_last = A.row_first + T.nib;
     A.notes = mutual_notes(ctx);
     A.weights = mutual_notes(ctx) + 1;
@@ -547,10 +550,10 @@ nb_status run_mutual(nb_ctx *ctx, const MutualShape &s, const float *x, const fl
     A.fault_unit = ctx_fault_unit(ctx);
     A.wait_ns = ctx_wait_ns(ctx);
     A.npad = mutual_npad(s, n);
-    A.pi_len = (int64_t)(es.cap[SLOT_MUTUAL_PI] / sizeof(float4));
-    A.pj_len = (int64_t)(es.cap[SLOT_MUTUAL_PJ] / sizeof(float4));
+    A.pi_len = (int64_t)(es.cap[mutual_slot(user, kPartPi)] / sizeof(float4));
+    A.pj_len = (int64_t)(es.cap[mutual_slot(user, kPartPj)] / sizeof(float4));
     MutualOut O{};
-    O.state = static_cast<float4 *>(es.buf[SLOT_MUTUAL_STATE]);
+    O.state = static_cast<float4 *>(part(kPartState));
     O.n = n;
     O.ib = s.ib;
     O.jt = s.jt;

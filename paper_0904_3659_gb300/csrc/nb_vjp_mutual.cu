@@ -526,7 +526,6 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     const Triangle T{(n + s.jt - 1) / s.jt, (n + s.ib - 1) / s.ib, s.ib / s.jt};
     const int64_t most = (int64_t)(kMutualPartialBytes / (2 * sizeof(float4))) / s.jt;  // tiles per panel
 
-    // Scratch, shared with the mutual force kernels (calls on a context run in order).
     int64_t pj = 1, rows = 1;
     bool panels = false;
     for (int64_t r0 = 0; r0 < T.nib;) {
@@ -537,23 +536,26 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
         r0 = r1;
     }
     ExtState &es = ctx_ext(ctx);
-    auto need = [&](int k, size_t bytes) { return ensure_buffer(&es.buf[k], &es.cap[k], bytes); };
-    cudaError_t e = need(SLOT_MUTUAL_CP, (size_t)npad * kVmRecords * sizeof(float4));
-    if (e == cudaSuccess) e = need(SLOT_MUTUAL_PI, (size_t)(resident + rows) * 4 * s.ib * sizeof(float4));
-    if (e == cudaSuccess) e = need(SLOT_MUTUAL_PJ, (size_t)pj * sizeof(float4));
-    if (e == cudaSuccess) e = need(SLOT_MUTUAL_ROWS, (size_t)2 * T.nib * sizeof(int));
-    if (e == cudaSuccess && panels) e = need(SLOT_MUTUAL_STATE, (size_t)n * 4 * sizeof(float4));
+    auto slot = [](MutualPart part) { return mutual_slot(kMutualVjp, part); };
+    auto need = [&](MutualPart part, size_t bytes) {
+        return ensure_buffer(&es.buf[slot(part)], &es.cap[slot(part)], bytes);
+    };
+    cudaError_t e = need(kPartCp, (size_t)npad * kVmRecords * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartPi, (size_t)(resident + rows) * 4 * s.ib * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartPj, (size_t)pj * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartRows, (size_t)2 * T.nib * sizeof(int));
+    if (e == cudaSuccess && panels) e = need(kPartState, (size_t)n * 4 * sizeof(float4));
     if (e != cudaSuccess) {
         if (e == cudaErrorMemoryAllocation) es.vjp_mutual_max_n = std::min(es.vjp_mutual_max_n, n - 1);
         return cuda_fail(ctx, e, "scratch allocation (mutual vjp)");
     }
 
     VmArgs A{};
-    float4 *cp = static_cast<float4 *>(es.buf[SLOT_MUTUAL_CP]);
+    float4 *cp = static_cast<float4 *>(es.buf[slot(kPartCp)]);
     A.cp = cp;
-    A.pi = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PI]);
-    A.pj = static_cast<float4 *>(es.buf[SLOT_MUTUAL_PJ]);
-    A.row_first = static_cast<int *>(es.buf[SLOT_MUTUAL_ROWS]);
+    A.pi = static_cast<float4 *>(es.buf[slot(kPartPi)]);
+    A.pj = static_cast<float4 *>(es.buf[slot(kPartPj)]);
+    A.row_first = static_cast<int *>(es.buf[slot(kPartRows)]);
     A.row_last = A.row_first + T.nib;
     A.err = ctx_err_word(ctx);
     A.njt = T.njt;
@@ -562,9 +564,9 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     A.fault_unit = ctx_fault_unit(ctx);
     A.wait_ns = ctx_wait_ns(ctx);
     A.npad = npad;
-    A.pi_len = (int64_t)(es.cap[SLOT_MUTUAL_PI] / sizeof(float4));
-    A.pj_len = (int64_t)(es.cap[SLOT_MUTUAL_PJ] / sizeof(float4));
-    VmOut O{gx,   gm,   state ? *state : VjpState{}, static_cast<float4 *>(es.buf[SLOT_MUTUAL_STATE]), n, s.ib,
+    A.pi_len = (int64_t)(es.cap[slot(kPartPi)] / sizeof(float4));
+    A.pj_len = (int64_t)(es.cap[slot(kPartPj)] / sizeof(float4));
+    VmOut O{gx,   gm,   state ? *state : VjpState{}, static_cast<float4 *>(es.buf[slot(kPartState)]), n, s.ib,
             s.jt, 0};
 
     const dim3 pack((unsigned)((npad + 127) / 128));
