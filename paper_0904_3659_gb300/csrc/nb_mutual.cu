@@ -487,22 +487,14 @@ nb_status mutual_reserve(nb_ctx *ctx, const MutualShape &s, int64_t n, MutualUse
         return ensure_buffer(&es.buf[k], &es.cap[k], bytes);
     };
     const Triangle T = triangle(s, n);
-    int64_t pj = 1, rows = 1;
-    bool panels = false;
-    for (int64_t r0 = 0; r0 < T.nib;) {
-        const int64_t r1 = T.panel_end(r0, panel_tiles(s));
-        pj = std::max(pj, T.tiles(r0, r1) * s.jt);
-        rows = std::max(rows, r1 - r0);
-        panels = panels || r1 < T.nib;
-        r0 = r1;
-    }
-    const int64_t pi = (most_resident(ctx, s) + rows) * 2 * s.ib;
+    const TriangleScratch size = triangle_scratch(T, panel_tiles(s));
+    const int64_t pi = (most_resident(ctx, s) + size.rows) * 2 * s.ib, pj = size.tiles * s.jt;
     const size_t records = s.hl ? kHLRecords : 1;
     cudaError_t e = need(kPartCp, (size_t)mutual_npad(s, n) * records * sizeof(MPart));
     if (e == cudaSuccess) e = need(kPartPi, (size_t)pi * sizeof(float4));
     if (e == cudaSuccess) e = need(kPartPj, (size_t)pj * sizeof(float4));
     if (e == cudaSuccess) e = need(kPartRows, (size_t)2 * T.nib * sizeof(int));
-    if (e == cudaSuccess && panels) e = need(kPartState, (size_t)n * 2 * sizeof(float4));
+    if (e == cudaSuccess && size.panels) e = need(kPartState, (size_t)n * 2 * sizeof(float4));
     if (e == cudaSuccess && !es.buf[SLOT_MUTUAL_NOTES]) {
         e = ensure_buffer(&es.buf[SLOT_MUTUAL_NOTES], &es.cap[SLOT_MUTUAL_NOTES], 2 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(es.buf[SLOT_MUTUAL_NOTES], 0, 2 * sizeof(int));

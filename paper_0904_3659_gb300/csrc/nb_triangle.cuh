@@ -52,6 +52,21 @@ inline int triangle_grid(int64_t tiles, int resident) {
     return (int)((tiles + each - 1) / each);
 }
 
+// Scratch for the triangle in panels of at most `most` tiles: tiles of a panel, rows of
+// one, and whether there are several. It is enough for every smaller triangle of the
+// same blocks too: one in a single panel may have more tiles or rows than the panels of
+// a larger one have.
+struct TriangleScratch {
+    int64_t tiles, rows;
+    bool panels;
+};
+inline TriangleScratch triangle_scratch(const Triangle &T, int64_t most) {
+    if (T.tiles(0, T.nib) <= most) return {T.tiles(0, T.nib), T.nib, false};
+    int64_t rows = 1;  // the most whose tiles, those of the end of a triangle, can be `most`
+    while (T.tpb * (rows * (rows + 1) / 2) + rows + 1 <= most) ++rows;
+    return {most > T.njt ? most : T.njt, rows, T.nib > 1};
+}
+
 // Whether, inside an i-block, warp `w` of WARPS (each with G groups) meets the
 // group `o`, counted from its own first group, for both sides: those of the
 // next warp, and two of the warps those of the warp after that (the other two

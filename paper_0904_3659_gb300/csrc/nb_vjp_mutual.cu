@@ -526,25 +526,17 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     const Triangle T{(n + s.jt - 1) / s.jt, (n + s.ib - 1) / s.ib, s.ib / s.jt};
     const int64_t most = (int64_t)(kMutualPartialBytes / (2 * sizeof(float4))) / s.jt;  // tiles per panel
 
-    int64_t pj = 1, rows = 1;
-    bool panels = false;
-    for (int64_t r0 = 0; r0 < T.nib;) {
-        const int64_t r1 = T.panel_end(r0, most);
-        pj = std::max(pj, T.tiles(r0, r1) * s.jt * 2);
-        rows = std::max(rows, r1 - r0);
-        panels = panels || r1 < T.nib;
-        r0 = r1;
-    }
+    const TriangleScratch sizes = triangle_scratch(T, most);
     ExtState &es = ctx_ext(ctx);
     auto slot = [](MutualPart part) { return mutual_slot(kMutualVjp, part); };
     auto need = [&](MutualPart part, size_t bytes) {
         return ensure_buffer(&es.buf[slot(part)], &es.cap[slot(part)], bytes);
     };
     cudaError_t e = need(kPartCp, (size_t)npad * kVmRecords * sizeof(float4));
-    if (e == cudaSuccess) e = need(kPartPi, (size_t)(resident + rows) * 4 * s.ib * sizeof(float4));
-    if (e == cudaSuccess) e = need(kPartPj, (size_t)pj * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartPi, (size_t)(resident + sizes.rows) * 4 * s.ib * sizeof(float4));
+    if (e == cudaSuccess) e = need(kPartPj, (size_t)sizes.tiles * s.jt * 2 * sizeof(float4));
     if (e == cudaSuccess) e = need(kPartRows, (size_t)2 * T.nib * sizeof(int));
-    if (e == cudaSuccess && panels) e = need(kPartState, (size_t)n * 4 * sizeof(float4));
+    if (e == cudaSuccess && sizes.panels) e = need(kPartState, (size_t)n * 4 * sizeof(float4));
     if (e != cudaSuccess) {
         if (e == cudaErrorMemoryAllocation) es.vjp_mutual_max_n = std::min(es.vjp_mutual_max_n, n - 1);
         return cuda_fail(ctx, e, "scratch allocation (mutual vjp)");

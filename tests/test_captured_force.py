@@ -47,3 +47,21 @@ def test_replay_after_calls_with_larger_scratch(nb, mode):
         graph.replay()
         nb.nb_synchronize(ctx)
         assert torch.equal(a.cpu(), want[0]) and torch.equal(p.cpu(), want[1])
+
+
+def test_reserved_scratch_serves_smaller_calls(nb):
+    # 371000 particles run in two panels of rows, 370000 in one that has more rows than
+    # either: after nb_reserve for the former, the latter allocates nothing.
+    import torch
+    n, small = 371000, 370000
+    x = torch.randn(n, 3, device="cuda")
+    m, a, p = torch.ones(n, device="cuda"), torch.empty((n, 3), device="cuda"), torch.empty(n, device="cuda")
+    with nb.Context(0) as ctx:
+        nb.nb_reserve(ctx, n, 0)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):  # an allocation here is an error
+            nb.nb_force(ctx, x, m, small, 0.01, a, p, 0)
+        graph.replay()
+        nb.nb_synchronize(ctx)
+        assert torch.isfinite(a[:small]).all() and torch.isfinite(p[:small]).all()
