@@ -6,14 +6,17 @@
 // For a pair (i, l), r = x_i - x_l, y = (|r|^2 + eps^2)^{-1/2}, with the scalar
 // products s_i = r.ga_i and s_l = r.ga_l, the coefficient of r is the same for
 // both particles:
-//   c = y^3 [ y^2 (3 m_i s_l - 3 m_l s_i) - (gp_i m_l + m_i gp_l) ]
+//   c = 3 y^3 [ m_i (y^2 s_l - gp_l / 3) - m_l (y^2 s_i + gp_i / 3) ]
 //   R_i += c r         R_l -= c r
 //   S_i += m_l y^3     S_l += m_i y^3
 //   V_i += y^3 ga_l    V_l += y^3 ga_i
 //   G_i += gp_l y - s_l y^3     G_l += gp_i y + s_i y^3
-// and gx = R + ga S - m V, gm = G. 38 FP32 operations and one reciprocal square
+// and gx = R + ga S - m V, gm = G. 37 FP32 operations and one reciprocal square
 // root per unordered pair (34 without gp), against 56 (52) when each ordered pair
-// is evaluated by itself.
+// is evaluated by itself. The masses enter last: y^2 s is of the order of the gradient
+// over a distance, whereas m s overflows FP32 in units of metres and kilograms. The
+// records hold gp / 3 and the factor 3 of c is the combine's. (Without gp the direct
+// kernel forms m s too, c = y^3 y^2 (3 m_i s_l - 3 m_l s_i), and so does this one.)
 #include <algorithm>
 
 #include "nb_device.cuh"
@@ -24,7 +27,7 @@
 namespace nbk {
 using namespace nbdev;
 
-// One particle: (-x, -y, -z, m), (ga_x, ga_y, ga_z, gp). Padding is all zero:
+// One particle: (-x, -y, -z, m), (ga_x, ga_y, ga_z, gp / 3). Padding is all zero:
 // without m, ga and gp a particle adds nothing to others.
 constexpr int kVmRecords = 2;
 
@@ -37,7 +40,7 @@ __global__ void vjp_mutual_pack_kernel(const float *__restrict__ x, const float 
     float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
     if (i < n) {
         u = make_float4(-x[3 * i], -x[3 * i + 1], -x[3 * i + 2], m[i]);
-        v = make_float4(ga[3 * i], ga[3 * i + 1], ga[3 * i + 2], gp ? gp[i] : 0.f);
+        v = make_float4(ga[3 * i], ga[3 * i + 1], ga[3 * i + 2], gp ? __fdiv_rn(gp[i], 3.f) : 0.f);
     }
     cp[kVmRecords * i] = u;
     cp[kVmRecords * i + 1] = v;
@@ -85,6 +88,7 @@ struct VmOut {
     float4 *state;         // [n][4] sums and carries between panels
     int64_t n;
     int ib, jt, last;
+    float r_factor;        // of the sums of R
 };
 
 // The i-particles of a thread: P packed pairs.
@@ -94,7 +98,7 @@ struct VmI {
 };
 
 // One half of a packed pair against one l; a: the sums of i, b: those of l.
-// Eight sums, and with GP a ninth: the two parts of G, sum s y^3 and sum gp y, stay
+// Eight sums, and with GP a ninth: the two parts of G, sum s y^3 and sum (gp / 3) y, stay
 // apart over a run of additions, because each addition to the larger rounds
 // (relative error of gm against FP64, N = 8192: 3.2e-7 in one sum, 2.3e-7 in two, 2.4e-7
 // the direct kernel).
@@ -107,10 +111,9 @@ __device__ __forceinline__ void vm_pair(float dx, float dy, float dz, float y, f
                                         float m3l, float *(&a)[kVmSums<GP>], float (&b)[kVmSums<GP>]) {
     const float si = __fmaf_rn(dz, giz, __fmaf_rn(dy, giy, __fmul_rn(dx, gix)));
     const float sl = __fmaf_rn(dz, g.z, __fmaf_rn(dy, g.y, __fmul_rn(dx, g.x)));
-    const float A = __fmaf_rn(-m3l, si, __fmul_rn(m3i, sl));
-    float t;
-    if (GP) t = __fmaf_rn(y2, A, -__fmaf_rn(mi, g.w, __fmul_rn(gpi, h.w)));
-    else t = __fmul_rn(y2, A);
+    float t;  // GP: without the factor 3
+    if (GP) t = __fmaf_rn(-h.w, __fmaf_rn(y2, si, gpi), __fmul_rn(mi, __fmaf_rn(y2, sl, -g.w)));
+    else t = __fmul_rn(y2, __fmaf_rn(-m3l, si, __fmul_rn(m3i, sl)));
     const float c = __fmul_rn(y3, t);
     *a[0] = __fmaf_rn(c, dx, *a[0]);
     *a[1] = __fmaf_rn(c, dy, *a[1]);
@@ -144,7 +147,7 @@ __device__ __forceinline__ void vm_group(const float4 *__restrict__ T, int lane,
     for (int t = 0; t < 32; ++t) {
         const int k = BOTH ? lane ^ t : t;
         const float4 h = T[kVmRecords * k], g = T[kVmRecords * k + 1];
-        const float m3l = __fmul_rn(3.f, h.w);
+        const float m3l = GP ? 0.f : __fmul_rn(3.f, h.w);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             const float2 dx = make_float2(__fadd_rn(I.x[q].x, h.x), __fadd_rn(I.x[q].y, h.x));
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) vjp_mutual_kernel(const VmAr
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             if constexpr (GP) {
-                acc[q][7] = add2(acc[q][7], acc[q][8]);
+                acc[q][7] = fma2(splat2(3.f), acc[q][8], acc[q][7]);
                 acc[q][8] = zero2;
             }
 #pragma unroll
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) vjp_mutual_kernel(const VmAr
             else if (o >= 0 && o < 2 * P)
                 vm_group<P, 1, GP, false>(G, lane, o, I, acc, ja, eps2);
             dst[64 * g] = make_float4(ja[0], ja[1], ja[2], ja[3]);
-            if constexpr (GP) ja[7] = __fadd_rn(ja[7], ja[8]);
+            if constexpr (GP) ja[7] = __fmaf_rn(3.f, ja[8], ja[7]);
             dst[64 * g + 1] = make_float4(ja[4], ja[5], ja[6], ja[7]);
         }
         if (++held == FOLD) fold();
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(32 * kVmCombineWarps) vjp_mutual_combine_kerne
     const float Sm = __fadd_rn(S[3], E[3]), gv[3] = {g.x, g.y, g.z};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {  // gx = R + ga S - m V
-        const float gx = __fadd_rn(__fadd_rn(S[c], E[c]),
+        const float gx = __fmaf_rn(O.r_factor, __fadd_rn(S[c], E[c]),
                                    __fmaf_rn(-u.w, __fadd_rn(S[4 + c], E[4 + c]), __fmul_rn(gv[c], Sm)));
         if (!O.adj.lx) {
             O.gx[3 * i + c] = gx;
@@ -522,6 +525,7 @@ static const VmShape kVmShapes[kVjpMutualSizes][2] = {
     {NB_VM(4, 2, 128, 3, 8, 3, false), NB_VM(4, 2, 128, 3, 8, 3, true)},
 };
 #undef NB_VM
+constexpr size_t kSmSharedBytes = 228 * 1024;
 
 }  // namespace nbk
 
@@ -574,7 +578,7 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     A.pi_len = (int64_t)(es.cap[slot(kPartPi)] / sizeof(float4));
     A.pj_len = (int64_t)(es.cap[slot(kPartPj)] / sizeof(float4));
     VmOut O{gx,   gm,   state ? *state : VjpState{}, static_cast<float4 *>(es.buf[slot(kPartState)]), n, s.ib,
-            s.jt, 0};
+            s.jt, 0,    gp ? 3.f : 1.f};
 
     const dim3 pack((unsigned)((npad + 127) / 128));
     e = state ? launch_with_pdl(vjp_mutual_pack_state_kernel, pack, dim3(128), 0, st, *state, m, n, npad, cp)
@@ -586,9 +590,20 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
         A.r1 = r1;
         A.tiles = T.tiles(r0, r1);
         A.grid = triangle_grid(A.tiles, resident);
+        // A grid that leaves places free asks for as much shared memory as keeps more
+        // CTAs than needed off an SM: the places go to whichever SMs the pack has left,
+        // and one with three CTAs takes as long as three (with gp, N = 4096, 288 CTAs for
+        // 456 places: 33.3 us without, 27.1 with).
+        const int sms = ctx_sm_count(ctx), per_sm = (A.grid + sms - 1) / sms;
+        size_t smem = s.smem;
+        if (per_sm * sms < resident) {
+            smem = std::max(smem, kSmSharedBytes / (per_sm + 1));
+            e = cudaFuncSetAttribute(s.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "vjp shared memory");
+        }
         {
             TimedLaunch t(ctx, 5, st);
-            e = s.launch(A, s.smem, st);
+            e = s.launch(A, smem, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "vjp kernel launch");
         O.last = r1 == T.nib;
