@@ -155,6 +155,7 @@ struct MutualShape {
 // weights, the same with a kernel for each, 128-particle tiles with the latter.
 enum MutualSize : int { kMutualSmall = 0, kMutualMid = 1, kMutualLarge = 2, kMutualSizes = 3 };
 constexpr int kVjpMutualSizes = 2;  // of the VJP's mutual shapes: 32- and 128-particle j-tiles
+constexpr int64_t kVjpMutualNoGpN = 17 << 10;  // without gp 32 again from here (nb_vjp.cu)
 const MutualShape &mutual_shape(int size, bool pot, bool hl);
 // Bound on the j-side sums held at once (a panel of one row may exceed it).
 constexpr size_t kMutualPartialBytes = size_t(1) << 30;

@@ -526,7 +526,6 @@ constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
 // FP32 operation fewer, 1-3% slower).
 constexpr int kVjpMutualSmall = 21, kVjpMutualLarge = 22;
 constexpr int64_t kVjpMutualLargeN = 10240;
-constexpr int64_t kVjpMutualNoGpN = 17 << 10;
 constexpr int kVjpSmall = 17, kVjpLarge = 18, kVjpNoGpSmall = 19, kVjpNoGpLarge = 2;
 
 const VjpVariant &vjp_variant(nb_ctx *ctx, int64_t n, bool with_gp) {

@@ -139,56 +139,75 @@ __device__ __forceinline__ void vm_pair(float dx, float dy, float dz, float y, f
 
 // 32 particles T[2k], T[2k + 1] against the warp's i-particles (BOTH: for both
 // sides, lane l meeting particle l ^ t at step t; else for the i-side alone, all
-// lanes meeting particle t, and slot `self` of lane l leaving out particle l).
-template <int P, int UNR, bool GP, bool BOTH>
+// lanes meeting particle t, and slot `self` of lane l leaving out particle l). The
+// sums of l are taken in runs of RUN steps, 2 P RUN terms, whose totals travel apart.
+template <int P, int UNR, bool GP, bool BOTH, int RUN>
 __device__ __forceinline__ void vm_group(const float4 *__restrict__ T, int lane, int self, const VmI<P> &I,
                                          float2 (&acc)[P][kVmSums<GP>], float (&b)[kVmSums<GP>], const float2 eps2) {
+    float bt[kVmSums<GP>] = {};
+#pragma unroll 1
+    for (int t0 = 0; t0 < 32; t0 += RUN) {
 #pragma unroll UNR
-    for (int t = 0; t < 32; ++t) {
-        const int k = BOTH ? lane ^ t : t;
-        const float4 h = T[kVmRecords * k], g = T[kVmRecords * k + 1];
-        const float m3l = GP ? 0.f : __fmul_rn(3.f, h.w);
+        for (int t1 = 0; t1 < RUN; ++t1) {
+            const int t = t0 + t1;
+            const int k = BOTH ? lane ^ t : t;
+            const float4 h = T[kVmRecords * k], g = T[kVmRecords * k + 1];
+            const float m3l = GP ? 0.f : __fmul_rn(3.f, h.w);
 #pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const float2 dx = make_float2(__fadd_rn(I.x[q].x, h.x), __fadd_rn(I.x[q].y, h.x));
-            const float2 dy = make_float2(__fadd_rn(I.y[q].x, h.y), __fadd_rn(I.y[q].y, h.y));
-            const float2 dz = make_float2(__fadd_rn(I.z[q].x, h.z), __fadd_rn(I.z[q].y, h.z));
-            float2 s = fma2(dx, dx, eps2);
-            s = fma2(dy, dy, s);
-            s = fma2(dz, dz, s);
-            float2 y = make_float2(rsqrt_sfu(s.x), rsqrt_sfu(s.y));
-            if (!BOTH) {
-                if (self == 2 * q && t == lane) y.x = 0.f;
-                if (self == 2 * q + 1 && t == lane) y.y = 0.f;
+            for (int q = 0; q < P; ++q) {
+                const float2 dx = make_float2(__fadd_rn(I.x[q].x, h.x), __fadd_rn(I.x[q].y, h.x));
+                const float2 dy = make_float2(__fadd_rn(I.y[q].x, h.y), __fadd_rn(I.y[q].y, h.y));
+                const float2 dz = make_float2(__fadd_rn(I.z[q].x, h.z), __fadd_rn(I.z[q].y, h.z));
+                float2 s = fma2(dx, dx, eps2);
+                s = fma2(dy, dy, s);
+                s = fma2(dz, dz, s);
+                float2 y = make_float2(rsqrt_sfu(s.x), rsqrt_sfu(s.y));
+                if (!BOTH) {
+                    if (self == 2 * q && t == lane) y.x = 0.f;
+                    if (self == 2 * q + 1 && t == lane) y.y = 0.f;
+                }
+                const float2 y2 = mul2(y, y), y3 = mul2(y2, y);
+                float *ax[kVmSums<GP>], *ay[kVmSums<GP>];
+#pragma unroll
+                for (int c = 0; c < kVmSums<GP>; ++c) {
+                    ax[c] = &acc[q][c].x;
+                    ay[c] = &acc[q][c].y;
+                }
+                vm_pair<GP, BOTH>(dx.x, dy.x, dz.x, y.x, y2.x, y3.x, I.m[q].x, I.m3[q].x, I.gx[q].x, I.gy[q].x,
+                                  I.gz[q].x, I.gp[q].x, h, g, m3l, ax, b);
+                vm_pair<GP, BOTH>(dx.y, dy.y, dz.y, y.y, y2.y, y3.y, I.m[q].y, I.m3[q].y, I.gx[q].y, I.gy[q].y,
+                                  I.gz[q].y, I.gp[q].y, h, g, m3l, ay, b);
             }
-            const float2 y2 = mul2(y, y), y3 = mul2(y2, y);
-            float *ax[kVmSums<GP>], *ay[kVmSums<GP>];
+            if (BOTH) {
+                const int move = (t ^ (t + 1)) & 31;
+#pragma unroll
+                for (int c = 0; c < kVmSums<GP>; ++c) b[c] = __shfl_xor_sync(0xffffffffu, b[c], move);
+            }
+        }
+            if (RUN < 32) {
+            const int move = (t0 ^ (t0 + RUN)) & 31;
 #pragma unroll
             for (int c = 0; c < kVmSums<GP>; ++c) {
-                ax[c] = &acc[q][c].x;
-                ay[c] = &acc[q][c].y;
+                bt[c] = __fadd_rn(__shfl_xor_sync(0xffffffffu, bt[c], move), b[c]);
+                b[c] = 0.f;
             }
-            vm_pair<GP, BOTH>(dx.x, dy.x, dz.x, y.x, y2.x, y3.x, I.m[q].x, I.m3[q].x, I.gx[q].x, I.gy[q].x,
-                              I.gz[q].x, I.gp[q].x, h, g, m3l, ax, b);
-            vm_pair<GP, BOTH>(dx.y, dy.y, dz.y, y.y, y2.y, y3.y, I.m[q].y, I.m3[q].y, I.gx[q].y, I.gy[q].y,
-                              I.gz[q].y, I.gp[q].y, h, g, m3l, ay, b);
-        }
-        if (BOTH) {
-            const int move = (t ^ (t + 1)) & 31;
-#pragma unroll
-            for (int c = 0; c < kVmSums<GP>; ++c) b[c] = __shfl_xor_sync(0xffffffffu, b[c], move);
         }
     }
+    if (RUN < 32)
+#pragma unroll
+        for (int c = 0; c < kVmSums<GP>; ++c) b[c] = bt[c];
 }
 
-// As mutual_kernel (nb_mutual.cu), with two records and eight sums per particle.
-template <int WARPS, int P, int JT, int STAGES, int UNR, int MINB, bool GP>
+// As mutual_kernel (nb_mutual.cu), with two records and eight sums per particle. FOLD:
+// groups of 32 l between two compensated additions.
+template <int WARPS, int P, int JT, int STAGES, int UNR, int MINB, bool GP, int RUN, int FOLD>
 __global__ void __launch_bounds__(WARPS * 32, MINB) vjp_mutual_kernel(const VmArgs A) {
     constexpr int THREADS = WARPS * 32;
     constexpr int IB = 64 * P * WARPS;
     constexpr int TPB = IB / JT;
     constexpr uint32_t TILE_BYTES = JT * kVmRecords * sizeof(float4);
-    constexpr int FOLD = JT >= 128 ? 1 : 128 / JT;  // tiles between two compensated additions
+    constexpr bool FOLD_IN_TILE = FOLD * 32 < JT;
+    static_assert(FOLD_IN_TILE || FOLD * 32 % JT == 0, "a fold ends a group or a tile");
     static_assert(IB % JT == 0 && JT % 32 == 0, "whole tiles per block, whole groups per tile");
 
     // Shared memory: [STAGES tiles][2 x WARPS x JT x 2 j-side sums][running sums,
@@ -348,14 +367,15 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) vjp_mutual_kernel(const VmAr
             float ja[kVmSums<GP>] = {};
             const int o = (int)own + g;
             if (t >= (b + 1) * TPB || met<WARPS, 2 * P>(o, warp, b & 1))
-                vm_group<P, UNR, GP, true>(G, lane, -1, I, acc, ja, eps2);
+                vm_group<P, UNR, GP, true, RUN>(G, lane, -1, I, acc, ja, eps2);
             else if (o >= 0 && o < 2 * P)
-                vm_group<P, 1, GP, false>(G, lane, o, I, acc, ja, eps2);
+                vm_group<P, 1, GP, false, 32>(G, lane, o, I, acc, ja, eps2);
             dst[64 * g] = make_float4(ja[0], ja[1], ja[2], ja[3]);
             if constexpr (GP) ja[7] = __fmaf_rn(3.f, ja[8], ja[7]);
             dst[64 * g + 1] = make_float4(ja[4], ja[5], ja[6], ja[7]);
+            if (FOLD_IN_TILE && (g + 1) % FOLD == 0) fold();
         }
-        if (++held == FOLD) fold();
+        if (!FOLD_IN_TILE && ++held == FOLD * 32 / JT) fold();
         if (++t == A.njt) {
             if (tid == 0) A.row_last[b] = (int)c;
             ++b;
@@ -498,9 +518,10 @@ constexpr size_t vm_smem() {
            (size_t)16 * P * WARPS * 32 * sizeof(float2) + (size_t)STAGES * (sizeof(uint64_t) + sizeof(int));
 }
 
-template <int W, int P, int J, int S, int U, int M, bool GP>
+template <int W, int P, int J, int S, int U, int M, bool GP, int RUN, int FOLD>
 static cudaError_t launch_vm(const VmArgs &a, size_t smem, cudaStream_t st) {
-    return launch_with_pdl(vjp_mutual_kernel<W, P, J, S, U, M, GP>, dim3((unsigned)a.grid), dim3(W * 32), smem, st, a);
+    return launch_with_pdl(vjp_mutual_kernel<W, P, J, S, U, M, GP, RUN, FOLD>, dim3((unsigned)a.grid), dim3(W * 32), smem,
+                           st, a);
 }
 
 struct VmShape {
@@ -510,9 +531,9 @@ struct VmShape {
     cudaError_t (*launch)(const VmArgs &, size_t, cudaStream_t);
 };
 
-#define NB_VM(W, P, J, S, U, M, GP)                                                           \
-    {W * 32, 64 * P * W, J, (const void *)vjp_mutual_kernel<W, P, J, S, U, M, GP>, vm_smem<W, P, J, S>(), \
-     launch_vm<W, P, J, S, U, M, GP>}
+#define NB_VM(J, U, GP, RUN, FOLD)                                                             \
+    {128, 512, J, (const void *)vjp_mutual_kernel<4, 2, J, 3, U, 3, GP, RUN, FOLD>, vm_smem<4, 2, J, 3>(), \
+     launch_vm<4, 2, J, 3, U, 3, GP, RUN, FOLD>}
 
 // [size][without, with an upstream gradient on p]. Like the force's, register
 // reads bound these: N = 65536 runs at 1299 G-pairs/s with gp and 1441 without it
@@ -520,10 +541,19 @@ struct VmShape {
 // (1228 / 1363) or 2 (1147 / 1283) with 128-particle tiles, four CTAs per SM (1159
 // / 1256), 8 i-particles per thread at two CTAs (1277 / 1496, but 1043 / 1217
 // against 1188 / 1333 at N = 16384).
+// Runs. Without gp the direct kernels sum 64 or 128 l at a time and gm has nothing but
+// sum s y^3 in it. With 128 terms to a run on both sides its error against FP64 was 1.04
+// to 1.19 times theirs from N = 6000 to 16384; as below it is 0.83 to 0.96 (N = 8192
+// 2.3e-7 -> 1.8e-7 and 60.9 -> 63.8 us, N = 16384 2.5e-7 -> 1.9e-7 and 197 -> 204 us;
+// runs of 16 steps there 209 us). With gp 128 terms are no more than the direct
+// kernel's.
 static const VmShape kVmShapes[kVjpMutualSizes][2] = {
-    {NB_VM(4, 2, 32, 3, 4, 3, false), NB_VM(4, 2, 32, 3, 4, 3, true)},
-    {NB_VM(4, 2, 128, 3, 8, 3, false), NB_VM(4, 2, 128, 3, 8, 3, true)},
+    {NB_VM(32, 4, false, 16, 2), NB_VM(32, 4, true, 32, 4)},
+    {NB_VM(128, 8, false, 8, 2), NB_VM(128, 8, true, 32, 4)},
 };
+// The first without gp for the largest n, whose errors the longer runs do not raise
+// above the direct kernels' (N = 20000 0.89 times, 298 us against 309).
+static const VmShape kVmShapeLarge = NB_VM(32, 4, false, 32, 2);
 #undef NB_VM
 constexpr size_t kSmSharedBytes = 228 * 1024;
 
@@ -535,7 +565,7 @@ namespace nbx {
 
 nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, int64_t n, float eps, const float *ga,
                          const float *gp, float *gx, float *gm, cudaStream_t st, const VjpState *state) {
-    const VmShape &s = kVmShapes[size][gp ? 1 : 0];
+    const VmShape &s = size == 0 && !gp && n >= kVjpMutualNoGpN ? kVmShapeLarge : kVmShapes[size][gp ? 1 : 0];
     PairVariant v{};
     v.tile.threads = s.threads;
     v.kernel = s.kernel;

@@ -1,5 +1,6 @@
-"""GPU: the VJP's mutual shapes are no less exact than the direct shape that they stand
-in for (two packed pairs per thread, 128-particle tiles). The errors against FP64 are
+"""GPU: the VJP's mutual shapes are no less exact than the direct shapes that they stand
+in for (with a gradient on p two packed pairs per thread and 128-particle tiles, without
+it one pair and 64-particle tiles). The errors against FP64 are
 2-norms over 1024 particles, root mean squares over six systems; 5% is allowed for
 what is left to chance (both errors are sums of some 10^7 independent roundings, but the
 largest terms, of the closest pairs, count most)."""
@@ -29,11 +30,10 @@ def exact_rows(x, m, eps, ga, gp, rows):
     return torch.cat(gx), torch.cat(gm)
 
 
-@pytest.mark.parametrize("n", [3000, 8192, 16384])
-def test_mass_gradient_with_a_gradient_on_p(nb, ctx, n):
+def compare(nb, ctx, n, with_gp, shape):
     import torch
-    eps, tiles = 1.0 / 64, nb.nb_list_vjp_tiles()
-    direct = [t for t in tiles if (t.threads, t.ipt, t.jtile, t.minblocks, t.release) == (128, 4, 128, 3, 1)]
+    eps = 1.0 / 64
+    direct = [t for t in nb.nb_list_vjp_tiles() if (t.threads, t.ipt, t.jtile, t.minblocks, t.release) == shape]
     assert len(direct) == 1
     error = [0.0, 0.0]  # of the built-in shape, a mutual one, and of the direct one
     assert nb.nb_get_vjp_tile(ctx, n).packed & 64
@@ -41,17 +41,27 @@ def test_mass_gradient_with_a_gradient_on_p(nb, ctx, n):
         x, _, m = workloads.plummer(n, seed=1000 * seed + n)
         rng = np.random.default_rng(seed)
         x, m, ga, gp = (torch.from_numpy(v.astype(np.float32)).cuda()
-                        for v in (x, m, rng.normal(size=(n, 3)), rng.normal(size=n)))
+                        for v in (x, m, rng.normal(size=(n, 3)), with_gp * rng.normal(size=n)))
         rows = workloads.sample_rows(n, 1024, seed)
         _, want = exact_rows(x, m, eps, ga, gp, rows)
         for k, tile in enumerate((None, direct[0])):
             gx, gm = torch.empty_like(x), torch.empty_like(m)
             nb.nb_set_vjp_tile(ctx, tile)
             try:
-                nb.nb_force_vjp(ctx, x, m, n, eps, ga, gp, gx, gm)
+                nb.nb_force_vjp(ctx, x, m, n, eps, ga, gp if with_gp else None, gx, gm)
                 nb.nb_synchronize(ctx)
             finally:
                 nb.nb_set_vjp_tile(ctx, None)
             e = gm[torch.from_numpy(rows).cuda()].double() - want
             error[k] += float(e.norm() / want.norm()) ** 2
     assert error[0] <= 1.05 ** 2 * error[1]
+
+
+@pytest.mark.parametrize("n", [3000, 8192, 16384])
+def test_mass_gradient_with_a_gradient_on_p(nb, ctx, n):
+    compare(nb, ctx, n, True, (128, 4, 128, 3, 1))
+
+
+@pytest.mark.parametrize("n", [6000, 8192, 11000, 16384, 18000])
+def test_mass_gradient_without_a_gradient_on_p(nb, ctx, n):
+    compare(nb, ctx, n, False, (512, 2, 64, 1, 0))
