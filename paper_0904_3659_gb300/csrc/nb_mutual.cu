@@ -63,9 +63,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) mutual_kernel(const MutualAr
     constexpr int RS = HL ? kHLRecords : 1;
     constexpr uint32_t TILE_BYTES = JT * RS * sizeof(MPart);
     constexpr int NC = POT ? 4 : 3;
-    // Tiles between two compensated additions to the running sums: the sums
-    // of at least 256 j-particles, as long as the direct kernels' tiles.
-    constexpr int FOLD = JT >= 256 ? 1 : 256 / JT;
+    // Tiles between two compensated additions to the running sums: 128 j-particles with
+    // 32-particle tiles, the direct kernels' tiles on FP64 state at those n (with 256 the
+    // error of p against FP64 was 1.06 to 1.12 times theirs from N = 12000 to 30000, as it
+    // is 0.94 to 0.99; N = 20000 194.3 -> 194.8 us a step), 256 with larger ones.
+    constexpr int FOLD = JT <= 32 ? 128 / JT : JT >= 256 ? 1 : 256 / JT;
     static_assert(IB % JT == 0 && JT % 32 == 0, "whole tiles per block, whole groups per tile");
     static_assert(TILE_BYTES % 16 == 0, "bulk copies move multiples of 16 bytes");
 
