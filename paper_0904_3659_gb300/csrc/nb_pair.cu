@@ -1344,15 +1344,19 @@ int pair_default_unfused_index(bool comp, int64_t n) {
 constexpr int64_t kClusterMaxN = (int64_t)76 * 128;
 constexpr int64_t kClusterWideMinN = (int64_t)3 << 10;
 constexpr int64_t kFusedMaxN = (int64_t)3 << 13;
-// Mutual shapes from kMutualMinN (equal / unequal masses, plain: N = 10007
+// Mutual shapes from kMutualMinN in plain mode (equal / unequal masses: N = 10007
 // 48.8 / 55.6 us against 53 for the stream-K form, N = 12288 66.7 / 75.8 against
-// 73.8, N = 16384 101 / 115 against 125, N = 65536 1298 / 1454 against 1717 for the
+// 73.8, N = 16384 101 / 112 against 125, N = 65536 1298 / 1454 against 1717 for the
 // packed shapes): one kernel for all forms of the weights below kMutualMidN, one
 // for each from there (N = 20000: 144 / 164 us against 146 / 162; N = 262144
 // 20.0 / 22.9 ms for the latter); 32-particle j-tiles, which split the work more
 // evenly, below kMutualLargeN, 128-particle tiles, with fewer barriers, from
 // there (N = 32768: 351 / 390 us against 360 / 408; N = 49152: 762 / 840 against
-// 745 / 836).
+// 745 / 836). In compensated mode from kMutualMidN only: the stream-K form below
+// compensates every 32 j-particles of a warp, the mutual one every 128 (relative error
+// of a against FP64, equal masses: N = 13312 3.9e-8 against 5.5e-8, N = 20000 3.7e-8
+// against 4.9e-8; with runs of 32 terms on both sides still 1.02 to 1.06 times the
+// former, 5% slower, and slower than it with massless particles up to N = 17000).
 constexpr int64_t kMutualMinN = (int64_t)13 << 10;
 constexpr int64_t kMutualMidN = kFusedMaxN;
 // On two-word positions one kernel per form pays earlier (leap-frog step with the
@@ -1381,9 +1385,9 @@ int pair_default_index(bool comp, int64_t n) {
     return k >= 0 ? k : pair_default_unfused_index(comp, n);
 }
 
-// The built-in mutual shape for n (nb_mutual.cu), or -1 below kMutualMinN.
+// The built-in mutual shape for n (nb_mutual.cu), or -1.
 int pair_mutual_index(bool comp, int64_t n) {
-    if (n < kMutualMinN) return -1;
+    if (n < (comp ? kMutualMidN : kMutualMinN)) return -1;
     const int size = n < kMutualMidN ? kMutualSmall : n < kMutualLargeN ? kMutualMid : kMutualLarge;
     for (int k = 0; k < pair_variant_count(comp); ++k)
         if (pair_variant(comp, k)->mutual == size) return k;
