@@ -284,7 +284,12 @@ __device__ __forceinline__ void self_group(const MPart *__restrict__ T, int lane
     }
 }
 
-// The group functions for the kernel's form of the weights.
+// The group functions for the kernel's form of the weights. With massless particles
+// (kWide) a kAny kernel unrolled once was slower than the direct kernels: nb_force N =
+// 13312 89.4 us and with UNR = 4 85.1 (stream-K form 85.0), N = 16896 135 and 127 (133),
+// 1024 clusters up to 4096 830 and 795; equal masses 1% more. On two-word positions once
+// is fast enough (300 clusters 131 us a step; 145 for the direct kernels), and 4 costs
+// equal masses 1%.
 template <int P, int UNR, bool POT, bool HL, int W>
 __device__ __forceinline__ void run_group(int weights, const MPart *G, int lane, const MutualI<P, HL> &I,
                                           float2 (&acc)[P][4], float (&ja)[4], float2 eps2) {
@@ -295,7 +300,7 @@ __device__ __forceinline__ void run_group(int weights, const MPart *G, int lane,
     else if (weights == kProduct)
         mutual_group<P, UNR, POT, HL, kProduct>(G, lane, I, acc, ja, eps2);
     else
-        mutual_group<P, 1, POT, HL, kWide>(G, lane, I, acc, ja, eps2);
+        mutual_group<P, (HL ? 1 : UNR), POT, HL, kWide>(G, lane, I, acc, ja, eps2);
 }
 
 template <int P, bool POT, bool HL, int W>
