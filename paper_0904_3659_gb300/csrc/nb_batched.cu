@@ -360,10 +360,11 @@ __device__ __forceinline__ void one_sided_group(int weights, const MPart *__rest
             float2 s = fma2(dx, dx, eps2);
             s = fma2(dy, dy, s);
             s = fma2(dz, dz, s);
-            float2 y = make_float2(rsqrt_sfu(s.x), rsqrt_sfu(s.y));
-            if (own == 2 * q) y.x = 0.f;
-            if (own == 2 * q + 1) y.y = 0.f;
-            const float2 f = product ? make_float2(__fmul_rn(I.hm[q].x, hj), __fmul_rn(I.hm[q].y, hj)) : splat2(hj);
+            const float2 y = make_float2(rsqrt_sfu(s.x), rsqrt_sfu(s.y));
+            float2 f = splat2(hj);  // (left out here: an infinite mass times y = 0 would be NaN)
+            if (own == 2 * q) f.x = 0.f;
+            if (own == 2 * q + 1) f.y = 0.f;
+            if (product) f = make_float2(__fmul_rn(I.hm[q].x, f.x), __fmul_rn(I.hm[q].y, f.y));
             const float2 p = mul2(f, y);
             acc[q][3] = add2(acc[q][3], p);
             const float2 w = mul2(p, mul2(y, y));
