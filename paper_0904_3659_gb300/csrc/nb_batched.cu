@@ -340,13 +340,17 @@ __device__ __forceinline__ int cluster_weights(const BmArgs &A, int c, int nt) {
 }
 
 // A group's particles on the first Q pairs of i-slots, for the i-side only; the
-// particles of slot `self` (-1: none) do not meet themselves. One code for every
-// kind of weights, w = (f y) y^2 with f = 1 where all masses are equal, so that the
-// kernel's loops stay in the instruction cache.
-template <int P, int Q, bool HL>
-__device__ __forceinline__ void one_sided_group(int weights, const MPart *__restrict__ T, int lane, int self,
-                                                const MutualI<P, HL> &I, float2 (&acc)[P][4], const float2 eps2) {
-    const bool equal = weights == kEqual, product = weights == kProduct;
+// particles of slot `self` (-1: none) do not meet themselves. w = (f y) y^2 with f = 1
+// where all masses are equal, c m_i m_j (PRODUCT) or m_j. On FP32 records a loop of its
+// own for PRODUCT and packed differences, the broadcast j costing a move per value: 2300
+// clusters of 200 particles 124 -> 112 us a call, 1900 of 256 108 -> 100, 1024 up to 512
+// 60 -> 53. Two-word records take one loop for both, the kernel's loops then staying in
+// the instruction cache (1024 up to 512, unequal masses: 91 us a step, 102 with two),
+// and scalar differences (packed 1 to 2% slower).
+template <int P, int Q, bool HL, bool PRODUCT>
+__device__ __forceinline__ void one_sided_loop(int weights, const MPart *__restrict__ T, int lane, int self,
+                                               const MutualI<P, HL> &I, float2 (&acc)[P][4], const float2 eps2) {
+    const bool equal = weights == kEqual, product = PRODUCT && (!HL || weights == kProduct);
 #pragma unroll 4
     for (int t = 0; t < 32; ++t) {
         const float4 h = T[HL ? 2 * t : t];
@@ -356,7 +360,13 @@ __device__ __forceinline__ void one_sided_group(int weights, const MPart *__rest
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             float2 dx, dy, dz;
-            mutual_diff<P, HL>(I, q, h, l, dx, dy, dz);
+            if constexpr (HL) {
+                mutual_diff<P, HL>(I, q, h, l, dx, dy, dz);
+            } else {
+                dx = add2(I.x[q], splat2(h.x));
+                dy = add2(I.y[q], splat2(h.y));
+                dz = add2(I.z[q], splat2(h.z));
+            }
             float2 s = fma2(dx, dx, eps2);
             s = fma2(dy, dy, s);
             s = fma2(dz, dz, s);
@@ -373,6 +383,13 @@ __device__ __forceinline__ void one_sided_group(int weights, const MPart *__rest
             acc[q][2] = fma2(w, dz, acc[q][2]);
         }
     }
+}
+
+template <int P, int Q, bool HL>
+__device__ __forceinline__ void one_sided_group(int weights, const MPart *__restrict__ T, int lane, int self,
+                                                const MutualI<P, HL> &I, float2 (&acc)[P][4], const float2 eps2) {
+    if (HL || weights == kProduct) one_sided_loop<P, Q, HL, true>(weights, T, lane, self, I, acc, eps2);
+    else one_sided_loop<P, Q, HL, false>(weights, T, lane, self, I, acc, eps2);
 }
 
 struct BmStage {
@@ -393,7 +410,7 @@ struct BmStage {
 // items' ends. 128 particles a block (4 per lane) against 256: half the padding and
 // half the own-block work, twice the j-side sums; 57 against 87 us up to 512, 667
 // against 687 up to 4096. Tiles of 64 against 128: 47 against 55 us up to 512.
-// Twelve warps' worth of registers (126 a lane: 16 resident); 12 items per warp
+// Twelve warps' worth of registers (142 a lane: 14 resident, 148 on two-word records); 12 items per warp
 // against 8: 669 against 678 us, against 4: 702.
 // Against one evaluation per (i, j): 1024 clusters up to 4096 particles 817 -> 685 us
 // (the pair kernel 777 -> 632; 904.8e6 unordered pairs, 66% of the FP32 lanes' issue
