@@ -49,7 +49,8 @@ struct BmArgs {
     BatchSplit *split;     // the batch's
     int max_band;          // blocks per band at most
     int64_t want_items;    // items wanted: kItemsPerWarp per resident warp
-    int *notes;            // [C] what the pack found of a cluster (MutualNote)
+    int *notes;            // [C] what the pack found of a cluster (MutualNote); zero before it
+    int *weights;          // [C] the form of its weights (MutualWeights), from the pair kernel
     MPart *cp;             // [cap_padded][1 or 2]
     float4 *pi;            // [item][kBlock] i-side sums
     float4 *pj;            // j-side sums (batch_pj_entry)
@@ -562,6 +563,7 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
             const int64_t row0 = A.poff[mt.cluster], nc = A.off[mt.cluster + 1] - A.off[mt.cluster];
             const int nt = (int)((A.poff[mt.cluster + 1] - row0) / kBlock), cb = cluster_band(band, nt), s0 = b / cb * cb;
             weights = cluster_weights(A, mt.cluster, nt);
+            if (lane == 0 && b == 0) A.weights[mt.cluster] = weights;
             direct = nt <= kDirectBlocks;
             band_end = min(s0 + cb, nt);
             slots = (int)min((nc - (int64_t)b * kBlock + 31) / 32, (int64_t)(2 * P));
@@ -639,6 +641,9 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
     const int c = B.cluster, b = B.b, nt = B.nt;
     const int64_t row0 = (int64_t)(blockIdx.x - b) * kBlock;
     const int64_t li = (int64_t)b * kBlock + threadIdx.x, o = A.off[c], nc = A.off[c + 1] - o;
+    // For the next evaluation of the call, which has no plan before it.
+    if (threadIdx.x == 0 && b == 0) A.notes[c] = 0;
+    if (threadIdx.x == 0 && blockIdx.x == 0) *A.head = 0;
     if (li >= nc) return;
     float S[4] = {0.f, 0.f, 0.f, 0.f}, E[4] = {0.f, 0.f, 0.f, 0.f};
     constexpr int K = 8;  // loads in flight
@@ -684,7 +689,7 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
         }
     }
     const float hm0 = A.cp[row0 * RS].w;
-    const int weights = cluster_weights(A, c, nt);
+    const int weights = __ldcg(A.weights + c);
     const float hm = A.cp[((int64_t)blockIdx.x * kBlock + threadIdx.x) * RS].w;
     const float f = weights == kProduct ? mutual_scale(hm, hm0, A.eps[c]) : hm0;
     float v[4];
@@ -704,16 +709,11 @@ constexpr size_t bm_smem() {
                         sizeof(int)) + (size_t)2 * 4 * kBatchP * 32 * sizeof(float2);
 }
 
-// Leap-frog pieces that do not pack (the batched pack follows them). The notes and
-// the queue head are cleared as the plan does: the steps after a call's first
-// evaluation run without one.
+// Leap-frog pieces that do not pack (the batched pack follows them).
 __global__ void batch_kick_drift_kernel(double *__restrict__ x, double *__restrict__ v,
                                         const float *__restrict__ a, int64_t n, double dt,
-                                        int kick_back, int *__restrict__ notes, int64_t C, int *__restrict__ head) {
+                                        int kick_back) {
     pdl_wait_then_release();
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += gridDim.x * (int64_t)blockDim.x)
-        notes[c] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *head = 0;
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= 3 * n) return;
     const double h = 0.5 * dt, g = -(double)a[k];
@@ -783,7 +783,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.max_band = small ? 1 : (int)std::min(most, std::max<int64_t>(kMinBand, kPjEntries / (blocks * (kBlock / 2))));
     const int64_t pj = (blocks + 1) * (kBlock / 2 * (A.max_band - 1));
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    // [the plan's key, item count, queue head, split][poff][ibase][planned offsets][notes][padded blocks]
+    // [the plan's key, item count, queue head, split][poff][ibase][planned offsets][notes][weights][padded blocks]
     const size_t b_off = al((size_t)(k.C + 1) * sizeof(int64_t)), b_c = al((size_t)k.C * sizeof(int));
     const size_t b_blk = al((size_t)blocks * sizeof(BmBlock));
     const size_t plan_before = es.cap[SLOT_BATCH_PLAN];
@@ -791,7 +791,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     auto need = [&](int slot, size_t bytes) {
         if (e == cudaSuccess) e = ensure_buffer(&es.buf[slot], &es.cap[slot], bytes);
     };
-    need(SLOT_BATCH_PLAN, 256 + 3 * b_off + b_c + b_blk);
+    need(SLOT_BATCH_PLAN, 256 + 3 * b_off + 2 * b_c + b_blk);
     if (es.cap[SLOT_BATCH_PLAN] != plan_before) es.batch_plan = false;
     need(SLOT_BATCH_ITEMS, (size_t)A.cap_items * sizeof(int4));
     need(SLOT_BATCH_CP, (size_t)A.cap_padded * (k.hl ? kHLRecords : 1) * sizeof(MPart));
@@ -809,7 +809,8 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.ibase = reinterpret_cast<int64_t *>(plan + b_off);
     A.planned_off = reinterpret_cast<int64_t *>(plan + 2 * b_off);
     A.notes = reinterpret_cast<int *>(plan + 3 * b_off);
-    A.block = reinterpret_cast<BmBlock *>(plan + 3 * b_off + b_c);
+    A.weights = reinterpret_cast<int *>(plan + 3 * b_off + b_c);
+    A.block = reinterpret_cast<BmBlock *>(plan + 3 * b_off + 2 * b_c);
     A.items = static_cast<int4 *>(es.buf[SLOT_BATCH_ITEMS]);
     A.cp = static_cast<MPart *>(es.buf[SLOT_BATCH_CP]);
     A.pi = static_cast<float4 *>(es.buf[SLOT_BATCH_PI]);
@@ -836,13 +837,14 @@ nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
     return bm_args(ctx, k, true, out);
 }
 
-// One evaluation. `planned`: this call has made one before, so its plan is there (on
-// FP64 state in compensated mode; 32 steps of 300 clusters 4070 -> 4010 us).
+// One evaluation. `planned`: this call has made one before, so its plan stands and the
+// combine has cleared what a plan clears (300 clusters up to 2048, us a step: plain 91.6 ->
+// 88, compensated 127 -> 125).
 nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource &src, bool planned, float *a, float *p,
                    cudaStream_t st) {
     ExtState &es = ctx_ext(ctx);
     cudaError_t e = cudaSuccess;
-    if (!(planned && k.hl && src.kick)) {
+    if (!planned) {
         A.fresh = !es.batch_plan;
         e = launch_with_pdl(bm_plan_kernel, dim3(1), dim3(kBmPlanThreads), 0, st, A);
         es.batch_plan = e == cudaSuccess;
@@ -855,7 +857,7 @@ nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource 
         double4 *frame = static_cast<double4 *>(es.buf[SLOT_BATCH_FRAME]);
         if (src.kick) {
             e = launch_with_pdl(batch_kick_drift_kernel, dim3((unsigned)((3 * k.n_total + 255) / 256)), dim3(256), 0, st,
-                                src.x64, src.v, src.a, k.n_total, src.dt, src.kick_back, A.notes, k.C, A.head);
+                                src.x64, src.v, src.a, k.n_total, src.dt, src.kick_back);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "leap-frog update launch");
         }
         e = launch_with_pdl(batch_frame_kernel, dim3((unsigned)k.C), dim3(kFrameThreads), 0, st,
