@@ -219,9 +219,12 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode);
  * places) is kept in the context and reused by the next call (batched force or
  * batched leap-frog) while n_clusters, n_total and the values of offsets stay the
  * same, which the device checks on every call; any change makes a new one.
- * Scratch, kept in the context: about 560 MiB, or 290 B per particle if that is
- * more; where it cannot be allocated about 50 B per particle, every pair then
- * being evaluated twice.
+ * Scratch, kept in the context: per block of 128 particles (every cluster is padded to
+ * whole blocks) 4.1 KiB, 6.1 KiB in compensated mode on FP64 state; 52 MiB; and for the
+ * sums of evaluating every pair once 512 MiB, or 248 B for every particle beyond the
+ * 256th of a cluster if that is more (or less, where one cluster of all particles would
+ * need less). Where it cannot be allocated the first alone, every pair then being
+ * evaluated twice.
  */
 nb_status nb_force_batched(nb_ctx *ctx, const float *x, const float *m, const int64_t *offsets,
                            int64_t n_clusters, int64_t n_total, const float *eps,

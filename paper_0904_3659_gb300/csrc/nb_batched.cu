@@ -27,8 +27,6 @@ constexpr int kBmPlanNear = 8192;  // clusters whose first blocks the plan keeps
 // Items per resident warp that the plan aims at: more of them even out the end of
 // the launch, fewer mean fewer partial sums.
 constexpr int kItemsPerWarp = 12;
-// Entries of j-side sums that bands above kMinBand may take (512 MiB).
-constexpr int64_t kPjEntries = (int64_t)32 << 20;
 constexpr int kBatchP = kBlock / 64;  // packed i-pairs per lane
 
 struct BmBlock {  // a padded block
@@ -47,13 +45,14 @@ struct BmArgs {
     int4 *items;           // [cap_items] (cluster, i-block, first and end met tile)
     int *nitems, *head;    // item count and queue head
     BatchSplit *split;     // the batch's
-    int max_band;          // blocks per band at most
+    int64_t *pjbase;       // [C] the cluster's first j-side entry
+    int64_t pj_entries;    // set aside
     int64_t want_items;    // items wanted: kItemsPerWarp per resident warp
     int *notes;            // [C] what the pack found of a cluster (MutualNote); zero before it
     int *weights;          // [C] the form of its weights (MutualWeights), from the pair kernel
     MPart *cp;             // [cap_padded][1 or 2]
     float4 *pi;            // [item][kBlock] i-side sums
-    float4 *pj;            // j-side sums (batch_pj_entry)
+    float4 *pj;            // j-side sums (batch_pj_row)
     int *err;
     uint64_t wait_ns;
     // What the plan in the scratch was made for. fresh: nothing.
@@ -103,7 +102,7 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
     const int t = threadIdx.x;
     for (int64_t c = t; c < P.C; c += kBmPlanThreads) P.notes[c] = 0;
     if (t == 0) *P.head = 0;
-    const BatchKey key{P.C, P.n_total, P.want_items, P.max_band};
+    const BatchKey key{P.C, P.n_total, P.want_items, P.pj_entries};
     const int stands = !P.fresh && same_plan(*P.planned, key);
     int bad = 0, replan = !stands;
     for (int64_t c = t; c < P.C; c += kBmPlanThreads) {
@@ -125,11 +124,11 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
         return;
     }
     auto blocks = [&](int64_t c) { return c < P.C ? (int)(padded_size(P.off[c + 1] - P.off[c]) / kBlock) : 0; };
-    __shared__ int band;  // the longest cluster's blocks, as far as they may be one band
+    __shared__ int longest;  // cluster, in blocks
     __shared__ int near[kBmPlanNear + 1];
-    if (t == 0) band = 1;
-    int longest = 1;
-    int64_t carry = 0, met = 0, nit = 0, total;
+    if (t == 0) longest = 1;
+    int most = 1;
+    int64_t carry = 0, met = 0, nit = 0, pj = 0, total;
     for (int64_t base = 0; base < P.C; base += kBmPlanThreads) {
         const int64_t c = base + t;
         const int nt = blocks(c);
@@ -137,16 +136,33 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
         if (c < P.C) P.poff[c] = ex * kBlock;
         if (c < kBmPlanNear) near[c] = (int)ex;
         carry += total;
-        longest = max(longest, min(nt, P.max_band));
+        most = max(most, nt);
     }
-    for (int d = 16; d > 0; d >>= 1) longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, d));
-    if ((t & 31) == 0) atomicMax(&band, longest);
+    for (int d = 16; d > 0; d >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, d));
+    if ((t & 31) == 0) atomicMax(&longest, most);
     __syncthreads();
+    // The longest band whose j-side sums fit: that of the longest cluster, or by bisection.
+    auto need = [&](int band) {
+        int64_t mine = 0, all;
+        for (int64_t c = t; c < P.C; c += kBmPlanThreads) mine += batch_pj_need(band, blocks(c));
+        bm_scan(mine, &all);
+        return all;
+    };
+    int band = longest;
+    if (need(band) > P.pj_entries) {
+        int lo = 1;  // (needs nothing)
+        while (band - lo > 1) {
+            const int mid = (lo + band) / 2;
+            if (need(mid) <= P.pj_entries) lo = mid;
+            else band = mid;
+        }
+        band = lo;
+    }
     for (int64_t base = 0; base < P.C; base += kBmPlanThreads) {
         bm_scan(batch_met(band, blocks(base + t)), &total);
         met += total;
     }
-    const BatchSplit split = batch_split(band, met, P.want_items);
+    const BatchSplit split = batch_split(band, longest, met, P.want_items);
     if (t == 0) {
         P.poff[P.C] = carry * kBlock;
         *P.split = split;
@@ -157,6 +173,9 @@ __global__ void __launch_bounds__(kBmPlanThreads) bm_plan_kernel(const BmArgs P)
         const int64_t ex = bm_scan(nt > 0 ? split.first(nt, nt) : 0, &total);
         if (c < P.C) P.ibase[c] = nit + ex;
         nit += total;
+        const int64_t px = bm_scan(batch_pj_need(band, nt), &total);
+        if (c < P.C) P.pjbase[c] = pj + px;
+        pj += total;
     }
     const bool ok = carry * kBlock <= P.cap_padded && nit <= P.cap_items;
     __syncthreads();  // poff, ibase, near
@@ -567,7 +586,7 @@ __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
             direct = nt <= kDirectBlocks;
             band_end = min(s0 + cb, nt);
             slots = (int)min((nc - (int64_t)b * kBlock + 31) / 32, (int64_t)(2 * P));
-            pj = A.pj + batch_pj_entry(band, row0, nt, b);
+            pj = A.pj + A.pjbase[mt.cluster] + batch_pj_row(band, nt, b);
             const float hm0 = A.cp[row0 * RS].w;
 #pragma unroll
             for (int q = 0; q < P; ++q) {
@@ -648,7 +667,7 @@ __global__ void __launch_bounds__(kBlock) bm_combine_kernel(const BmArgs A, floa
     float S[4] = {0.f, 0.f, 0.f, 0.f}, E[4] = {0.f, 0.f, 0.f, 0.f};
     constexpr int K = 8;  // loads in flight
     const int cb = cluster_band(split.band, nt), s0 = b / cb * cb, len = min(s0 + cb, nt) - s0;
-    const int64_t pj0 = batch_pj_entry(split.band, row0, nt, s0) + threadIdx.x;
+    const int64_t pj0 = A.pjbase[c] + batch_pj_row(split.band, nt, s0) + threadIdx.x;
     for (int r = s0; r < b; r += K) {
         float4 v[K];
 #pragma unroll
@@ -776,14 +795,14 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.C = k.C;
     A.n_total = k.n_total;
     A.cap_padded = k.n_total + k.C * (int64_t)kBlock;
-    const int64_t blocks = A.cap_padded / kBlock, most = padded_size(k.n_total) / kBlock;
-    A.want_items = small ? blocks : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k.hl));
+    const int64_t blocks = A.cap_padded / kBlock;
+    // small: one item per row and no j-side sums.
+    A.want_items = small ? 1 : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k.hl));
     A.cap_items = blocks + A.want_items + 1;  // at most one per row beyond the number wanted
     if (A.cap_items > INT_MAX || k.C > INT_MAX) return fail(ctx, NB_ERR_ARG, "batch too large for 32-bit work items");
-    A.max_band = small ? 1 : (int)std::min(most, std::max<int64_t>(kMinBand, kPjEntries / (blocks * (kBlock / 2))));
-    const int64_t pj = (blocks + 1) * (kBlock / 2 * (A.max_band - 1));
+    A.pj_entries = small ? 0 : batch_pj_entries(k.C, k.n_total);
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    // [the plan's key, item count, queue head, split][poff][ibase][planned offsets][notes][weights][padded blocks]
+    // [the plan's key, item count, queue head, split][poff][ibase][pjbase][planned offsets][notes][weights][padded blocks]
     const size_t b_off = al((size_t)(k.C + 1) * sizeof(int64_t)), b_c = al((size_t)k.C * sizeof(int));
     const size_t b_blk = al((size_t)blocks * sizeof(BmBlock));
     const size_t plan_before = es.cap[SLOT_BATCH_PLAN];
@@ -791,12 +810,12 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     auto need = [&](int slot, size_t bytes) {
         if (e == cudaSuccess) e = ensure_buffer(&es.buf[slot], &es.cap[slot], bytes);
     };
-    need(SLOT_BATCH_PLAN, 256 + 3 * b_off + 2 * b_c + b_blk);
+    need(SLOT_BATCH_PLAN, 256 + 4 * b_off + 2 * b_c + b_blk);
     if (es.cap[SLOT_BATCH_PLAN] != plan_before) es.batch_plan = false;
     need(SLOT_BATCH_ITEMS, (size_t)A.cap_items * sizeof(int4));
     need(SLOT_BATCH_CP, (size_t)A.cap_padded * (k.hl ? kHLRecords : 1) * sizeof(MPart));
     need(SLOT_BATCH_PI, (size_t)A.cap_items * kBlock * sizeof(float4));
-    need(SLOT_BATCH_PJ, (size_t)pj * sizeof(float4));
+    need(SLOT_BATCH_PJ, (size_t)A.pj_entries * sizeof(float4));
     if (k.hl) need(SLOT_BATCH_FRAME, (size_t)k.C * sizeof(double4));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch allocation (batched)");
     unsigned char *plan = static_cast<unsigned char *>(es.buf[SLOT_BATCH_PLAN]);
@@ -807,10 +826,11 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     plan += 256;
     A.poff = reinterpret_cast<int64_t *>(plan);
     A.ibase = reinterpret_cast<int64_t *>(plan + b_off);
-    A.planned_off = reinterpret_cast<int64_t *>(plan + 2 * b_off);
-    A.notes = reinterpret_cast<int *>(plan + 3 * b_off);
-    A.weights = reinterpret_cast<int *>(plan + 3 * b_off + b_c);
-    A.block = reinterpret_cast<BmBlock *>(plan + 3 * b_off + 2 * b_c);
+    A.pjbase = reinterpret_cast<int64_t *>(plan + 2 * b_off);
+    A.planned_off = reinterpret_cast<int64_t *>(plan + 3 * b_off);
+    A.notes = reinterpret_cast<int *>(plan + 4 * b_off);
+    A.weights = reinterpret_cast<int *>(plan + 4 * b_off + b_c);
+    A.block = reinterpret_cast<BmBlock *>(plan + 4 * b_off + 2 * b_c);
     A.items = static_cast<int4 *>(es.buf[SLOT_BATCH_ITEMS]);
     A.cp = static_cast<MPart *>(es.buf[SLOT_BATCH_CP]);
     A.pi = static_cast<float4 *>(es.buf[SLOT_BATCH_PI]);
@@ -823,9 +843,11 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     return NB_OK;
 }
 
-// Arguments of a call's kernels; allocates the scratch: up to 512 MiB (or 248 B per
-// particle, if that is more) of j-side sums and 60 MB of i-side sums, or, where that
-// cannot be had, no j-side sums (every pair evaluated twice) and 32 B per particle.
+// Arguments of a call's kernels; allocates the scratch: per padded block 2 KiB of
+// records (4 on two-word positions), 2 of i-side sums and 32 bytes; 12 items a warp of
+// i-side sums (52 MiB); the j-side sums (batch_pj_entries: 512 MiB, or 248 B for every
+// particle beyond the 256th of a cluster). Where that cannot be had, the first alone,
+// every pair then being evaluated twice. (10^6 clusters of 32: 5.7 GB.)
 nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
     ExtState &es = ctx_ext(ctx);
     const int64_t size = k.n_total + k.C * (int64_t)kBlock;

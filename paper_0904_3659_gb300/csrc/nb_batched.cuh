@@ -5,9 +5,9 @@
 // on the i-side, held by one warp. In a band of consecutive blocks it meets its own
 // block and those of other bands for its own side, the later blocks of its band for
 // both sides. A band is as long as the batch's longest cluster (nothing is then met
-// twice but the own blocks), unless its j-side sums would take more than the scratch
-// set aside: one float4 per (row, particle of a later block of the band), at most
-// (band - 1) / 2 per particle whatever the sizes, which stay on the device.
+// twice but the own blocks), unless the j-side sums, one float4 per (row, particle of a
+// later block of its band), would take more than the scratch set aside: then as long as
+// they may be, which the plan finds out, the sizes being on the device.
 //
 // A row has nt - r blocks to meet (nt blocks in the cluster, r its place in the
 // band): its own, the later ones of the band, then the others. It is cut into items
@@ -22,21 +22,25 @@ namespace nbk {
 constexpr int kBlock = 128;  // particles per block: 4 per lane
 constexpr int kTile = 64;    // particles per copy
 constexpr int kBlockTiles = kBlock / kTile;
-constexpr int kMinBand = 32;  // blocks that a band may always have
+// j-side entries set aside: 512 MiB, or the need of bands of kMinBand blocks for every
+// particle beyond the 256th of a cluster (the sizes are not known: on average), but no
+// more than the need of a single cluster.
+constexpr int64_t kPjEntries = (int64_t)32 << 20;
+constexpr int kMinBand = 32;
 // Clusters of up to so many blocks are evaluated per (i, j), every block by every row
 // (a band of one block): they have few pairs to save (cluster_weights, nb_batched.cu).
 constexpr int kDirectBlocks = 2;
 
 __host__ __device__ inline int cluster_band(int band, int64_t nt) { return nt <= kDirectBlocks ? 1 : band; }
 
-// What a plan depends on besides the offsets. A plan made for longer bands than a
-// call has scratch for must not stand: its j-side sums would go past their buffer.
+// What a plan depends on besides the offsets. A plan made for more j-side entries than
+// a call has scratch for must not stand: its sums would go past their buffer.
 struct BatchKey {
-    int64_t clusters, n_total, want_items, max_band;  // clusters -1: no plan
+    int64_t clusters, n_total, want_items, pj_entries;  // clusters -1: no plan
 };
 __host__ __device__ inline bool same_plan(const BatchKey &a, const BatchKey &b) {
     return a.clusters == b.clusters && a.n_total == b.n_total && a.want_items == b.want_items &&
-           a.max_band == b.max_band;
+           a.pj_entries == b.pj_entries;
 }
 
 struct BatchSplit {
@@ -72,11 +76,12 @@ struct BatchSplit {
     }
 };
 
-// The split of a batch whose rows meet `met` blocks in all, for `want` items: at
-// most one item per row more.
-__host__ __device__ inline BatchSplit batch_split(int band, int64_t met, int64_t want) {
+// The split of a batch whose rows meet `met` blocks in all, `longest` at most, for
+// `want` items: at most one item per row more.
+__host__ __device__ inline BatchSplit batch_split(int band, int longest, int64_t met, int64_t want) {
     BatchSplit s{band, 1, 1};
-    if (met > want) s.chunk = (int)((met + want - 1) / want);
+    const int64_t chunk = (met + want - 1) / want;
+    if (met > want) s.chunk = chunk < longest ? (int)chunk : longest;
     else while (2 * s.parts <= kBlockTiles && 2 * s.parts * met <= want) s.parts *= 2;
     return s;
 }
@@ -99,13 +104,26 @@ __host__ __device__ inline int batch_met_tile(int band, int nt, int b, int v) {
     return batch_met_block(band, nt, b, v / kBlockTiles) * kBlockTiles + v % kBlockTiles;
 }
 
-// The first j-side entry of row b (those of its band's later blocks' particles
-// follow) of a cluster whose first padded row is row0: kBlock (band - 1) / 2
-// entries are set aside per block.
-__host__ __device__ inline int64_t batch_pj_entry(int band, int64_t row0, int nt, int b) {
-    const int s0 = b / band * band, s1 = s0 + band < nt ? s0 + band : nt;
-    const int64_t r = b - s0, len = (int64_t)(s1 - s0) * kBlock;
-    return (row0 / kBlock + s0) * (kBlock / 2 * (band - 1)) + r * len - kBlock * (r * (r + 1) / 2);
+// j-side entries of a cluster of nt blocks.
+__host__ __device__ inline int64_t batch_pj_need(int band, int64_t nt) {
+    const int64_t cb = cluster_band(band, nt), k = nt / cb, rest = nt - k * cb;
+    return (k * (cb * (cb - 1) / 2) + rest * (rest - 1) / 2) * kBlock;
+}
+
+// The first j-side entry of row b, counted from the cluster's first (those of the
+// particles of its band's later blocks follow).
+__host__ __device__ inline int64_t batch_pj_row(int band, int nt, int b) {
+    const int cb = cluster_band(band, nt), k = b / cb, s0 = k * cb;  // (32-bit divisions: once per item)
+    const int64_t r = b - s0, len = cb < nt - s0 ? cb : nt - s0;
+    return (k * ((int64_t)cb * (cb - 1) / 2) + r * len - r * (r + 1) / 2) * kBlock;
+}
+
+// Entries set aside for a batch.
+inline int64_t batch_pj_entries(int64_t clusters, int64_t n_total) {
+    const int64_t most = (n_total + kBlock - 1) / kBlock, one = most * (most - 1) / 2 * kBlock;
+    const int64_t beyond = n_total - clusters * (kDirectBlocks * kBlock);
+    const int64_t want = beyond * (kMinBand - 1) / 2 > kPjEntries ? beyond * (kMinBand - 1) / 2 : kPjEntries;
+    return want < one ? want : one;
 }
 
 }  // namespace nbk
