@@ -221,7 +221,7 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode);
  * same, which the device checks on every call; any change makes a new one.
  * Scratch, kept in the context: per block of 128 particles (every cluster is padded to
  * whole blocks) 4.1 KiB, 6.1 KiB in compensated mode on FP64 state; 52 MiB; and for the
- * sums of evaluating every pair once 512 MiB, or 248 B for every particle beyond the
+ * sums of evaluating every pair once 512 MiB, or 265 B for every particle beyond the
  * 256th of a cluster if that is more (or less, where one cluster of all particles would
  * need less). Where it cannot be allocated the first alone, every pair then being
  * evaluated twice.

@@ -22,9 +22,9 @@ namespace nbk {
 constexpr int kBlock = 128;  // particles per block: 4 per lane
 constexpr int kTile = 64;    // particles per copy
 constexpr int kBlockTiles = kBlock / kTile;
-// j-side entries set aside: 512 MiB, or the need of bands of kMinBand blocks for every
-// particle beyond the 256th of a cluster (the sizes are not known: on average), but no
-// more than the need of a single cluster.
+// j-side entries set aside: 512 MiB, or what bands of kMinBand blocks need of clusters of
+// that many blocks or more, by the particles beyond the 256th of a cluster (on average:
+// the sizes are not known), but no more than the need of a single cluster.
 constexpr int64_t kPjEntries = (int64_t)32 << 20;
 constexpr int kMinBand = 32;
 // Clusters of up to so many blocks are evaluated per (i, j), every block by every row
@@ -122,7 +122,9 @@ __host__ __device__ inline int64_t batch_pj_row(int band, int nt, int b) {
 inline int64_t batch_pj_entries(int64_t clusters, int64_t n_total) {
     const int64_t most = (n_total + kBlock - 1) / kBlock, one = most * (most - 1) / 2 * kBlock;
     const int64_t beyond = n_total - clusters * (kDirectBlocks * kBlock);
-    const int64_t want = beyond * (kMinBand - 1) / 2 > kPjEntries ? beyond * (kMinBand - 1) / 2 : kPjEntries;
+    // (kMinBand - 1) / 2 entries for every one of their particles
+    const int64_t bands = beyond * (kMinBand - 1) * kMinBand / (2 * (kMinBand - kDirectBlocks));
+    const int64_t want = bands > kPjEntries ? bands : kPjEntries;
     return want < one ? want : one;
 }
 

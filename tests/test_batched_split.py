@@ -71,9 +71,10 @@ int main() {
     CHECK(batch_pj_entries(1000000, 32000000) == kPjEntries);
     CHECK(batch_pj_entries(1, 1000) == 8 * 7 / 2 * kBlock);
     CHECK(batch_pj_entries(100, 100) == 0);
-    CHECK(batch_pj_entries(2000, 2000 * 4096) >= 2000 * batch_pj_need(32, 30));
+    for (int64_t nt : {3, 10, 31, 32, 33, 64, 500})  // bands of 32 blocks in many large clusters
+        CHECK(batch_pj_entries(100000, 100000 * nt * kBlock) >= 100000 * batch_pj_need(32, nt));
     for (int64_t n : {1000, 100000, 10000000})
-        for (int64_t c : {1, 30, 100000}) CHECK(batch_pj_entries(c, n) <= (n * 31 / 2 > kPjEntries ? n * 31 / 2 : kPjEntries));
+        for (int64_t c : {1, 30, 100000}) CHECK(batch_pj_entries(c, n) <= (n * 17 > kPjEntries ? n * 17 : kPjEntries));
 }
 """)
 
