@@ -761,14 +761,11 @@ namespace {
 constexpr int kBmStages = 3;
 constexpr auto kBmPair = bm_pair_kernel<kBmStages, 12, 4, false>;
 constexpr auto kBmPairHL = bm_pair_kernel<kBmStages, 12, 4, true>;
-
-PairVariant bm_variant(bool hl) {
-    PairVariant v{};
-    v.tile.threads = 32;
-    v.kernel = (const void *)(hl ? kBmPairHL : kBmPair);
-    v.smem = hl ? bm_smem<kBmStages, true>() : bm_smem<kBmStages, false>();
-    return v;
-}
+// Of a tiny cluster's item little is arithmetic: more warps (16 an SM, 128 registers a
+// lane) hide more of the rest. 100000 clusters of 8 particles 510 -> 473 us, of 64 703 ->
+// 671; the same at 100, 128 particles 67 -> 73 us.
+constexpr auto kBmPairTiny = bm_pair_kernel<kBmStages, 16, 4, false>;
+constexpr int64_t kTinyMean = 64;  // particles per cluster
 
 struct BatchCall {
     const int64_t *offsets;
@@ -776,6 +773,16 @@ struct BatchCall {
     const float *eps;
     bool hl;  // HL records (compensated mode on FP64 state)
 };
+
+auto bm_kernel(const BatchCall &k) { return k.hl ? kBmPairHL : k.n_total <= kTinyMean * k.C ? kBmPairTiny : kBmPair; }
+
+PairVariant bm_variant(const BatchCall &k) {
+    PairVariant v{};
+    v.tile.threads = 32;
+    v.kernel = (const void *)bm_kernel(k);
+    v.smem = k.hl ? bm_smem<kBmStages, true>() : bm_smem<kBmStages, false>();
+    return v;
+}
 
 // Where a call's positions come from: FP32, or FP64 state with the leap-frog's
 // kicks and drift to be applied first (kick).
@@ -797,7 +804,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.cap_padded = k.n_total + k.C * (int64_t)kBlock;
     const int64_t blocks = A.cap_padded / kBlock;
     // small: one item per row and no j-side sums.
-    A.want_items = small ? 1 : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k.hl));
+    A.want_items = small ? 1 : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k));
     A.cap_items = blocks + A.want_items + 1;  // at most one per row beyond the number wanted
     if (A.cap_items > INT_MAX || k.C > INT_MAX) return fail(ctx, NB_ERR_ARG, "batch too large for 32-bit work items");
     A.pj_entries = small ? 0 : batch_pj_entries(k.C, k.n_total);
@@ -845,7 +852,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
 
 // Arguments of a call's kernels; allocates the scratch: per padded block 2 KiB of
 // records (4 on two-word positions), 2 of i-side sums and 32 bytes; 12 items a warp of
-// i-side sums (52 MiB); the j-side sums (batch_pj_entries: 512 MiB, or 248 B for every
+// i-side sums (52 MiB); the j-side sums (batch_pj_entries: 512 MiB, or 265 B for every
 // particle beyond the 256th of a cluster). Where that cannot be had, the first alone,
 // every pair then being evaluated twice. (10^6 clusters of 32: 5.7 GB.)
 nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
@@ -898,10 +905,10 @@ nb_status bm_force(nb_ctx *ctx, const BatchCall &k, BmArgs A, const BatchSource 
                             0);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batched pack launch");
-    const PairVariant v = bm_variant(k.hl);
+    const PairVariant v = bm_variant(k);
     {
         TimedLaunch t(ctx, 4, st);
-        e = launch_with_pdl(k.hl ? kBmPairHL : kBmPair, dim3((unsigned)resident_ctas(ctx, v)), dim3(32), v.smem, st, A);
+        e = launch_with_pdl(bm_kernel(k), dim3((unsigned)resident_ctas(ctx, v)), dim3(32), v.smem, st, A);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batched pair kernel launch");
     e = launch_with_pdl(k.hl ? bm_combine_kernel<true> : bm_combine_kernel<false>, blocks, threads, 0, st, A, a, p);
