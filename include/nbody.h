@@ -127,19 +127,22 @@ typedef struct nb_ctx nb_ctx;
  * clusters at once, the call runs the chunked form of the same shape. All
  * single-launch shapes are launched with programmatic stream serialization:
  * the next kernel on the stream may be scheduled while the previous one runs,
- * and each waits for its predecessor's results before reading. Callers that
- * pass FP64 state (the leap-frog) leave a single-launch shape for their
- * built-in choice.
- * `packed` & 64 marks a mutual shape (the built-in choice from n = 13312, and at
- * every n for the calls on FP64 positions): each unordered pair is evaluated once
+ * and each waits for its predecessor's results before reading. The plain
+ * leap-frog runs them up to n = 9728, built in or forced, on its FP64 positions
+ * rounded to FP32; above, and in compensated mode, calls on FP64 state leave a
+ * single-launch shape for their built-in choice.
+ * `packed` & 64 marks a mutual shape (the built-in choice from n = 13312, in
+ * compensated mode from n = 24576; for the leap-frog from n = 9729, in compensated
+ * mode at every n): each unordered pair is evaluated once
  * and added to both particles, in 8 to 9.5 FP32 operations per ordered pair (8
  * when all masses are equal; which form a call takes is decided on the device).
  * It packs, sums and combines in launches of its own; `fused` = 2 then marks the
  * shape that runs every form in one kernel instead of one each. Its i-blocks hold `threads` * `ipt`
  * particles, its running sums are always compensated (NB_PLAIN and
  * NB_COMPENSATED run the same kernel), and its scratch grows with n^2, n^2 / 128
- * bytes up to 1 GiB; where that cannot be allocated the built-in choice for that n
- * and above is a direct shape instead. */
+ * bytes up to 1 GiB (nb_force, the calls on FP64 state and the VJP have theirs
+ * apart); where that cannot be allocated the built-in choice for that n and above is
+ * a direct shape instead. */
 typedef struct nb_tile {
     int threads;
     int ipt;
@@ -220,7 +223,7 @@ nb_status nb_reserve(nb_ctx *ctx, int64_t n, nb_mode mode);
  * batched leap-frog) while n_clusters, n_total and the values of offsets stay the
  * same, which the device checks on every call; any change makes a new one.
  * Scratch, kept in the context: per block of 128 particles (every cluster is padded to
- * whole blocks) 4.1 KiB, 6.1 KiB in compensated mode on FP64 state; 52 MiB; and for the
+ * whole blocks) 4.1 KiB, 6.1 KiB in compensated mode on FP64 state; 57 MiB; and for the
  * sums of evaluating every pair once 512 MiB, or 265 B for every particle beyond the
  * 256th of a cluster if that is more (or less, where one cluster of all particles would
  * need less). Where it cannot be allocated the first alone, every pair then being
@@ -262,7 +265,8 @@ nb_status nb_leapfrog_batched_step(nb_ctx *ctx, double *x, double *v, const floa
  *                on exit Eq. (gravity) at the exit positions
  *   p    [n]    FP32 device, out: potentials at the exit positions, or NULL:
  *                the integrator needs only a, so the force kernels then leave
- *                the potential out (12 instead of 13 FP32 operations per pair)
+ *                the potential out (two FP32 operations fewer per unordered pair;
+ *                the single-launch shapes sum it all the same)
  * Asynchronous. In NB_COMPENSATED mode the FP64 positions enter the pair
  * kernel relative to the centre of their bounding box (recomputed at every
  * force evaluation), each coordinate as an exact FP32 grid part plus an FP32
@@ -321,7 +325,7 @@ nb_status nb_energy(nb_ctx *ctx, const double *x, const double *v, const float *
  * respect to the positions, gx [n][3], and masses, gm [n]. All FP32 device
  * arrays; gp may be NULL (no upstream gradient on p: a kernel without its
  * terms runs). Each unordered pair is evaluated once and added to both
- * particles, 19 FP32 operations per ordered pair (17 without gp), in a fixed
+ * particles, 18.5 FP32 operations per ordered pair (17 without gp), in a fixed
  * order without atomics, so the result is reproducible. Scratch grows with n^2
  * (n^2 / 32 bytes, up to 1 GiB; where that cannot be allocated, a gather over all
  * ordered pairs runs instead). Asynchronous.

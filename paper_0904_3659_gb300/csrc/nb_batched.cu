@@ -4,7 +4,7 @@
 // "Method" over such a batch (nb_batched.cuh has the layout and the work split).
 //
 // An evaluation is four launches: plan (padded offsets and blocks; a plan for the
-// same sizes, offsets and eps stands), pack (records and work items), pair kernel
+// same sizes and offsets stands, and serves all steps of a call), pack (records and work items), pair kernel
 // (its warps pop items from an atomic counter), combine. Every sum has a fixed
 // order, so the results do not depend on which warp pops what.
 #include <algorithm>
@@ -24,9 +24,12 @@ using namespace nbdev;
 
 constexpr int kBmPlanThreads = 1024;
 constexpr int kBmPlanNear = 8192;  // clusters whose first blocks the plan keeps in shared memory
-// Items per resident warp that the plan aims at: more of them even out the end of
-// the launch, fewer mean fewer partial sums.
-constexpr int kItemsPerWarp = 12;
+// Items per SM that the plan aims at, 16 for a resident warp (12 on two-word records):
+// more of them even out the end of the launch, fewer mean fewer partial sums. FP32
+// records, 192 an SM against 144: 8 clusters of 6000 to 20000 540 us against 553, 500 of
+// 4096 2868 against 2887 (one of 20000 206 against 164, where 144 happen to divide well);
+// two-word records, 144 against 192: one of 20000 222 us a step against 261, the rest equal.
+constexpr int64_t kItemsPerSm = 192, kItemsPerSmHL = 144;
 constexpr int kBatchP = kBlock / 64;  // packed i-pairs per lane
 
 struct BmBlock {  // a padded block
@@ -47,7 +50,7 @@ struct BmArgs {
     BatchSplit *split;     // the batch's
     int64_t *pjbase;       // [C] the cluster's first j-side entry
     int64_t pj_entries;    // set aside
-    int64_t want_items;    // items wanted: kItemsPerWarp per resident warp
+    int64_t want_items;    // items wanted (kItemsPerSm)
     int *notes;            // [C] what the pack found of a cluster (MutualNote); zero before it
     int *weights;          // [C] the form of its weights (MutualWeights), from the pair kernel
     MPart *cp;             // [cap_padded][1 or 2]
@@ -323,7 +326,7 @@ __global__ void __launch_bounds__(kFrameThreads) batch_frame_kernel(const double
 }
 
 // Compensated mode on FP64 state: HL records in the cluster's frame (centre of
-// its bounding box, grid; see kHLRecords and batch_pack_hl_kernel).
+// its bounding box, grid; see kHLRecords).
 __global__ void __launch_bounds__(kBlock) bm_pack_hl_kernel(const BmArgs A, const double *__restrict__ x,
                                                             const float *__restrict__ m,
                                                             const double4 *__restrict__ frame) {
@@ -430,13 +433,11 @@ struct BmStage {
 // items' ends. 128 particles a block (4 per lane) against 256: half the padding and
 // half the own-block work, twice the j-side sums; 57 against 87 us up to 512, 667
 // against 687 up to 4096. Tiles of 64 against 128: 47 against 55 us up to 512.
-// Twelve warps' worth of registers (142 a lane: 14 resident, 148 on two-word records); 12 items per warp
-// against 8: 669 against 678 us, against 4: 702.
+// Twelve warps an SM (140 registers a lane, 147 on two-word records).
 // Against one evaluation per (i, j): 1024 clusters up to 4096 particles 817 -> 685 us
 // (the pair kernel 777 -> 632; 904.8e6 unordered pairs, 66% of the FP32 lanes' issue
-// rate counting 18 operations a pair and the padding), 1024 up to 512 82 -> 63, 300
-// up to 2048 113 -> 87, a step of those on FP64 state 150 -> 120, 8 of 6000 to 20000
-// 730 -> 510.
+// rate counting 18 operations a pair and the padding), 1024 up to 512 82 -> 53, 300
+// up to 2048 113 -> 81, a step of those on FP64 state 150 -> 116.
 template <int STAGES, int MINB, int UNR, bool HL>
 __global__ void __launch_bounds__(32, MINB) bm_pair_kernel(const BmArgs A) {
     constexpr int P = kBatchP;
@@ -804,7 +805,7 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
     A.cap_padded = k.n_total + k.C * (int64_t)kBlock;
     const int64_t blocks = A.cap_padded / kBlock;
     // small: one item per row and no j-side sums.
-    A.want_items = small ? 1 : (int64_t)kItemsPerWarp * resident_ctas(ctx, bm_variant(k));
+    A.want_items = small ? 1 : (k.hl ? kItemsPerSmHL : kItemsPerSm) * ctx_sm_count(ctx);
     A.cap_items = blocks + A.want_items + 1;  // at most one per row beyond the number wanted
     if (A.cap_items > INT_MAX || k.C > INT_MAX) return fail(ctx, NB_ERR_ARG, "batch too large for 32-bit work items");
     A.pj_entries = small ? 0 : batch_pj_entries(k.C, k.n_total);
@@ -851,8 +852,8 @@ nb_status bm_args(nb_ctx *ctx, const BatchCall &k, bool small, BmArgs *out) {
 }
 
 // Arguments of a call's kernels; allocates the scratch: per padded block 2 KiB of
-// records (4 on two-word positions), 2 of i-side sums and 32 bytes; 12 items a warp of
-// i-side sums (52 MiB); the j-side sums (batch_pj_entries: 512 MiB, or 265 B for every
+// records (4 on two-word positions), 2 of i-side sums and 32 bytes; kItemsPerSm items'
+// i-side sums (57 MiB); the j-side sums (batch_pj_entries: 512 MiB, or 265 B for every
 // particle beyond the 256th of a cluster). Where that cannot be had, the first alone,
 // every pair then being evaluated twice. (10^6 clusters of 32: 5.7 GB.)
 nb_status bm_prepare(nb_ctx *ctx, const BatchCall &k, BmArgs *out) {
