@@ -494,7 +494,7 @@ def extra_adjoint(nb, ctx, dev, torch, plain_rate, oracle_ref=False):
         nb.nb_force(ctx, x, mt, n, eps, a, p)
     f1.record()
     # The trajectory adjoint's case: no upstream gradient on p (34 instead of
-    # 38 FP32 operations per unordered pair).
+    # 37 FP32 operations per unordered pair).
     for _ in range(3):
         nb.nb_force_vjp(ctx, x, mt, n, eps, ga, None, gx, gm)
     g0, g1 = _events(torch)

@@ -50,7 +50,8 @@ __global__ void mutual_pack_f32_kernel(const float *__restrict__ x, const float 
 // STAGES buffers, UNR the unroll of the j loop (16 no longer fits the instruction
 // cache: 25% slower), MINB the CTAs per SM that the registers are held to, POT
 // with the potential, HL on two-word positions.
-// W: the form of the weights. From n = 24576 the three forms are three kernels;
+// W: the form of the weights. From n = 24576 (18432 on two-word positions) the three
+// forms are three kernels;
 // all are launched and those not meant return at once (the choice is the pack's,
 // on the device): with the loops in one kernel (kAny) each of them runs 5-8%
 // slower, the registers being allocated for the worst. Below, the two launches

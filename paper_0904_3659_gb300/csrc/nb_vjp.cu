@@ -502,14 +502,14 @@ const VjpVariant kVjp[] = {
 #undef NB_VJP_MR
 constexpr int kVjpCount = (int)(sizeof(kVjp) / sizeof(kVjp[0]));
 // Built-in: the mutual shapes at every size (us with / without gp, against the
-// direct shapes below: N = 1000 15 / 13.5 against 19.5 / 18.4, N = 4096 29.5 / 27
-// against 33 / 35, N = 16384 225 / 201 against 268 / 245, N = 65536 3305 / 2980
+// direct shapes below: N = 1000 13.5 / 12.7 against 18.2 / 18.0, N = 4096 27 / 26.5
+// against 32 / 34, N = 16384 219 / 202 against 268 / 245, N = 65536 3225 / 2989
 // against 4090 / 3655), with 32-particle j-tiles below kVjpMutualLargeN (N = 8192
-// 71 / 62 against 72 / 65) and 128-particle tiles from there (N = 12000 133 / 119
-// against 138 / 120), but 32 again without gp from kVjpMutualNoGpN (N = 16384 201.2
-// for 128 against 201.9, 20000 312 against 296, 32768 776 against 751, 65536 2990
-// against 2961). The direct shapes remain for n whose mutual scratch cannot
-// be allocated.
+// 66.6 / 63.8 against 68.4 / 64.1) and 128-particle tiles from there (N = 12000 130 /
+// 119.5 against 132 / 126, N = 15000 188 / 174 against 188 / 179; where the tiles divide
+// better the other way round, N = 14000 187 / 174 against 166 / 158), but 32 again
+// without gp from kVjpMutualNoGpN (20000 297 against 313). The direct shapes remain for n
+// whose mutual scratch cannot be allocated.
 // Direct shapes (GB300 sweep, G-pairs/s). With an upstream gradient on p:
 // two packed pairs per thread in 128-thread CTAs with the barrier-free stage
 // release; below 2^15, 128-particle j-tiles at three CTAs per SM (at most 168

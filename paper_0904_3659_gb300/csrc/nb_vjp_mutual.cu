@@ -536,7 +536,7 @@ struct VmShape {
      launch_vm<4, 2, J, 3, U, 3, GP, RUN, FOLD>}
 
 // [size][without, with an upstream gradient on p]. Like the force's, register
-// reads bound these: N = 65536 runs at 1299 G-pairs/s with gp and 1441 without it
+// reads bound these: N = 65536 runs at 1332 G-pairs/s with gp and 1437 without it
 // (direct kernels 1050 and 1175). Measured and not kept there: an unroll of 4
 // (1228 / 1363) or 2 (1147 / 1283) with 128-particle tiles, four CTAs per SM (1159
 // / 1256), 8 i-particles per thread at two CTAs (1277 / 1496, but 1043 / 1217
