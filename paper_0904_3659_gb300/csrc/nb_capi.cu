@@ -176,11 +176,11 @@ cudaError_t ensure_counters(nb_ctx *ctx, int64_t nib) {
     return cudaSuccess;
 }
 
-int resident_ctas(nb_ctx *ctx, const PairVariant &v) {
+int resident_ctas(nb_ctx *ctx, const PairVariant &v, size_t most) {
     auto it = ctx->occupancy.find(v.kernel);
     if (it != ctx->occupancy.end()) return it->second * ctx->sm_count;
-    if (v.smem > 48 * 1024)
-        cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem);
+    if (std::max(v.smem, most) > 48 * 1024)
+        cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(v.smem, most));
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.kernel, v.tile.threads, v.smem) !=
             cudaSuccess ||

@@ -92,7 +92,10 @@ ExtState &ctx_ext(nb_ctx *ctx);
 bool ctx_set_timing(nb_ctx *ctx, bool on);
 
 cudaError_t ensure_buffer(void **ptr, size_t *cap, size_t bytes);
-int resident_ctas(nb_ctx *ctx, const nbk::PairVariant &v);
+// CTAs of the kernel on the GPU at once. `most`: the most dynamic shared memory that a
+// launch of it asks for, where that is more than v.smem; the same for every context,
+// because the limit it sets on the kernel is the process's.
+int resident_ctas(nb_ctx *ctx, const nbk::PairVariant &v, size_t most = 0);
 const nbk::PairVariant &choose_variant(nb_ctx *ctx, int64_t n, bool comp);
 
 // Compensated path on FP64 state: pair kernel on HL records (two JParts per

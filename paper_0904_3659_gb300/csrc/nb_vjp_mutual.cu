@@ -570,7 +570,7 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
     v.tile.threads = s.threads;
     v.kernel = s.kernel;
     v.smem = s.smem;
-    const int resident = resident_ctas(ctx, v);
+    const int resident = resident_ctas(ctx, v, kSmSharedBytes / 2);
     const int64_t npad = round_up(std::max<int64_t>(n, 1), s.ib);
     const Triangle T{(n + s.jt - 1) / s.jt, (n + s.ib - 1) / s.ib, s.ib / s.jt};
     const int64_t most = (int64_t)(kMutualPartialBytes / (2 * sizeof(float4))) / s.jt;  // tiles per panel
@@ -626,11 +626,7 @@ nb_status run_vjp_mutual(nb_ctx *ctx, int size, const float *x, const float *m, 
         // 456 places: 33.3 us without, 27.1 with).
         const int sms = ctx_sm_count(ctx), per_sm = (A.grid + sms - 1) / sms;
         size_t smem = s.smem;
-        if (per_sm * sms < resident) {
-            smem = std::max(smem, kSmSharedBytes / (per_sm + 1));
-            e = cudaFuncSetAttribute(s.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "vjp shared memory");
-        }
+        if (per_sm * sms < resident) smem = std::max(smem, kSmSharedBytes / (per_sm + 1));
         {
             TimedLaunch t(ctx, 5, st);
             e = s.launch(A, smem, st);
